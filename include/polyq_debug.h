@@ -35,7 +35,7 @@ int polyq_debug_gemv_codes(const polyq_dev_layer* layer, const void* x, int batc
 
 /* polyq_linear_gemm; w_out: device uint16 [N][K], the fp16 weight of every
  * (row, clustered position) as the GEMM's dequantisers wrote it into the
- * tensor cores' B operand tile (for 16-bit blocks, as TMA loaded it),
+ * tensor cores' operand tile (for 16-bit blocks, as TMA loaded it),
  * fp16_rn((q - zero) * scale) for b < 16. */
 int polyq_debug_gemm_weights(const polyq_dev_layer* layer, const void* X, int64_t M, float* Y,
                              void* workspace, size_t workspace_bytes, uint16_t* w_out,

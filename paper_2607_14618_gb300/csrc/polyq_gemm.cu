@@ -1,81 +1,193 @@
 // Prefill GEMM of the PolyQ mixed-bit layer on the 5th-generation tensor
-// cores (tcgen05, tensor memory):
+// cores (tcgen05, tensor memory), on pairs of SMs:
 //
 //   Y[m][n] = sum_p X[m][gather[p]] * W'[n][p]        (Section 4.1 product)
 //
-// The contraction runs over 32-wide K tiles (half a quantisation group); every
-// tile lies inside one bit block (Section 4.2) and one group, so each weight
-// row of a tile has one (scale, zero).
-//  1. gemm_prep gathers X through `gather` into a clustered fp16 matrix Xg
-//     (workspace), zero-padded at block ends, with the K order inside each
-//     tile permuted the same way the dequantiser emits codes.  Xg is stored
-//     as the shared-memory images of the producer's copies: one 16 KB block
-//     per (pair of M tiles, K tile), 256 rows of 64 bytes in the 64-byte
-//     swizzle, so that one contiguous bulk copy fetches a stage's X.
-//     Each row m is scaled by the power of two 2^-e_m that brings its largest
-//     |x * t| into [2^14, 2^15), so that any finite bf16 row rounds to fp16
-//     without overflow and without dropping small values into subnormals;
-//     the epilogue multiplies row m of Y by 2^e_m.
-//  2. gemm_main: one persistent CTA per SM, 10 warps.
-//       warp 0      TMA producer: Xg blocks (bulk copies), packed code
-//                   bytes and meta of 256 weight rows, or for 16-bit blocks the
-//                   fp16 weights straight into the operand buffer;
-//       warp 1      allocates 512 TMEM columns and issues tcgen05.mma
-//                   (M=128, N=256, K=16, fp16 in, fp32 accumulate): the
-//                   weights are the A operand, 128 rows per MMA, and the
-//                   256 tokens of an M pair the B operand, so a TMEM lane
-//                   holds one output column;
-//       warps 2..9  dequantise: (q - z) * s in fp16 via magic-number decode,
-//                   written in the UMMA 64-byte-swizzle K-major layout.  Warps
-//                   2-5 take the even stages and 6-9 the odd ones, two weight
-//                   rows per thread; afterwards all eight drain the
-//                   accumulator with tcgen05.ld and store fp32 Y, each warp
-//                   store covering 32 consecutive columns of one row.
-//     Five pipeline stages.  When the (M, N) tiles cannot fill the GPU the K
-//     range is split, uniformly or stream-K (each CTA an equal contiguous
-//     share of all (tile, K tile) pairs), and the pieces are added into a
-//     zeroed Y (so the order of those additions varies); otherwise Y is
-//     stored directly.  Every wait is bounded and reports through the
-//     workspace status word.
+// The contraction runs over K tiles of 32 or 64 (half or all of a quantisation
+// group); every tile lies inside one bit block (Section 4.2) and one group, so
+// each weight row of a tile has one (scale, zero).
+//  1. A pre-pass (gemm_prep, or gemm_prep_small for a few rows) gathers X
+//     through `gather` into a clustered fp16 matrix Xg (workspace),
+//     zero-padded at block ends, with the K order inside each tile permuted
+//     the same way the dequantiser emits codes.  Xg is stored as the
+//     shared-memory images of the producer's copies: per (CTA's tokens, 32 K
+//     slots) one block of R rows of 64 bytes in the 64-byte swizzle, so that
+//     one contiguous bulk copy fetches a stage's X.  Each row m is scaled by
+//     the power of two 2^-e_m that brings its largest |x * t| into
+//     [2^14, 2^15), so that any finite bf16 row rounds to fp16 without
+//     overflow and without dropping small values into subnormals; the
+//     epilogue multiplies row m of Y by 2^e_m.
+//  2. gemm_main: persistent clusters of two CTAs, one CTA per SM.  A work unit
+//     is 256 weight rows by T tokens; CTA r of the pair holds weight rows
+//     128 r.. and half of the tokens, and one tcgen05.mma.cta_group::2
+//     (M = 256, N = 32..256, K = 16, fp16 in, fp32 accumulate) multiplies all
+//     rows with all tokens, so each weight is dequantised by one SM only and
+//     each operand byte is read from shared memory once per SM pair.  The
+//     weights are the A operand, so a TMEM lane holds one output column.
+//       warp 0      TMA producer: Xg blocks (bulk copies), packed code bytes
+//                   and meta of the CTA's 128 weight rows, or for 16-bit
+//                   blocks the fp16 weights straight into the operand buffer;
+//       warp 1      allocates 512 TMEM columns; in the leader CTA it issues
+//                   the MMAs;
+//       warps 2..   groups of four warps dequantise, one weight row per
+//                   thread, alternating over the stages: (q - z) * s in fp16,
+//                   written in the UMMA 64-byte-swizzle K-major layout;
+//       last four   drain the accumulators with tcgen05.ld and store fp32 Y,
+//                   each warp store covering 32 consecutive columns of a row.
+//     When the (M, N) tiles cannot fill the GPU the K range is split,
+//     uniformly or stream-K (each pair an equal contiguous share of all (tile,
+//     K tile) pairs), and the pieces are added into a zeroed Y (so the order
+//     of those additions varies); otherwise Y is stored directly.  Every wait
+//     is bounded and reports through the workspace status word.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
+#include <atomic>
+#include <cstring>
 
 #include "polyq.h"
 #ifdef POLYQ_DEBUG
 #include "polyq_debug.h"
 #endif
 #include "polyq_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
+#include "polyq_gemv_dev.cuh"
 #include "polyq_internal.h"
 
 namespace {
 
 using namespace polyq;
 
-constexpr int BM = 128;           // rows per MMA
-constexpr int MT = 2;             // M tiles per work unit (share one weight tile)
-constexpr int BN = 256;           // weight rows per work unit
-constexpr int BK = 32;            // K per tile: half a quantisation group
-constexpr int kStagesG = 5;
-constexpr int kCodeBox = 32;      // code bytes per row loaded per tile: the tile's codes from a
-                                  // 16-byte aligned start (offset <= 12 with at most 16 bytes of
-                                  // codes, or 32 bytes of 8-bit codes at offset 0), one TMA
-                                  // row request each (48-byte rows take two)
-constexpr int kATile = BM * BK * 2;             // 8 KB (64-byte rows)
-constexpr int kBTile = BN * BK * 2;             // 16 KB
-constexpr int kCodes = BN * kCodeBox;           // 8 KB
-constexpr int kMeta = BN * 16;                  // 4 KB
-constexpr int kStageG = MT * kATile + kBTile + kCodes + kMeta;  // 44 KB
-constexpr int kThreadsG = 320;
-constexpr int kDqWarps = 8;
-constexpr double kUnitCostTiles = 12.0;  // per-piece overhead, in K-tile stages, of the split model
-constexpr double kStageSeconds = 0.6e-6;  // one K-tile stage of a CTA, measured
-constexpr double kZeroBytesPerS = 5e12;   // the pre-pass zeroing Y
+constexpr int kRowsN = 256;       // weight rows per work unit
+constexpr int kRowsCta = 128;     // of which each CTA of a pair holds half
+constexpr int kSlots = 32;        // K slots of an Xg block and of a 64-byte operand row
+constexpr int kCodeBox = 32;      // code bytes per row of one code box: the codes of a tile of 32
+                                  // from a 16-byte aligned start (offset <= 12 with at most 16
+                                  // bytes of codes, or 32 bytes of 8-bit codes at offset 0), or of
+                                  // a tile of 64 at 2 to 4 bits (24 bytes at offset 0 or 8, else
+                                  // at offset 0); one TMA row request each (48-byte rows take two)
+constexpr int kBoxBytes = kRowsCta * kCodeBox;  // 4 KB
+constexpr int kMetaBytes = kRowsCta * 16;       // 2 KB
+constexpr int kHalfTile = kRowsCta * kSlots * 2;  // 8 KB: 128 operand rows of 64 bytes
+constexpr double kZeroBytesPerS = 5e12;  // the pre-pass zeroing Y
 constexpr uint32_t kTmemCols = 512;
-constexpr uint32_t kIdesc = umma_idesc_f16(BM, BN);
+// Cost model of the split of K (plan_split), seconds: one stage of a pair and
+// the overhead of a piece, by token tile.
+constexpr double kStage32 = 0.27e-6, kPiece32 = 2.5e-6;
+constexpr double kStage64 = 0.27e-6, kPiece64 = 2.5e-6;
+constexpr double kStage128 = 0.29e-6, kPiece128 = 3e-6;
+constexpr double kStage256 = 0.31e-6, kPiece256 = 4.5e-6;
+constexpr double kStage512 = 0.27e-6, kPiece512 = 5.5e-6;
+
+// One kernel per token count T of a work unit.
+//   TN      tokens per MMA (its N); CTA r of the pair holds TN / 2 of them
+//   NACC    accumulators of a unit (T = NACC * TN); with one, two units'
+//           accumulators alternate, so that one drains while the next fills
+//   BK      K of a stage
+//   OPS     weight slots: a dequantised tile
+//   XS      token slots: the tile's X
+//   CODES   code slots: packed codes and meta, free again once a dequantiser
+//           holds them in registers, so that the copies of the packed weights
+//           run CODES stages ahead whatever the MMAs do
+//   GROUPS  dequantiser groups of four warps (CODES a multiple of it)
+//   EPI     epilogue warps (a multiple of four)
+template <int TN_, int NACC_, int BK_, int OPS_, int XS_, int CODES_, int GROUPS_, int EPI_>
+struct Cfg {
+  static constexpr int TN = TN_, NACC = NACC_, BK = BK_, OPS = OPS_, XS = XS_;
+  static constexpr int CODES = CODES_, GROUPS = GROUPS_, EPI = EPI_;
+  static constexpr int T = TN * NACC;
+  static constexpr int R = T / 2;           // tokens (rows of X) per CTA
+  static constexpr int NBUF = NACC == 1 ? 2 : 1;
+  static constexpr int HALVES = BK / kSlots;
+  static constexpr int kA = HALVES * kHalfTile;
+  static constexpr int kX = HALVES * R * kSlots * 2;
+  static constexpr int kCodes = HALVES * kBoxBytes;
+  static constexpr int kCode = kCodes + kMetaBytes;
+  static constexpr int kCodeProd = 2;  // producer warps of the codes
+  static constexpr int kEpiWarp = 16, kWarps = kEpiWarp + EPI;
+  static constexpr int kThreads = 32 * kWarps;
+  static constexpr int kXOff = OPS * kA, kCodeOff = kXOff + XS * kX;  // in shared memory
+  static constexpr size_t kSmem = (size_t)kCodeOff + CODES * kCode + 1024;
+  static constexpr uint32_t kIdesc = umma_idesc_f16(kRowsN, TN);
+  static_assert(kX % 1024 == 0 && kSmem <= 225 * 1024 + 512 && NACC * NBUF * TN <= (int)kTmemCols, "");
+  static_assert(GROUPS == 3 && CODES % GROUPS == 0 && OPS % GROUPS == 0 && kCodeProd <= CODES, "");
+};
+using Cfg32 = Cfg<32, 1, 64, 6, 16, 9, 3, 4>;
+using Cfg64 = Cfg<64, 1, 64, 6, 8, 9, 3, 4>;
+using Cfg128 = Cfg<128, 1, 64, 6, 6, 6, 3, 4>;
+using Cfg256 = Cfg<256, 1, 64, 6, 4, 6, 3, 4>;
+using Cfg512 = Cfg<256, 2, 32, 6, 7, 9, 3, 8>;
+// Warps 0, 4, 8 and 12, which share a scheduler, are the lone-thread roles
+// (two code producers, the X producer, the MMA issuer), the other twelve of
+// the first sixteen the dequantisers: their long unrolled code would evict a
+// role's few instructions from the scheduler's instruction cache every stage
+// (gate at M = 2048: 186 us with the roles spread over all schedulers, 180 us).
+enum Role { kRoleCode0 = 0, kRoleCode1, kRoleX, kRoleMma, kRoleDequant, kRoleEpilogue };
 
 struct GmBlock {
   int bits, n_ch, pos0, seg_off, grp_off, n_grp;
@@ -83,16 +195,21 @@ struct GmBlock {
 };
 
 struct GmParams {
-  CUtensorMap tm_codes;  // packed [N][S] u8, box {kCodeBox, 256}
-  CUtensorMap tm_meta;   // meta [N][meta_stride] u32, box {4, 256}
-  CUtensorMap tm_w16;    // packed [N][S/2] u16, box {32, 256}, 64B swizzle
+  CUtensorMap tm_codes;  // packed [N][S] u8, box {kCodeBox, 128}
+  CUtensorMap tm_meta;   // meta [N][meta_stride] u32, box {4, 128}
+  CUtensorMap tm_w16;    // packed [N][S/2] u16, box {32, 128}, 64B swizzle
   GmBlock blk[POLYQ_MAX_BLOCKS];
   int n_blocks;
-  int M, N, K, KT;
-  int units_m, units_n, ksplit, units;  // work units: (M pair, N tile, K split)
-  int streamk;  // 1: each CTA takes an equal contiguous range of (unit, K tile) pairs
+  int M, N, K, KT;  // KT: K tiles of BK
+  int bk;           // 32 or 64
+  int r_log2;       // rows of X per CTA and unit: 2^r_log2
+  int units_m, units_n, ksplit, units;  // work units: (token tile, N tile, K split)
+  int streamk;  // 1: each pair takes an equal contiguous range of (unit, K tile) pairs:
+  int sk_share, sk_extra;  // sk_share of them, the first sk_extra pairs one more
   int has_meta;
   int prep_staged;  // 1: the pre-pass stages each row of X in shared memory
+  int prep_seg;     // gemm_prep_small: CTAs per row
+  int prep_rows;    // gemm_prep_small: CTAs that gather rows (the others zero Y)
   const __nv_bfloat16* x;
   const int32_t* gather;
   const float* xscale;  // Section 3.4 activation factors (clustered order) or NULL
@@ -102,13 +219,79 @@ struct GmParams {
   int* status;
 };
 
+// ---------------------------------------------------------------------------
+// CTA pairs
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t cluster_ctarank() {
+  uint32_t r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+// One thread of the (converged) warp, in the form that tells the compiler so:
+// with `lane == 0` instead the lone-thread roles took 440 to 480 cycles for a
+// stage's copies and 360 for its MMAs, with this 180 and 90.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile("{\n .reg .pred p;\n elect.sync _|p, 0xffffffff;\n selp.u32 %0, 1, 0, p;\n}\n" : "=r"(p));
+  return p != 0;
+}
+__device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void cluster_sync() {
+  asm volatile("barrier.cluster.arrive.release;\n barrier.cluster.wait.acquire;" ::: "memory");
+}
+// Arrive on a barrier of a CTA of the cluster (address from mapa).  With the
+// default scope: what such an arrival announces (weights and X in this CTA's
+// shared memory, drained tensor memory) reaches the other side only through
+// the tensor core, which fence.proxy.async and the tcgen05 fences order.  A
+// release at cluster scope waits for all of the warp's memory traffic at every
+// stage: gate at M = 2048 took 352 us with it and 281 us without.
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cluster.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+__device__ __forceinline__ void tmem_alloc2(uint32_t dst_smem, uint32_t ncols) {
+  asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem),
+               "r"(ncols)
+               : "memory");
+}
+__device__ __forceinline__ void tmem_relinquish2() {
+  asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void tmem_dealloc2(uint32_t taddr, uint32_t ncols) {
+  asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;" ::"r"(taddr), "r"(ncols)
+               : "memory");
+}
+// D[tmem of both CTAs] (+)= A * B^T over the pair's operands: descriptors are
+// this CTA's, and the peer's operands lie at the same offsets.
+__device__ __forceinline__ void tc_mma2_f16(uint32_t d_tmem, uint64_t a_desc, uint64_t b_desc,
+                                            uint32_t idesc, uint32_t accumulate) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
+      " tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d_tmem),
+      "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
+      : "memory");
+}
+// Arrive (once) on the barrier at this offset in both CTAs when all tcgen05
+// operations issued so far by this thread have completed.
+__device__ __forceinline__ void tc_commit2(uint32_t bar) {
+  asm volatile(
+      "tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64"
+      " [%0], %1;" ::"r"(bar),
+      "h"((uint16_t)3)
+      : "memory");
+}
+
 // try_wait that lets the hardware suspend the thread for up to `hint_ns`
 // (it wakes when the phase completes) instead of returning at once.
 __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity,
                                                    uint32_t hint_ns) {
   uint32_t ok;
   asm volatile(
-      "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
+      "{\n .reg .pred p;\n"
+      " mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2, %3;\n"
       " selp.u32 %0, 1, 0, p;\n}\n"
       : "=r"(ok)
       : "r"(bar), "r"(parity), "r"(hint_ns)
@@ -116,7 +299,7 @@ __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity
   return ok != 0;
 }
 
-// Bounded waits that also give up once another role of the CTA has failed:
+// Bounded waits that also give up once another role of the pair has failed:
 // 0 when the phase completed, 1 on a timeout, 2 when `abort` was raised.  The
 // flag is read only after a poll has failed, so that a stage whose barrier
 // has already completed costs one poll and no shared load.  The lone producer
@@ -142,43 +325,82 @@ __device__ __forceinline__ int wait_sleep_ab(uint32_t bar, uint32_t parity,
   return kWaitTimeout;
 }
 
-// The pieces of work a CTA takes, in order: an output tile (um, un) and a
-// range [kt_lo, kt_hi) of its K tiles.  Units are strided over the grid, each
-// with its K split's range; with `streamk`, a CTA takes the K tiles
-// [T*b/C, T*(b+1)/C) of the T = units * KT (unit, K tile) pairs in unit-major
-// order, which cuts at most two units per CTA short.  Every role of a CTA
-// walks the same sequence.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+  uint32_t ok;
+  asm volatile(
+      "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+      " selp.u32 %0, 1, 0, p;\n}\n"
+      : "=r"(ok)
+      : "r"(bar), "r"(parity)
+      : "memory");
+  return ok != 0;
+}
+// Bit i: whether the phase of the i-th slot from `s` on, every STEP-th of N,
+// has completed (parity `ph` up to the ring's end, the other after it).  A
+// poll's answer takes 200 to 300 cycles here, behind the dequantisers' shared
+// memory traffic, but polls follow each other every 15: a lone thread that
+// polls B stages at once pays that latency once for all that are ready.
+template <int B, int N, int STEP = 1>
+__device__ __forceinline__ uint32_t poll_ahead(uint32_t bar0, int s, uint32_t ph) {
+  static_assert((B - 1) * STEP < N, "one phase per slot");
+  uint32_t ok = 0;
+#pragma unroll
+  for (int i = 0; i < B; ++i) {
+    int k = s + i * STEP;
+    uint32_t p = ph;
+    if (k >= N) {
+      k -= N;
+      p ^= 1u;
+    }
+    ok |= (mbar_test(bar0 + 8 * k, p) ? 1u : 0u) << i;
+  }
+  return ok;
+}
+// Stages ready in a row.
+__device__ __forceinline__ int leading(uint32_t ok) { return __ffs(~ok) - 1; }
+
+// The pieces of work a CTA pair takes, in order: an output tile (um, un) and a
+// range [kt_lo, kt_hi) of its K tiles.  Units are strided over the pairs, each
+// with its K split's range; with `streamk`, a pair takes an equal contiguous
+// share (to one) of the units * KT (unit, K tile) pairs in unit-major order,
+// which cuts at most two units per pair short.  Every role of both CTAs walks
+// the same sequence.
 struct Pieces {
-  long long g, g_hi;
-  int u;
+  int g, g_hi;  // stream-K: (unit, K tile) pairs; else: unit
   __device__ __forceinline__ void init(const GmParams& P) {
+    const int b = blockIdx.x >> 1;
     if (P.streamk) {
-      const long long T = (long long)P.units * P.KT;
-      g = T * blockIdx.x / gridDim.x;
-      g_hi = T * (blockIdx.x + 1) / gridDim.x;
+      g = b * P.sk_share + min(b, P.sk_extra);
+      g_hi = g + P.sk_share + (b < P.sk_extra ? 1 : 0);
     } else {
-      u = blockIdx.x;
+      g = b;
     }
   }
   __device__ __forceinline__ bool next(const GmParams& P, int& um, int& un, int& kt_lo,
                                        int& kt_hi) {
-    int uu;
+    int uu, ks = 0;
     if (P.streamk) {
       if (g >= g_hi) return false;
-      uu = (int)(g / P.KT);
-      kt_lo = (int)(g - (long long)uu * P.KT);
-      kt_hi = (int)min((long long)P.KT, (long long)kt_lo + (g_hi - g));
+      uu = g / P.KT;
+      kt_lo = g - uu * P.KT;
+      kt_hi = min(P.KT, kt_lo + (g_hi - g));
       g += kt_hi - kt_lo;
     } else {
-      if (u >= P.units) return false;
-      uu = u;
-      u += gridDim.x;
-      const int ks = uu / (P.units_m * P.units_n);
-      kt_lo = (int)((long long)ks * P.KT / P.ksplit);
-      kt_hi = (int)((long long)(ks + 1) * P.KT / P.ksplit);
+      if (g >= P.units) return false;
+      uu = g;
+      g += gridDim.x >> 1;
+      kt_lo = 0;
+      kt_hi = P.KT;
     }
-    um = uu % P.units_m;
-    un = (uu / P.units_m) % P.units_n;
+    const int q = uu / P.units_m;
+    um = uu - q * P.units_m;
+    un = q;
+    if (P.ksplit > 1) {
+      ks = q / P.units_n;
+      un = q - ks * P.units_n;
+      kt_lo = ks * P.KT / P.ksplit;
+      kt_hi = (ks + 1) * P.KT / P.ksplit;
+    }
     return true;
   }
 };
@@ -216,53 +438,95 @@ struct BlockCursor {
 };
 
 // Position inside a 32-code half group of the code that fills K slot `s`
-// (0..31) of a tile (the order in which the dequantiser emits its fp16 pairs).
+// (0..31) of a tile: the halves of the decoder's pair s / 2 (2, 3 and 4 bits:
+// the pair tables of the GEMV's decoder; 8 and 16 bits: natural order).
 __host__ __device__ inline int slot_code(int bits, int s) {
-  const int h = s & 1;
-  switch (bits) {
-    case 2: return 16 * (s >> 4) + ((s & 15) >> 1) + 8 * h;
-    case 3: return (s >> 1) + 16 * h;
-    case 4: return 8 * (s >> 3) + ((s & 7) >> 1) + 4 * h;
-    default: return s;  // 8- and 16-bit: natural order
+  if (bits > 4) return s;
+  const int gp = gv::group_pairs(bits), j = s >> 1;
+  const gv::PairDef d = gv::pair_def(bits, j % gp);
+  return (j / gp) * gv::group_units(bits) + ((s & 1) ? d.hi : d.lo);
+}
+
+// Shared copy of the block table and of slot_code for every width.
+struct PrepTables {
+  GmBlock blk[POLYQ_MAX_BLOCKS];
+  uint8_t code[5][kSlots];
+};
+__device__ __forceinline__ int width_index(int bits) {
+  return bits <= 4 ? bits - 2 : (bits == 8 ? 3 : 4);
+}
+__device__ __forceinline__ void load_blocks(const GmParams& P, GmBlock* sblk) {
+  if (threadIdx.x < POLYQ_MAX_BLOCKS) {  // constant-offset parameter reads only
+    switch (threadIdx.x) {
+      case 0: sblk[0] = P.blk[0]; break;
+      case 1: sblk[1] = P.blk[1]; break;
+      case 2: sblk[2] = P.blk[2]; break;
+      case 3: sblk[3] = P.blk[3]; break;
+      default: sblk[4] = P.blk[4]; break;
+    }
+  }
+}
+__device__ __forceinline__ void load_tables(const GmParams& P, PrepTables* S) {
+  load_blocks(P, S->blk);
+  if (threadIdx.x < 5 * kSlots) {
+    const int w = threadIdx.x / kSlots;
+    const int bits = w < 3 ? w + 2 : (w == 3 ? 8 : 16);
+    S->code[w][threadIdx.x % kSlots] = (uint8_t)slot_code(bits, threadIdx.x % kSlots);
   }
 }
 
 // ---------------------------------------------------------------------------
-// pre-pass: Xg(m, kt*32 + s) = fp16(X[m][gather[p]] * xscale[p] * 2^-e_m) with
-// p = pos0 + 32 h + slot_code(s)
-// for the h-th 32-code half group of the block (tile kt).  Each CTA first
-// builds, in shared memory, the map from a clustered slot to the source
-// channel it reads (and its activation factor); then, one row at a time, it
-// copies the row of X into shared memory with 16-byte loads (finding the
-// row's largest magnitude on the way) and gathers from there.  Rows up to
-// 16384 wide are held in registers, the next row's loads in flight while the
-// current row is gathered.  Global reads and writes are so coalesced whatever
-// the permutation.  Layers too wide for shared memory (see prep_smem_bytes)
-// gather from global memory instead.  Y is zeroed when the K range is split
-// over CTAs.
+// pre-pass: Xg(m, k) = fp16(X[m][gather[p]] * xscale[p] * 2^-e_m), p the
+// position that fills K slot k (slot_pos).
 // ---------------------------------------------------------------------------
 constexpr int kRowExp = 14;       // a row's largest magnitude becomes [2^14, 2^15)
 constexpr int kRowExpMin = -126;  // 2^e stays a normal float
 constexpr int kPrepThreads = 256;
 constexpr int kPrepMaxSmem = 200 * 1024;
 constexpr int kRowVec = 8;  // 16-byte pieces of a row a thread holds (rows up to 16384 wide)
+constexpr int kSmallQuads = 4;                // 4-slot quads per thread of gemm_prep_small
+constexpr int kSmallMaxK = 32768;             // widest row it stages
 
-// Element offset of Xg(m, k) in the blocked layout: block (m / 256, k / 32)
-// of 256 rows x 32 fp16, row m % 256 at 64 bytes each, its 16-byte chunks
-// in the 64-byte swizzle (chunk index XOR bits 7..8 of the byte address).
-__device__ __forceinline__ size_t xg_off(int m, int k, int KT) {
-  const int r = m & (MT * BM - 1), c = (k >> 3) & 3;
-  return (((size_t)(m / (MT * BM)) * KT + (k >> 5)) * (MT * BM) + r) * BK +
+// Element offset of Xg(m, k) in the blocked layout: block (m / R, k / 32) of
+// R rows x 32 fp16, row m % R at 64 bytes each, its 16-byte chunks in the
+// 64-byte swizzle (chunk index XOR bits 7..8 of the byte address).
+__device__ __forceinline__ size_t xg_off(int m, int k, int kslots, int r_log2) {
+  const int r = m & ((1 << r_log2) - 1), c = (k >> 3) & 3;
+  return ((((size_t)(m >> r_log2) * kslots + (k >> 5)) << r_log2) + r) * kSlots +
          ((c ^ ((r >> 1) & 3)) << 3) + (k & 7);
 }
 
 // Clustered K slot k of a row: the position p it takes its value from, or -1
 // past the end of a block.
-__device__ __forceinline__ int slot_pos(const GmBlock* sblk, int nblk, int k) {
-  const int kt = k / BK, s = k % BK;
-  const GmBlock& B = sblk[find_kblock(sblk, nblk, kt)];
-  const int w = 32 * (kt - B.kt0) + slot_code(B.bits, s);
+__device__ __forceinline__ int slot_pos(const PrepTables& S, int nblk, int bk, int k) {
+  const int kt = bk == 64 ? k >> 6 : k >> 5;
+  const GmBlock& B = S.blk[find_kblock(S.blk, nblk, kt)];
+  const int o = k - B.kt0 * bk;
+  const int w = (o & ~(kSlots - 1)) + S.code[width_index(B.bits)][o & (kSlots - 1)];
   return w < B.n_ch ? B.pos0 + w : -1;
+}
+
+// Y = 0 by CTA `cta` of `n_cta` (Y is 16-byte aligned).
+__device__ __forceinline__ void zero_y(const GmParams& P, int cta, int n_cta) {
+  const long long total = (long long)P.M * P.N, total4 = total / 4;
+  for (long long e = (long long)cta * blockDim.x + threadIdx.x; e < total4;
+       e += (long long)n_cta * blockDim.x)
+    reinterpret_cast<float4*>(P.y)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
+  if (cta == 0 && threadIdx.x < (int)(total & 3)) P.y[total4 * 4 + threadIdx.x] = 0.f;
+}
+
+// e_m = floor(log2(max)) - kRowExp of a row whose largest magnitude has the
+// fp32 bits mx, an fp32 subnormal maximum counting as 2^-127.  2^e and 2^-e
+// are normal floats (-126 <= e <= 113), so the products with 2^-e are exact
+// scalings (rounded like any product where they fall below the normal range).
+__device__ __forceinline__ int row_exp(uint32_t mx) {
+  return mx ? max((int)(mx >> 23) - 127 - kRowExp, kRowExpMin) : 0;
+}
+__device__ __forceinline__ uint32_t bf16x8_max(const uint4& v, uint32_t mx) {
+  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+  for (int q = 0; q < 4; ++q) mx = max(mx, max(w[q] & 0x7FFFu, (w[q] >> 16) & 0x7FFFu));
+  return mx;
 }
 
 // Shared memory of the staged pre-pass: the slot -> source map (int32 [Kp]),
@@ -273,22 +537,24 @@ size_t prep_smem_bytes(int K, int Kp, bool xscale) {
   return b <= (size_t)kPrepMaxSmem ? b : 0;
 }
 
+// Many rows: each CTA first builds, in shared memory, the map from a clustered
+// slot to the source channel it reads (and its activation factor); then, one
+// row at a time, it copies the row of X into shared memory with 16-byte loads
+// (finding the row's largest magnitude on the way) and gathers from there.
+// Rows up to 16384 wide are held in registers, the next row's loads in flight
+// while the current row is gathered.  Global reads and writes are so coalesced
+// whatever the permutation.  Layers too wide for shared memory (see
+// prep_smem_bytes) gather from global memory instead.  Y is zeroed when the K
+// range is split over CTAs.
 __global__ void __launch_bounds__(kPrepThreads) gemm_prep(const __grid_constant__ GmParams P) {
   extern __shared__ __align__(16) uint8_t psm[];
   pdl_trigger();
-  __shared__ GmBlock sblk[POLYQ_MAX_BLOCKS];
+  __shared__ PrepTables S;
   __shared__ uint32_t s_wmax[kPrepThreads / 32];
-  if (threadIdx.x < POLYQ_MAX_BLOCKS) {
-    switch (threadIdx.x) {
-      case 0: sblk[0] = P.blk[0]; break;
-      case 1: sblk[1] = P.blk[1]; break;
-      case 2: sblk[2] = P.blk[2]; break;
-      case 3: sblk[3] = P.blk[3]; break;
-      default: sblk[4] = P.blk[4]; break;
-    }
-  }
+  load_tables(P, &S);
   __syncthreads();
-  const int Kp = P.KT * BK, half = Kp / 2;  // slots and fp16 pairs per row of Xg
+  const int Kp = P.KT * P.bk, half = Kp / 2;  // slots and fp16 pairs per row of Xg
+  const int ks = Kp / kSlots;
   const bool staged = P.prep_staged != 0;
   int* s_src = reinterpret_cast<int*>(psm);
   float* s_fac = reinterpret_cast<float*>(psm + (size_t)Kp * 4);
@@ -303,7 +569,7 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep(const __grid_constant_
 #pragma unroll
       for (int u = 0; u < U; ++u) {
         const int k = k0 + u * kPrepThreads;
-        pos[u] = k < Kp ? slot_pos(sblk, P.n_blocks, k) : -1;
+        pos[u] = k < Kp ? slot_pos(S, P.n_blocks, P.bk, k) : -1;
       }
 #pragma unroll
       for (int u = 0; u < U; ++u) {
@@ -322,12 +588,7 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep(const __grid_constant_
   }
   pdl_wait();  // X comes from the previous kernel; Y and the workspace may still be in use
   if (blockIdx.x == 0 && threadIdx.x == 0) *P.status = 0;
-  if (P.ksplit > 1 || P.streamk) {
-    const long long total4 = (long long)P.M * P.N / 4;
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total4;
-         e += (long long)gridDim.x * blockDim.x)
-      reinterpret_cast<float4*>(P.y)[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-  }
+  if (P.ksplit > 1 || P.streamk) zero_y(P, blockIdx.x, gridDim.x);
   // the value at clustered slot k of row m
   auto value = [&](int m, int k) -> float {
     int src;
@@ -337,29 +598,26 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep(const __grid_constant_
       if (src < 0) return 0.f;
       if (P.xscale) f = s_fac[k];
     } else {
-      const int p = slot_pos(sblk, P.n_blocks, k);
+      const int p = slot_pos(S, P.n_blocks, P.bk, k);
       if (p < 0) return 0.f;
       src = P.gather ? __ldg(P.gather + p) : p;
       if (P.xscale) f = __ldg(P.xscale + p);
     }
     const uint16_t b = staged ? s_row[src]
-                              : __ldg(reinterpret_cast<const uint16_t*>(P.x) + (size_t)m * P.K + src);
+                              : __ldcg(reinterpret_cast<const uint16_t*>(P.x) + (size_t)m * P.K + src);
     return __uint_as_float((uint32_t)b << 16) * f;
   };
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // Row scale of row m from its largest magnitude bits mx (fp32 bit pattern,
-  // per thread): e_m = floor(log2(max)) - kRowExp, an fp32 subnormal maximum
-  // counting as 2^-127.  2^e and 2^-e are normal floats (-126 <= e <= 113),
-  // so the products with 2^-e are exact scalings (rounded like any product
-  // where they fall below the normal range).  Returns 2^-e_m.
-  // The rows of the last M pair past M are zero (their MMA columns are not
-  // stored, but they must be finite).
+  // The rows of the last token tile past M are zero (their MMA columns are
+  // not stored, but they must be finite).
   auto zero_pad_rows = [&]() {
-    const int Mp = P.units_m * (MT * BM);
+    const int Mp = P.units_m << (P.r_log2 + 1);
     for (int m = P.M + blockIdx.x; m < Mp; m += gridDim.x)
       for (int i = threadIdx.x; i < Kp / 4; i += kPrepThreads)
-        *reinterpret_cast<uint2*>(P.xg + xg_off(m, 4 * i, P.KT)) = make_uint2(0u, 0u);
+        *reinterpret_cast<uint2*>(P.xg + xg_off(m, 4 * i, ks, P.r_log2)) = make_uint2(0u, 0u);
   };
+  // Row scale of row m from its largest magnitude bits mx (fp32 bit pattern,
+  // per thread).  Returns 2^-e_m.
   auto row_scale = [&](int m, uint32_t mx) -> float {
     if (P.xscale) {
       mx = 0;
@@ -371,7 +629,7 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep(const __grid_constant_
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < kPrepThreads / 32; ++w) mx = max(mx, s_wmax[w]);
-    const int e = mx ? max((int)(mx >> 23) - 127 - kRowExp, kRowExpMin) : 0;
+    const int e = row_exp(mx);
     if (threadIdx.x == 0) P.rowscale[m] = __int_as_float((127 + e) << 23);
     return __int_as_float((127 - e) << 23);
   };
@@ -387,7 +645,7 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep(const __grid_constant_
 #pragma unroll
       for (int u = 0; u < kRowVec; ++u) {
         const int i = threadIdx.x + u * kPrepThreads;
-        v[u] = i < n8 ? __ldg(row + i) : make_uint4(0u, 0u, 0u, 0u);
+        v[u] = i < n8 ? __ldcg(row + i) : make_uint4(0u, 0u, 0u, 0u);
       }
     };
     uint4 v[kRowVec];
@@ -399,9 +657,7 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep(const __grid_constant_
         const int i = threadIdx.x + u * kPrepThreads;
         if (i < n8) {
           reinterpret_cast<uint4*>(s_row)[i] = v[u];
-          const uint32_t w[4] = {v[u].x, v[u].y, v[u].z, v[u].w};
-#pragma unroll
-          for (int q = 0; q < 4; ++q) mx = max(mx, max(w[q] & 0x7FFFu, (w[q] >> 16) & 0x7FFFu));
+          mx = bf16x8_max(v[u], mx);
         }
       }
       mx <<= 16;  // bf16 magnitude bits -> fp32 bits
@@ -418,7 +674,7 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep(const __grid_constant_
                                            __float2half_rn(value(m, 4 * i + 2 * q + 1) * inv));
           w[q] = *reinterpret_cast<const uint32_t*>(&h);
         }
-        *reinterpret_cast<uint2*>(P.xg + xg_off(m, 4 * i, P.KT)) = make_uint2(w[0], w[1]);
+        *reinterpret_cast<uint2*>(P.xg + xg_off(m, 4 * i, ks, P.r_log2)) = make_uint2(w[0], w[1]);
       }
       __syncthreads();  // the row buffer and s_wmax are reused by the next row
     }
@@ -433,15 +689,13 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep(const __grid_constant_
     uint32_t mx = 0;
     if ((P.K & 7) == 0 && (reinterpret_cast<uintptr_t>(row) & 15) == 0) {
       for (int i = threadIdx.x; i < P.K / 8; i += kPrepThreads) {
-        const uint4 v = __ldg(reinterpret_cast<const uint4*>(row) + i);
+        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(row) + i);
         if (staged) reinterpret_cast<uint4*>(s_row)[i] = v;
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-        for (int q = 0; q < 4; ++q) mx = max(mx, max(w[q] & 0x7FFFu, (w[q] >> 16) & 0x7FFFu));
+        mx = bf16x8_max(v, mx);
       }
     } else {
       for (int i = threadIdx.x; i < P.K; i += kPrepThreads) {
-        const uint16_t v = __ldg(row + i);
+        const uint16_t v = __ldcg(row + i);
         if (staged) s_row[i] = v;
         mx = max(mx, (uint32_t)(v & 0x7FFFu));
       }
@@ -450,7 +704,7 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep(const __grid_constant_
     __syncthreads();  // the staged row (and, on the first row, the map) is complete
     const float inv = row_scale(m, mx);
     for (int i = threadIdx.x; i < half; i += kPrepThreads)
-      *reinterpret_cast<__half2*>(P.xg + xg_off(m, 2 * i, P.KT)) =
+      *reinterpret_cast<__half2*>(P.xg + xg_off(m, 2 * i, ks, P.r_log2)) =
           __halves2half2(__float2half_rn(value(m, 2 * i) * inv),
                          __float2half_rn(value(m, 2 * i + 1) * inv));
     __syncthreads();  // the row buffer and s_wmax are reused by the next row
@@ -458,104 +712,207 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep(const __grid_constant_
   zero_pad_rows();
 }
 
-// ---------------------------------------------------------------------------
-// dequantisation of one weight row of one tile into the swizzled B operand
-// ---------------------------------------------------------------------------
-// Row r, 16-byte chunk c (0..3) of a K-major tile with 64-byte rows and the
-// 64-byte swizzle (chunk index XOR bits 7..8 of the address).
-__device__ __forceinline__ void store_pairs_sw64(uint8_t* btile, int r, int chunk,
-                                                 const uint32_t (&p)[4]) {
-  uint8_t* dst = btile + r * 64 + ((chunk ^ ((r >> 1) & 3)) << 4);
-  *reinterpret_cast<uint4*>(dst) = make_uint4(p[0], p[1], p[2], p[3]);
+// A few rows: prep_seg CTAs per row (of all rows of the token tiles), each
+// gathering a segment of the row's slots, so that even one row is spread over
+// the GPU; further CTAs zero Y.  Every CTA stages the whole row in shared
+// memory and finds its largest magnitude itself.  A thread's gather indices
+// (and factors) are loaded before the wait for the previous kernel.
+__global__ void __launch_bounds__(kPrepThreads) gemm_prep_small(const __grid_constant__ GmParams P) {
+  extern __shared__ __align__(16) uint8_t psm[];
+  pdl_trigger();
+  if ((int)blockIdx.x >= P.prep_rows) {
+    pdl_wait();  // Y may still be in use
+    zero_y(P, (int)blockIdx.x - P.prep_rows, (int)gridDim.x - P.prep_rows);
+    return;
+  }
+  __shared__ PrepTables S;
+  __shared__ uint32_t s_wmax[kPrepThreads / 32];
+  load_tables(P, &S);
+  __syncthreads();
+  const int m = blockIdx.x / P.prep_seg, seg = blockIdx.x % P.prep_seg;
+  const int quads = P.KT * P.bk / 4, ks = P.KT * P.bk / kSlots;
+  const int q_lo = (int)((long long)seg * quads / P.prep_seg);
+  const int q_hi = (int)((long long)(seg + 1) * quads / P.prep_seg);
+  int src[kSmallQuads][4];
+  float fac[kSmallQuads][4];
+#pragma unroll
+  for (int u = 0; u < kSmallQuads; ++u) {
+    const int i = q_lo + u * kPrepThreads + threadIdx.x;
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int p = i < q_hi && m < P.M ? slot_pos(S, P.n_blocks, P.bk, 4 * i + e) : -1;
+      src[u][e] = p < 0 ? -1 : (P.gather ? __ldg(P.gather + p) : p);
+      fac[u][e] = (P.xscale && p >= 0) ? __ldg(P.xscale + p) : 1.f;
+    }
+  }
+  pdl_wait();  // X comes from the previous kernel; the workspace may still be in use
+  if (blockIdx.x == 0 && threadIdx.x == 0) *P.status = 0;
+  float inv = 0.f;
+  const uint16_t* s_row = reinterpret_cast<const uint16_t*>(psm);
+  if (m < P.M) {
+    const uint16_t* row = reinterpret_cast<const uint16_t*>(P.x) + (size_t)m * P.K;
+    uint32_t mx = 0;
+    if ((P.K & 7) == 0 && (reinterpret_cast<uintptr_t>(row) & 15) == 0) {
+      for (int i = threadIdx.x; i < P.K / 8; i += kPrepThreads) {
+        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(row) + i);
+        reinterpret_cast<uint4*>(psm)[i] = v;
+        mx = bf16x8_max(v, mx);
+      }
+    } else {
+      for (int i = threadIdx.x; i < P.K; i += kPrepThreads) {
+        const uint16_t v = __ldcg(row + i);
+        reinterpret_cast<uint16_t*>(psm)[i] = v;
+        mx = max(mx, (uint32_t)(v & 0x7FFFu));
+      }
+    }
+    mx <<= 16;  // bf16 magnitude bits -> fp32 bits
+    __syncthreads();
+    if (P.xscale) {  // the largest |x * t| over the whole row
+      mx = 0;
+      for (int p = threadIdx.x; p < P.K; p += kPrepThreads) {
+        const int c = P.gather ? __ldg(P.gather + p) : p;
+        mx = max(mx, __float_as_uint(fabsf(__uint_as_float((uint32_t)s_row[c] << 16) *
+                                           __ldg(P.xscale + p))));
+      }
+    }
+    mx = __reduce_max_sync(0xffffffffu, mx);
+    if ((threadIdx.x & 31) == 0) s_wmax[threadIdx.x >> 5] = mx;
+    __syncthreads();
+#pragma unroll
+    for (int w = 0; w < kPrepThreads / 32; ++w) mx = max(mx, s_wmax[w]);
+    const int e = row_exp(mx);
+    if (seg == 0 && threadIdx.x == 0) P.rowscale[m] = __int_as_float((127 + e) << 23);
+    inv = __int_as_float((127 - e) << 23);
+  }
+#pragma unroll
+  for (int u = 0; u < kSmallQuads; ++u) {
+    const int i = q_lo + u * kPrepThreads + threadIdx.x;
+    if (i >= q_hi) break;
+    float v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e)
+      v[e] = src[u][e] < 0
+                 ? 0.f
+                 : __uint_as_float((uint32_t)s_row[src[u][e]] << 16) * fac[u][e] * inv;
+    const __half2 a = __halves2half2(__float2half_rn(v[0]), __float2half_rn(v[1]));
+    const __half2 b = __halves2half2(__float2half_rn(v[2]), __float2half_rn(v[3]));
+    *reinterpret_cast<uint2*>(P.xg + xg_off(m, 4 * i, ks, P.r_log2)) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+  }
 }
 
+// ---------------------------------------------------------------------------
+// dequantisation of one weight row of one tile into the swizzled A operand
+// ---------------------------------------------------------------------------
 __device__ __forceinline__ void red_add_f32(float* p, float a) {
   asm volatile("red.global.add.f32 [%0], %1;" ::"l"(p), "f"(a) : "memory");
 }
 
-__device__ __forceinline__ uint32_t dq_pair(uint32_t raw, __half2 zz, __half2 ss) {
-  // raw holds fp16 (1024 + q) in each half: (q - z) is exact, the product
-  // (q - z) * s is rounded once to fp16.
-  const __half2 d = __hsub2(*reinterpret_cast<const __half2*>(&raw), zz);
-  const __half2 w = __hmul2(d, ss);
-  return *reinterpret_cast<const uint32_t*>(&w);
+__device__ __forceinline__ __half2 half2_bits(uint32_t v) {
+  return *reinterpret_cast<const __half2*>(&v);
+}
+// fp16 bits of 2^-p and of -1024 * 2^-p (0 <= p <= 8)
+__host__ __device__ constexpr uint32_t h_pow2(int p) { return (uint32_t)(15 - p) << 10; }
+__host__ __device__ constexpr uint32_t h_neg_magic(int p) {
+  return 0x8000u | ((uint32_t)(25 - p) << 10);
 }
 
-// Dequantise 32 codes of weight row r.  `w` holds the row's code words
-// starting at the first code (2-bit: 2 words, 3-bit: 3, 4-bit: 4, 8-bit: 8).
-__device__ __forceinline__ void dequant_row(int bits, const uint32_t (&w)[8], uint32_t meta,
-                                            uint8_t* btile, int r) {
-  const uint32_t magic = 0x64006400u;
-  const __half s = __ushort_as_half((uint16_t)(meta & 0xFFFFu));
-  const __half z = __ushort_as_half((uint16_t)(meta >> 16));
-  const __half2 ss = __halves2half2(s, s);
-  const __half zz1 = __hadd(z, __float2half(1024.f));
-  const __half2 zz = __halves2half2(zz1, zz1);
-  if (bits == 2) {
+// Dequantise the 32 codes of a half group (w: its code words, from the first
+// code's bit 0) into the 16 fp16 pairs of an operand row.  A code pair is cut out of the
+// stream as two fp16 values 1024 + q * 2^p with one LOP3 (the GEMV decoder's
+// windows); an FMA by 2^-p with -(1024 * 2^-p + z) gives q - z exactly (every
+// intermediate is an integer or a short binary fraction of at most 11 bits),
+// and the product with s is rounded once to fp16.  Three instructions a pair
+// and seven window shifts per 32 codes at 3 bits, instead of six a pair with
+// every code shifted to bit 0.
+template <int BITS>
+__device__ __forceinline__ void dequant_half(const uint32_t* w, __half2 zz, __half2 ss,
+                                             uint32_t magic, uint32_t* p) {
 #pragma unroll
-    for (int wd = 0; wd < 2; ++wd) {
-#pragma unroll
-      for (int c2 = 0; c2 < 2; ++c2) {
-        uint32_t p[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int ii = 4 * c2 + i;
-          p[i] = dq_pair(((w[wd] >> (2 * ii)) & 0x00030003u) | magic, zz, ss);
-        }
-        store_pairs_sw64(btile, r, 2 * wd + c2, p);
-      }
+  for (int j = 0; j < 16; ++j) {
+    __half2 d;
+    if constexpr (BITS == 8) {
+      const uint32_t v = __byte_perm(w[j >> 1], 0x64646464u, (j & 1) ? 0x4342 : 0x4140);
+      d = __hadd2(half2_bits(v), __hsub2(half2_bits(h_neg_magic(0) * 0x10001u), zz));
+    } else {
+      const gv::PairDef pd = gv::pair_def(BITS, j % gv::group_pairs(BITS));
+      const uint32_t v = gv::make_pair<BITS>(w, j, magic);
+      const uint32_t mul = h_pow2(pd.plo) | (h_pow2(pd.phi) << 16);
+      const uint32_t neg = h_neg_magic(pd.plo) | (h_neg_magic(pd.phi) << 16);
+      d = __hfma2(half2_bits(v), half2_bits(mul), __hsub2(half2_bits(neg), zz));
     }
-  } else if (bits == 3) {
-    const uint32_t a = w[0], b = w[1], c = w[2];
-#pragma unroll
-    for (int c4 = 0; c4 < 4; ++c4) {
-      uint32_t p[4];
-#pragma unroll
-      for (int i4 = 0; i4 < 4; ++i4) {
-        const int i = 4 * c4 + i4;  // codes i and i + 16
-        const int o = 3 * i;
-        const uint32_t lo = o < 32 ? __funnelshift_r(a, b, o) : __funnelshift_r(b, c, o - 32);
-        const uint32_t hi = o < 32 ? __funnelshift_r(b, c, o) : (c >> (o - 32));
-        p[i4] = dq_pair((__byte_perm(lo, hi, 0x7610) & 0x00070007u) | magic, zz, ss);
-      }
-      store_pairs_sw64(btile, r, c4, p);
-    }
-  } else if (bits == 4) {
-#pragma unroll
-    for (int wd = 0; wd < 4; ++wd) {
-      uint32_t p[4];
-#pragma unroll
-      for (int i = 0; i < 4; ++i) p[i] = dq_pair(((w[wd] >> (4 * i)) & 0x000F000Fu) | magic, zz, ss);
-      store_pairs_sw64(btile, r, wd, p);
-    }
-  } else {  // 8-bit
-#pragma unroll
-    for (int c = 0; c < 4; ++c) {
-      uint32_t p[4];
-      p[0] = dq_pair(__byte_perm(w[2 * c], 0x64646464u, 0x4140), zz, ss);
-      p[1] = dq_pair(__byte_perm(w[2 * c], 0x64646464u, 0x4342), zz, ss);
-      p[2] = dq_pair(__byte_perm(w[2 * c + 1], 0x64646464u, 0x4140), zz, ss);
-      p[3] = dq_pair(__byte_perm(w[2 * c + 1], 0x64646464u, 0x4342), zz, ss);
-      store_pairs_sw64(btile, r, c, p);
-    }
+    const __half2 q = __hmul2(d, ss);
+    p[j] = *reinterpret_cast<const uint32_t*>(&q);
   }
 }
 
+template <int V>
+struct IntC {
+  static constexpr int value = V;
+};
+
+// Shared memory by 32-bit address (the tile pointers, aligned by hand, are
+// generic to the compiler, and generic accesses cost it 64-bit arithmetic).
+__device__ __forceinline__ uint32_t lds32(uint32_t a) {
+  uint32_t v;
+  asm volatile("ld.shared.u32 %0, [%1];" : "=r"(v) : "r"(a) : "memory");
+  return v;
+}
+__device__ __forceinline__ void lds128(uint32_t a, uint32_t* v) {
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v[0]), "=r"(v[1]), "=r"(v[2]), "=r"(v[3])
+               : "r"(a)
+               : "memory");
+}
+__device__ __forceinline__ void sts128(uint32_t a, const uint32_t* v) {
+  asm volatile("st.shared.v4.u32 [%0], {%1,%2,%3,%4};" ::"r"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]),
+               "r"(v[3])
+               : "memory");
+}
+
+// The code words of a tile row in registers, from the first code's bit 0: the
+// codes start `off` bytes (uniform over the CTA) into the row's box row at
+// address `a`: at 0 or (3 bits) 8 for a tile of 64, also at 4 or 12 for one of
+// 32.  An 8-bit tile of 64 has a second box, read by the caller.
+template <int BITS, int HALVES>
+struct CodeWords {
+  static constexpr int N = BITS == 8 ? 8 : BITS * HALVES;
+  uint32_t w[N];
+  __device__ __forceinline__ void load(uint32_t a, int off) {
+    constexpr bool kShift = BITS == 3 || (BITS == 2 && HALVES == 1);
+    uint32_t cw[8];
+    lds128(a, cw);
+    if (kShift || N > 4) lds128(a + 16, cw + 4);
+    const int sh = kShift ? off >> 2 : 0;
+#pragma unroll
+    for (int k = 0; k < N; ++k) {
+      uint32_t v = cw[k];
+      if (kShift) v = sh >= 2 ? cw[k + 2] : v;
+      if (BITS == 3 && HALVES == 1) {
+        const uint32_t o = sh >= 2 ? cw[k + 3] : cw[k + 1];
+        v = (sh & 1) ? o : v;
+      }
+      w[k] = v;
+    }
+  }
+};
+
 #ifdef POLYQ_DEBUG
 // Debug build only: every fp16 weight the dequantisers (or, for 16-bit
-// blocks, TMA) place in a B tile is written to g_dbg_w[n][position] (the
+// blocks, TMA) place in an A tile is written to g_dbg_w[n][position] (the
 // layer's clustered order), read back from the swizzled tile.
 __device__ uint16_t* g_dbg_w;
 __device__ long long g_dbg_wK;
 
-__device__ __forceinline__ void dbg_row(const uint8_t* btile, int r, int n, int N,
+// Half tile `tile` holds the block's half group hg.
+__device__ __forceinline__ void dbg_row(const uint8_t* tile, int r, int n, int N,
                                         const GmBlock& B, int hg) {
   uint16_t* out = g_dbg_w;
   if (!out || n >= N) return;
 #pragma unroll
   for (int c = 0; c < 4; ++c) {
     const uint16_t* src =
-        reinterpret_cast<const uint16_t*>(btile + r * 64 + ((c ^ ((r >> 1) & 3)) << 4));
+        reinterpret_cast<const uint16_t*>(tile + r * 64 + ((c ^ ((r >> 1) & 3)) << 4));
 #pragma unroll
     for (int e = 0; e < 8; ++e) {
       const int w = 32 * hg + slot_code(B.bits, 8 * c + e);
@@ -565,320 +922,498 @@ __device__ __forceinline__ void dbg_row(const uint8_t* btile, int r, int n, int 
 }
 #endif
 
-__global__ void __launch_bounds__(kThreadsG, 1) gemm_main(const __grid_constant__ GmParams P) {
+// One chunk of 32 accumulator columns (tokens m0.., lane j holding token j's
+// row scale) of the warp's 32 output columns into Y: v * 2^e_m, stored or
+// (split K) added.  Nothing here depends from token to token (a token's
+// address is one multiply), because a warp runs this alone and waits out
+// every dependent instruction: with a running 64-bit pointer and a test per
+// token the chunk took 2500 cycles whatever the number of warps, now 1100.
+template <bool ADD>
+__device__ __forceinline__ void store_chunk(float* __restrict__ y, uint32_t N, bool ok, int jn,
+                                            const uint32_t (&v)[32], float rs_l) {
+  float f[32];
+#pragma unroll
+  for (int j = 0; j < 32; ++j)
+    f[j] = __uint_as_float(v[j]) * __shfl_sync(0xffffffffu, rs_l, j);
+  if (!ok) return;
+  if (jn == 32) {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+      float* dst = y + (size_t)N * (uint32_t)j;
+      if (ADD) red_add_f32(dst, f[j]);
+      else *dst = f[j];
+    }
+  } else {
+#pragma unroll
+    for (int j = 0; j < 32; ++j) {
+      float* dst = y + (size_t)N * (uint32_t)j;
+      if (j < jn) {
+        if (ADD) red_add_f32(dst, f[j]);
+        else *dst = f[j];
+      }
+    }
+  }
+}
+
+// What bounds it, by token tile (13824 x 5120 at B = 3, one call): with 512
+// tokens the tensor core: a stage of 32 K takes 507 cycles of the MMAs' 512,
+// an accumulator drain 9400 cycles per 95000 of a unit (M = 2048: 277 -> 177
+// us; M = 4096: 529 -> 354 us, 1640 TFLOP/s).  With 256 and fewer the latency
+// of a stage of 64 K through its rings, 540 to 620 cycles (M = 256: 53.6 -> 38
+// us, M = 96: 54 -> 30 us, M = 16: 53 -> 26 us): the copy of 128 code rows and
+// 128 meta rows (325 cycles of the TMA unit, which takes a row a cycle and 32
+// bytes across a 32-byte boundary as two), dequantisation, the arrival at the
+// leader and the commit back.  "Before" is one CTA per tile of 256 x 256
+// whatever M, which dequantised every weight once per SM and 256 tokens.
+template <class C>
+__global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constant__ GmParams P,
+                                                            uint32_t magic) {
   extern __shared__ __align__(1024) uint8_t smem_raw[];
-  // 1024-byte alignment of the operand tiles (128-byte swizzle atoms)
+  // 1024-byte alignment of the operand tiles; both CTAs of the pair have the
+  // same layout, so the offsets agree, as the MMA's descriptors need
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~(uintptr_t)1023);
-  __shared__ uint64_t bar_full[kStagesG], bar_bready[kStagesG], bar_sfree[kStagesG];
-  __shared__ uint64_t bar_accf, bar_acce;
+  uint8_t* smem_codes = smem + C::kCodeOff;
+  __shared__ uint64_t bar_cfull[C::CODES];  // a code slot's copies have landed
+  __shared__ uint64_t bar_cfree[C::CODES];  // its dequantisers hold the codes in registers
+  __shared__ uint64_t bar_xfull[C::XS];     // a token slot's copy has landed (leader: both CTAs')
+  __shared__ uint64_t bar_xfree[C::XS];     // its MMAs are done
+  __shared__ uint64_t bar_bready[C::OPS];   // leader: both CTAs' weights are in place
+  __shared__ uint64_t bar_sfree[C::OPS];    // a weight slot's MMAs are done
+  __shared__ uint64_t bar_w16[C::GROUPS];   // a group's tile of fp16 weights has landed
+  __shared__ uint64_t bar_accf[C::NBUF];    // an accumulator is complete
+  __shared__ uint64_t bar_acce[C::NBUF];    // leader: both CTAs have drained it
+  __shared__ uint64_t bar_done;             // every MMA is done (the leader waits for it)
   __shared__ uint32_t tmem_base_slot;
   __shared__ GmBlock sblk[POLYQ_MAX_BLOCKS];
   __shared__ volatile int s_abort;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t rank = cluster_ctarank();
+  const int role = warp >= C::kEpiWarp ? kRoleEpilogue : (warp & 3) == 0 ? warp >> 2 : kRoleDequant;
 
-  if (threadIdx.x < POLYQ_MAX_BLOCKS) {
-    switch (threadIdx.x) {
-      case 0: sblk[0] = P.blk[0]; break;
-      case 1: sblk[1] = P.blk[1]; break;
-      case 2: sblk[2] = P.blk[2]; break;
-      case 3: sblk[3] = P.blk[3]; break;
-      default: sblk[4] = P.blk[4]; break;
-    }
-  }
+  load_blocks(P, sblk);
   if (threadIdx.x == 0) {
     s_abort = 0;
-    for (int s = 0; s < kStagesG; ++s) {
-      mbar_init(smem_u32(&bar_full[s]), 1);
-      mbar_init(smem_u32(&bar_bready[s]), kDqWarps / 2);  // one group of four warps per stage
+    for (int s = 0; s < C::CODES; ++s) {
+      mbar_init(smem_u32(&bar_cfull[s]), 1);
+      mbar_init(smem_u32(&bar_cfree[s]), 4);  // one group of four warps
+    }
+    for (int s = 0; s < C::OPS; ++s) {
+      mbar_init(smem_u32(&bar_bready[s]), 2 * 4);  // a group of each CTA
       mbar_init(smem_u32(&bar_sfree[s]), 1);
     }
-    mbar_init(smem_u32(&bar_accf), 1);
-    mbar_init(smem_u32(&bar_acce), kDqWarps);
+    for (int s = 0; s < C::XS; ++s) {
+      mbar_init(smem_u32(&bar_xfull[s]), rank == 0 ? 2 : 1);  // the producer; the peer's relay
+      mbar_init(smem_u32(&bar_xfree[s]), 1);
+    }
+    for (int g = 0; g < C::GROUPS; ++g) mbar_init(smem_u32(&bar_w16[g]), 1);
+    for (int b = 0; b < C::NBUF; ++b) {
+      mbar_init(smem_u32(&bar_accf[b]), 1);
+      mbar_init(smem_u32(&bar_acce[b]), 2 * C::EPI);
+    }
+    mbar_init(smem_u32(&bar_done), 1);
     mbar_fence_init();
   }
-  if (warp == 1) {
-    tmem_alloc(smem_u32(&tmem_base_slot), kTmemCols);
-    tmem_relinquish();
+  // one warp of each CTA of the pair allocates, and later frees, for the pair
+  if (role == kRoleMma) {
+    tmem_alloc2(smem_u32(&tmem_base_slot), kTmemCols);
+    tmem_relinquish2();
   }
   tc_fence_before();
   __syncthreads();
+  cluster_sync();  // the peer's barriers are initialised too
   tc_fence_after();
   const uint32_t tmem = tmem_base_slot;
   pdl_trigger();
 
   const int nblk = P.n_blocks;
-  auto stage_ptr = [&](int s) { return smem + s * kStageG; };
   auto fail = [&](int code) {
     s_abort = 1;
+    const uint32_t peer = mapa(smem_u32((const void*)&s_abort), rank ^ 1u);
+    asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(peer), "r"(1) : "memory");
     atomicExch(P.status, code);
   };
+  Pieces pc;
+  pc.init(P);
+  int um, un, kt_lo, kt_hi;
+  BlockCursor B;
 
-  if (warp == 0) {
-    // ---------------- TMA producer ----------------
-    if (lane == 0) {
+  if (role <= kRoleCode1) {
+    // ---------------- code producers: stages k with k % kCodeProd == role ----------------
+    // The packed weights do not depend on earlier kernels, so these copies
+    // start before the pre-pass is done.
+    if (elect_one()) {
       prefetch_tmap(&P.tm_codes);
       if (P.has_meta) prefetch_tmap(&P.tm_meta);
-      prefetch_tmap(&P.tm_w16);
-      pdl_wait();  // Xg comes from the pre-pass
-      int kg = 0;
-      Pieces pc;
-      pc.init(P);
-      int um, un, kt_lo, kt_hi;
-      BlockCursor B;
+      constexpr int kAhead = C::CODES / C::kCodeProd / 2;  // stages polled at once
+      int kg = 0, last = -1;  // stages before this piece; last stage issued
+      int s = role, free = 0;
+      uint32_t ph = 1;  // a fresh barrier's parity-1 phase counts as complete
       while (!s_abort && pc.next(P, um, un, kt_lo, kt_hi)) {
         B.seek(sblk, nblk, kt_lo);
-        for (int kt = kt_lo; kt < kt_hi; ++kt, ++kg) {
-          const int s = kg % kStagesG, use = kg / kStagesG;
-          if (use > 0) {
-            const int w = wait_sleep_ab(smem_u32(&bar_sfree[s]), (use - 1) & 1, &s_abort);
-            if (w != kWaitOk) {
-              if (w == kWaitTimeout) fail(kStatusTimeoutEmpty);
-              break;
+        const int n_row = un * kRowsN + (int)rank * kRowsCta;
+        int kt = kt_lo + (role + C::kCodeProd - kg % C::kCodeProd) % C::kCodeProd;
+        for (; kt < kt_hi; kt += C::kCodeProd) {
+          if (free == 0) {
+            free = leading(poll_ahead<kAhead, C::CODES, C::kCodeProd>(smem_u32(&bar_cfree[0]), s, ph));
+            if (free == 0) {
+              const int w = wait_sleep_ab(smem_u32(&bar_cfree[s]), ph, &s_abort);
+              if (w != kWaitOk) {
+                if (w == kWaitTimeout) fail(kStatusTimeoutEmpty);
+                break;
+              }
+              free = 1;
             }
           }
+          --free;
           B.advance(sblk, nblk, kt);
-          const int hg = kt - B.kt0;  // half group
-          uint8_t* st = stage_ptr(s);
-          const uint32_t bar = smem_u32(&bar_full[s]);
-          const bool w16 = B.bits == 16;
-          mbar_expect_tx(bar, MT * kATile + (w16 ? kBTile : kCodes + kMeta));
-          // both M tiles of X: one 16 KB block of Xg, already in the
-          // swizzled shared-memory layout
-          bulk_load(smem_u32(st), P.xg + ((size_t)um * P.KT + kt) * (MT * BM * BK), MT * kATile,
-                    bar);
-          if (w16) {
-            tma_load_2d(smem_u32(st + MT * kATile), &P.tm_w16, (B.seg_off + 64 * hg) / 2, un * BN,
-                        bar);
+          const uint32_t bar = smem_u32(&bar_cfull[s]);
+          if (B.bits == 16) {  // no codes: the weights go straight to the weight slot
+            mbar_arrive(bar);
           } else {
-            const int start = B.seg_off + 4 * B.bits * hg;
-            tma_load_2d(smem_u32(st + MT * kATile + kBTile), &P.tm_codes, start & ~15, un * BN,
-                        bar);
-            tma_load_2d(smem_u32(st + MT * kATile + kBTile + kCodes), &P.tm_meta,
-                        (B.grp_off + hg / 2) & ~3, un * BN, bar);
+            const uint32_t st = smem_u32(smem_codes + s * C::kCode);
+            const int tb = kt - B.kt0;  // tile of the block
+            const int boxes = B.bits == 8 ? C::HALVES : 1;
+            const int start = B.seg_off + (C::BK / 8) * B.bits * tb;
+            mbar_expect_tx(bar, boxes * kBoxBytes + kMetaBytes);
+            tma_load_2d(st, &P.tm_codes, start & ~15, n_row, bar);
+            if (boxes == 2) tma_load_2d(st + kBoxBytes, &P.tm_codes, start + kCodeBox, n_row, bar);
+            tma_load_2d(st + C::kCodes, &P.tm_meta, (B.grp_off + tb * C::BK / 64) & ~3, n_row, bar);
+          }
+          last = kg + (kt - kt_lo);
+          s += C::kCodeProd;
+          if (s >= C::CODES) {
+            s -= C::CODES;
+            ph ^= 1u;
+          }
+        }
+        kg += kt_hi - kt_lo;
+      }
+      // wait (bounded) for the copies still in flight: only a slot's last use,
+      // whose phase no other producer has moved on
+      for (int k = last; k >= 0 && k > (s_abort ? last : kg - 1) - C::CODES; k -= C::kCodeProd)
+        mbar_wait(smem_u32(&bar_cfull[k % C::CODES]), (k / C::CODES) & 1);
+    }
+  } else if (role == kRoleX) {
+    // ---------------- X producer ----------------
+    if (elect_one()) {
+      pdl_wait();  // Xg comes from the pre-pass
+      constexpr int kAhead = C::XS / 2;
+      int k = 0, s = 0, free = 0;
+      uint32_t ph = 1;
+      while (!s_abort && pc.next(P, um, un, kt_lo, kt_hi)) {
+        const __half* xg = P.xg + (size_t)(um * 2 + (int)rank) * P.KT * (C::BK * C::R);
+        for (int kt = kt_lo; kt < kt_hi; ++kt, ++k) {
+          if (free == 0) {
+            free = leading(poll_ahead<kAhead, C::XS>(smem_u32(&bar_xfree[0]), s, ph));
+            if (free == 0) {
+              const int w = wait_sleep_ab(smem_u32(&bar_xfree[s]), ph, &s_abort);
+              if (w != kWaitOk) {
+                if (w == kWaitTimeout) fail(kStatusTimeoutEmpty);
+                break;
+              }
+              free = 1;
+            }
+          }
+          --free;
+          // this CTA's tokens: one contiguous block of Xg, already swizzled
+          const uint32_t bar = smem_u32(&bar_xfull[s]);
+          mbar_expect_tx(bar, C::kX);
+          bulk_load(smem_u32(smem + C::kXOff + s * C::kX), xg + (size_t)kt * (C::BK * C::R), C::kX,
+                    bar);
+          if (++s == C::XS) {
+            s = 0;
+            ph ^= 1u;
+          }
+        }
+      }
+      if (rank != 0)  // copies still in flight (the leader's MMA thread waits for its own)
+        for (int j = max(0, k - C::XS); j < k; ++j)
+          mbar_wait(smem_u32(&bar_xfull[j % C::XS]), (j / C::XS) & 1);
+    }
+  } else if (role == kRoleMma && rank != 0) {
+    // ---------------- X relay (second CTA) ----------------
+    // Tells the leader's MMA thread that this CTA's X of a stage has landed.
+    if (elect_one()) {
+      const uint32_t xfull0 = mapa(smem_u32(&bar_xfull[0]), 0);
+      constexpr int kAhead = C::XS / 2;
+      int s = 0, ready = 0;
+      uint32_t ph = 0;
+      while (!s_abort && pc.next(P, um, un, kt_lo, kt_hi)) {
+        for (int kt = kt_lo; kt < kt_hi; ++kt) {
+          if (ready == 0) {
+            ready = leading(poll_ahead<kAhead, C::XS>(smem_u32(&bar_xfull[0]), s, ph));
+            if (ready == 0) {
+              const int w = wait_sleep_ab(smem_u32(&bar_xfull[s]), ph, &s_abort);
+              if (w != kWaitOk) {
+                if (w == kWaitTimeout) fail(kStatusTimeoutFull);
+                break;
+              }
+              ready = 1;
+            }
+          }
+          --ready;
+          mbar_arrive_cluster(xfull0 + 8 * s);
+          if (++s == C::XS) {
+            s = 0;
+            ph ^= 1u;
           }
         }
       }
     }
-  } else if (warp == 1) {
-    // ---------------- MMA issuer ----------------
-    if (lane == 0) {
-      int uc = 0, s = 0;
-      uint32_t ph = 0;
-      const uint64_t dx0 = umma_desc_sw64(smem_u32(smem));
-      const uint64_t dw0 = umma_desc_sw64(smem_u32(smem + MT * kATile));
-      Pieces pc;
-      pc.init(P);
-      int um, un, kt_lo, kt_hi;
+  } else if (role == kRoleMma) {
+    // ---------------- MMA issuer (leader CTA) ----------------
+    if (elect_one()) {
+      constexpr int kAhead = C::OPS / 2;
+      int uc = 0, s = 0, xs = 0, ready = 0;
+      uint32_t ph = 0, xph = 0;
+      const uint64_t da0 = umma_desc_sw64(smem_u32(smem));
+      const uint64_t dx0 = umma_desc_sw64(smem_u32(smem + C::kXOff));
       for (; !s_abort && pc.next(P, um, un, kt_lo, kt_hi); ++uc) {
-        if (uc > 0) {
-          const int w = wait_sleep_ab(smem_u32(&bar_acce), (uc - 1) & 1, &s_abort);
+        const int buf = uc % C::NBUF;
+        if (uc >= C::NBUF) {
+          const int w =
+              wait_sleep_ab(smem_u32(&bar_acce[buf]), (uc / C::NBUF - 1) & 1, &s_abort);
           if (w != kWaitOk) {
             if (w == kWaitTimeout) fail(kStatusTimeoutEmpty);
             break;
           }
         }
         tc_fence_after();
+        const uint32_t acc = tmem + buf * (C::NACC * C::TN);
         for (int kt = kt_lo; kt < kt_hi; ++kt) {
-          // Every dequantiser warp of the stage's group waits for the
-          // stage's copies (bar_full) before it arrives on bar_bready, so
-          // bar_bready alone orders the MMAs after the X tile and the weights.
-          const int w = wait_sleep_ab(smem_u32(&bar_bready[s]), ph, &s_abort);
-          if (w != kWaitOk) {
-            if (w == kWaitTimeout) fail(kStatusTimeoutFull);
-            break;
+          if (ready == 0) {
+            ready = leading(poll_ahead<kAhead, C::OPS>(smem_u32(&bar_bready[0]), s, ph) &
+                            poll_ahead<kAhead, C::XS>(smem_u32(&bar_xfull[0]), xs, xph));
+            if (ready == 0) {
+              int w = wait_sleep_ab(smem_u32(&bar_bready[s]), ph, &s_abort);
+              if (w == kWaitOk) w = wait_sleep_ab(smem_u32(&bar_xfull[xs]), xph, &s_abort);
+              if (w != kWaitOk) {
+                if (w == kWaitTimeout) fail(kStatusTimeoutFull);
+                break;
+              }
+              ready = 1;
+            }
           }
+          --ready;
           tc_fence_after();
-          // A: 128 of the tile's 256 weight rows; B: all 256 tokens of the M
-          // pair (one 256-row box).  Accumulator t holds weight rows 128 t..
-          // in its TMEM lanes and the tokens in its 256 columns.  The slot's
-          // descriptors are those of slot 0 plus its offset (address >> 4).
-          const uint64_t so = (uint64_t)((s * kStageG) >> 4);
-          const uint64_t dx = dx0 + so, dw = dw0 + so;
+          // A: the pair's 256 weight rows; B: accumulator a's TN tokens.  The
+          // slots' descriptors are those of slot 0 plus an offset (>> 4).
+          const uint64_t da = da0 + (uint64_t)((s * C::kA) >> 4);
+          const uint64_t dx = dx0 + (uint64_t)((xs * C::kX) >> 4);
 #pragma unroll
-          for (int t = 0; t < MT; ++t)
+          for (int a = 0; a < C::NACC; ++a)
 #pragma unroll
-            for (int kk = 0; kk < BK / 16; ++kk)
-              tc_mma_f16(tmem + t * BN, dw + (uint64_t)((t * BM * BK * 2) >> 4) + 2 * kk, dx + 2 * kk,
-                         kIdesc, (kt > kt_lo || kk > 0) ? 1u : 0u);
-          tc_commit(smem_u32(&bar_sfree[s]));
-          if (++s == kStagesG) {
+            for (int kk = 0; kk < C::BK / 16; ++kk)
+              tc_mma2_f16(acc + a * C::TN,
+                          da + (uint64_t)((kk / 2) * (kHalfTile >> 4) + 2 * (kk & 1)),
+                          dx + (uint64_t)((kk / 2) * ((C::R * 64) >> 4) + a * ((C::TN / 2 * 64) >> 4) +
+                                          2 * (kk & 1)),
+                          C::kIdesc, (kt > kt_lo || kk > 0) ? 1u : 0u);
+          tc_commit2(smem_u32(&bar_sfree[s]));
+          tc_commit2(smem_u32(&bar_xfree[xs]));
+          if (++s == C::OPS) {
             s = 0;
             ph ^= 1u;
           }
+          if (++xs == C::XS) {
+            xs = 0;
+            xph ^= 1u;
+          }
         }
-        tc_commit(smem_u32(&bar_accf));
+        tc_commit2(smem_u32(&bar_accf[buf]));
       }
+      // the pair's shared and tensor memory stay in use until the last MMA is done
+      tc_commit2(smem_u32(&bar_done));
+      mbar_wait(smem_u32(&bar_done), 0);
     }
-  } else {
-    // ---------------- dequantisation + epilogue (8 warps) ----------------
-    // Two groups of four warps take alternate stages (group g the stages
-    // with kg % 2 == g); a thread dequantises rows r0 and r0 + 128 of its
-    // group's stages.  Each group so has two stage periods for its
-    // latency-bound work, and each thread two independent rows.
-    const int dq = threadIdx.x - 64;  // 0..255
-    const int grp = dq >> 7;
-    const int r0 = dq & 127;
-    const int q = warp & 3;          // TMEM lane quarter this warp may access
-    const int half = (warp - 2) >> 2;
-    int kg = 0, uc = 0;
-    Pieces pc;
-    pc.init(P);
-    int um, un, kt_lo, kt_hi;
-    BlockCursor B;
-    for (; !s_abort && pc.next(P, um, un, kt_lo, kt_hi); ++uc) {
+  } else if (role == kRoleDequant) {
+    // ---------------- dequantisation ----------------
+    // Group g takes the stages k with k % GROUPS == g, thread r of the group
+    // weight row r of the CTA.  (Copies may land out of order, and a parity
+    // wait cannot tell a phase from the last but one: a code slot always
+    // belongs to one group, as GROUPS divides CODES.)
+    const int dq = (warp >> 2) * 3 + (warp & 3) - 1;  // 0..11
+    const int grp = dq >> 2;
+    const int r = (dq & 3) * 32 + lane;
+    const uint32_t code_row = smem_u32(smem_codes) + r * kCodeBox;
+    const uint32_t meta_row = smem_u32(smem_codes) + C::kCodes + r * 16;
+    // 16-byte chunk c of operand row r lies at (c XOR bits 7..8 of the row's
+    // address) under the 64-byte swizzle
+    const uint32_t op_row = smem_u32(smem) + r * 64 + (((r >> 1) & 3) << 4);
+    const uint32_t bready0 = mapa(smem_u32(&bar_bready[0]), 0);  // the leader's
+    int sc = grp, s = grp;  // code and weight slot of the group's next stage
+    uint32_t cph = 0, sph = 1, w16_ph = 0;
+    int skip = grp;  // stages until the group's next one
+    while (!s_abort && pc.next(P, um, un, kt_lo, kt_hi)) {
       B.seek(sblk, nblk, kt_lo);
-      for (int kt = kt_lo; kt < kt_hi; ++kt, ++kg) {
-        if ((kg & 1) != grp) continue;
-        const int s = kg % kStagesG, use = kg / kStagesG;
-        // The producer issues a slot's copies only after the MMAs of its
-        // previous use are done, so once they have landed the weight tile
-        // may be overwritten too.
-        const int w = wait_ab(smem_u32(&bar_full[s]), use & 1, &s_abort);
+      int kt = kt_lo + skip;
+      for (; kt < kt_hi; kt += C::GROUPS) {
+        int w = wait_ab(smem_u32(&bar_cfull[sc]), cph, &s_abort);
         if (w != kWaitOk) {
           if (w == kWaitTimeout) fail(kStatusTimeoutFull);
           break;
         }
+        // polled once while the codes are on their way to registers; the slot
+        // is waited for only before the stores
+        const bool free = mbar_test(smem_u32(&bar_sfree[s]), sph);
         B.advance(sblk, nblk, kt);
-        if (B.bits != 16) {
-          const int hg = kt - B.kt0;
-          uint8_t* st = stage_ptr(s);
-          const int start = B.seg_off + 4 * B.bits * hg;
-          const int mslot = (B.grp_off + hg / 2) & 3;
-          const int sh = (start & 15) >> 2;  // uniform over the CTA
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const int r = r0 + 128 * h;
-            // the row's code bytes start at offset (start & 15) of a 16-byte
-            // aligned window; two conflict-free 16-byte reads cover them
-            const uint4* rp =
-                reinterpret_cast<const uint4*>(st + MT * kATile + kBTile + r * kCodeBox);
-            const uint4 c0 = rp[0], c1 = rp[1];
-            const uint32_t cw[8] = {c0.x, c0.y, c0.z, c0.w, c1.x, c1.y, c1.z, c1.w};
-            uint32_t w[8];
-            switch (sh) {
-              case 0:
-#pragma unroll
-                for (int k = 0; k < 8; ++k) w[k] = cw[k];
-                break;
-              case 1:
-#pragma unroll
-                for (int k = 0; k < 7; ++k) w[k] = cw[k + 1];
-                w[7] = 0;
-                break;
-              case 2:
-#pragma unroll
-                for (int k = 0; k < 6; ++k) w[k] = cw[k + 2];
-                w[6] = w[7] = 0;
-                break;
-              default:
-#pragma unroll
-                for (int k = 0; k < 5; ++k) w[k] = cw[k + 3];
-                w[5] = w[6] = w[7] = 0;
-                break;
+        const int tb = kt - B.kt0;
+        const uint32_t op = op_row + s * C::kA;
+        const uint32_t codes = code_row + sc * C::kCode;
+        auto dequant = [&](auto bits) {
+          constexpr int BITS = decltype(bits)::value;
+          const uint32_t meta =
+              lds32(meta_row + sc * C::kCode + ((B.grp_off + tb * C::BK / 64) & 3) * 4);
+          CodeWords<BITS, C::HALVES> cw;
+          cw.load(codes, (B.seg_off + (C::BK / 8) * BITS * tb) & 15);
+          const __half s16 = __ushort_as_half((uint16_t)(meta & 0xFFFFu));
+          const __half z16 = __ushort_as_half((uint16_t)(meta >> 16));
+          const __half2 ss = __halves2half2(s16, s16), zz = __halves2half2(z16, z16);
+#pragma unroll 1  // one copy of the code for both halves
+          for (int h = 0;;) {
+            uint32_t p[16];
+            dequant_half<BITS>(cw.w, zz, ss, magic, p);
+            if (h == 0 && !free) {
+              w = wait_ab(smem_u32(&bar_sfree[s]), sph, &s_abort);
+              if (w != kWaitOk) break;
             }
-            const uint32_t meta = reinterpret_cast<const uint32_t*>(
-                st + MT * kATile + kBTile + kCodes)[r * 4 + mslot];
-            dequant_row(B.bits, w, meta, st + MT * kATile, r);
-#ifdef POLYQ_DEBUG
-            dbg_row(st + MT * kATile, r, un * BN + r, P.N, sblk[B.bi], hg);
-#endif
+#pragma unroll
+            for (int c = 0; c < 4; ++c) sts128((op + h * kHalfTile) ^ (c << 4), p + 4 * c);
+            if (++h == C::HALVES) break;
+            if constexpr (BITS == 8) {
+              cw.load(codes + kBoxBytes, 0);
+            } else if constexpr (C::HALVES == 2) {
+#pragma unroll
+              for (int k = 0; k < BITS; ++k) cw.w[k] = cw.w[k + BITS];
+            }
           }
           fence_proxy_async_smem();
+        };
+        switch (B.bits) {
+          case 2: dequant(IntC<2>()); break;
+          case 3: dequant(IntC<3>()); break;
+          case 4: dequant(IntC<4>()); break;
+          case 8: dequant(IntC<8>()); break;
+          default:  // fp16 weights: copied straight into the weight slot
+            if (!free) w = wait_ab(smem_u32(&bar_sfree[s]), sph, &s_abort);
+            if (w != kWaitOk) break;
+            if (r == 0) {
+              const uint32_t bar = smem_u32(&bar_w16[grp]);
+              mbar_expect_tx(bar, C::kA);
+#pragma unroll
+              for (int h = 0; h < C::HALVES; ++h)
+                tma_load_2d(smem_u32(smem) + s * C::kA + h * kHalfTile, &P.tm_w16,
+                            B.seg_off / 2 + C::BK * tb + kSlots * h,
+                            un * kRowsN + (int)rank * kRowsCta, bar);
+            }
+            w = wait_ab(smem_u32(&bar_w16[grp]), w16_ph, &s_abort);
+            w16_ph ^= 1u;
+            break;
+        }
+        if (w != kWaitOk) {
+          if (w == kWaitTimeout) fail(kStatusTimeoutEmpty);
+          break;
         }
 #ifdef POLYQ_DEBUG
-        else {
-          for (int h = 0; h < 2; ++h)
-            dbg_row(stage_ptr(s) + MT * kATile, r0 + 128 * h, un * BN + r0 + 128 * h, P.N,
-                    sblk[B.bi], kt - B.kt0);
-        }
+        for (int h = 0; h < C::HALVES; ++h)
+          dbg_row(smem + s * C::kA + h * kHalfTile, r, un * kRowsN + (int)rank * kRowsCta + r, P.N,
+                  sblk[B.bi], tb * C::HALVES + h);
 #endif
         __syncwarp();
-        if (lane == 0) mbar_arrive(smem_u32(&bar_bready[s]));
+        if (lane == 0) {
+          mbar_arrive_cluster(bready0 + 8 * s);
+          mbar_arrive(smem_u32(&bar_cfree[sc]));
+        }
+        sc += C::GROUPS;
+        if (sc >= C::CODES) {
+          sc = grp;
+          cph ^= 1u;
+        }
+        s += C::GROUPS;
+        if (s >= C::OPS) {
+          s = grp;
+          sph ^= 1u;
+        }
       }
-      if (s_abort) break;
-      // epilogue: lane i of a warp owns output column n = weight row
-      // 128 t + 32 q + i of the tile, and each TMEM column one token of the
-      // M pair, so every store of a warp writes 32 consecutive floats of one
-      // row of Y.  Tokens [128 half, +128) of the pair, 32 at a time.  The
-      // 2^e_m of the pre-pass (one token per lane, broadcast by shuffles) are
-      // loaded together, and both accumulators' TMEM loads of a chunk share
-      // one wait.  (The loads follow the accumulator's barrier, which orders
-      // them after the pre-pass even for a warp that took no stage.)
+      skip = kt - kt_hi;
+    }
+  } else {
+    // ---------------- epilogue ----------------
+    // Lane i of a warp owns output column n = weight row 128 rank + 32 q + i
+    // of the unit, and each TMEM column one token, so every store of a warp
+    // writes 32 consecutive floats of one row of Y, 32 tokens at a time.
+    const int q = warp & 3;  // TMEM lane quarter this warp may access
+    const int e0 = (warp - C::kEpiWarp) >> 2;  // chunks e0, e0 + EPI / 4, ...
+    constexpr int kChunks = C::T / 32 / (C::EPI / 4);
+    const uint32_t acce0 = mapa(smem_u32(&bar_acce[0]), 0);
+    const bool add = P.ksplit > 1 || P.streamk;  // Y was zeroed by the pre-pass
+    pdl_wait();  // the row scales come from the pre-pass
+    for (int uc = 0; !s_abort && pc.next(P, um, un, kt_lo, kt_hi); ++uc) {
+      const int buf = uc % C::NBUF;
+      // column 32 c of the unit's accumulators: with two, columns [0, TN / 2)
+      // of accumulator a are tokens a * TN / 2.. of CTA 0's R, the others of
+      // CTA 1's
+      auto token0 = [&](int c) {
+        const int a = 32 * c / C::TN, col = 32 * c % C::TN;
+        return um * C::T + (col / (C::TN / 2)) * C::R + a * (C::TN / 2) + col % (C::TN / 2);
+      };
+      float rs[kChunks];  // 2^e_m of the pre-pass, token token0 + lane of each chunk
+#pragma unroll
+      for (int i = 0; i < kChunks; ++i) {
+        const int m = token0(e0 + i * (C::EPI / 4)) + lane;
+        rs[i] = m < P.M ? __ldcg(P.rowscale + m) : 0.f;
+      }
       {
-        const int w = wait_ab(smem_u32(&bar_accf), uc & 1, &s_abort);
+        const int w = wait_sleep_ab(smem_u32(&bar_accf[buf]), (uc / C::NBUF) & 1, &s_abort);
         if (w != kWaitOk) {
           if (w == kWaitTimeout) fail(kStatusTimeoutFull);
           break;
         }
       }
       tc_fence_after();
-      const int mh = um * (MT * BM) + 128 * half;
-      float rs_l[4];
-#pragma unroll
-      for (int c4 = 0; c4 < 4; ++c4)
-        rs_l[c4] = mh + 32 * c4 + lane < P.M ? P.rowscale[mh + 32 * c4 + lane] : 0.f;
-      const bool add = P.ksplit > 1 || P.streamk;  // Y was zeroed by the pre-pass
-      const int n0 = un * BN + 32 * q + lane;       // + BM for the second accumulator
-#pragma unroll
-      for (int c4 = 0; c4 < 4; ++c4) {
-        const int m0 = mh + 32 * c4;
+      const int n = un * kRowsN + (int)rank * kRowsCta + 32 * q + lane;
+      const uint32_t t0 = tmem + ((uint32_t)(32 * q) << 16) + buf * (C::NACC * C::TN);
+#pragma unroll 1
+      for (int i = 0; i < kChunks; ++i) {
+        const int c = e0 + i * (C::EPI / 4);
+        const int m0 = token0(c);
         const int jn = min(32, P.M - m0);  // tokens of this chunk inside M
-        if (jn <= 0) break;
-        uint32_t v0[32], v1[32];
-        const uint32_t ta = tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(128 * half + 32 * c4);
-        tc_ld_32x32b_x32(ta, v0);
-        tc_ld_32x32b_x32(ta + BN, v1);
-        tc_wait_ld();
-        tc_regs_ready(v0);
-        tc_regs_ready(v1);
-        float* dst = P.y + (size_t)m0 * P.N + n0;
-        const bool ok0 = n0 < P.N, ok1 = n0 + BM < P.N;
+        if (jn > 0) {
+          uint32_t v[32];
+          tc_ld_32x32b_x32(t0 + 32 * c, v);
+          float rs_l = rs[0];
 #pragma unroll
-        for (int j = 0; j < 32; ++j) {
-          const float rs = __shfl_sync(0xffffffffu, rs_l[c4], j);
-          if (j < jn) {
-            const float f0 = __uint_as_float(v0[j]) * rs, f1 = __uint_as_float(v1[j]) * rs;
-            if (add) {
-              if (ok0) red_add_f32(dst, f0);
-              if (ok1) red_add_f32(dst + BM, f1);
-            } else {
-              if (ok0) dst[0] = f0;
-              if (ok1) dst[BM] = f1;
-            }
-          }
-          dst += P.N;
+          for (int k = 1; k < kChunks; ++k) rs_l = k == i ? rs[k] : rs_l;
+          tc_wait_ld();
+          tc_regs_ready(v);
+          float* dst = P.y + (size_t)m0 * P.N + n;
+          if (add) store_chunk<true>(dst, P.N, n < P.N, jn, v, rs_l);
+          else store_chunk<false>(dst, P.N, n < P.N, jn, v, rs_l);
+          __syncwarp();
         }
       }
       tc_fence_before();
       __syncwarp();
-      if (lane == 0) mbar_arrive(smem_u32(&bar_acce));
+      if (lane == 0) mbar_arrive_cluster(acce0 + 8 * buf);
     }
   }
 
-  // all roles done (or aborted): wait for the last tensor-core work, free TMEM
+  // all roles of both CTAs done (or aborted): free TMEM; neither CTA exits
+  // while its peer may still reach its shared memory
   __syncthreads();
-  if (warp == 1) {
-    if (lane == 0) {
-      // the last commit of this CTA went to bar_accf; its completion means all
-      // MMAs have finished reading shared memory and writing TMEM
-      int uc = 0;
-      Pieces pc;
-      pc.init(P);
-      int um, un, kt_lo, kt_hi;
-      while (pc.next(P, um, un, kt_lo, kt_hi)) ++uc;
-      if (uc > 0) mbar_wait(smem_u32(&bar_accf), (uc - 1) & 1);
-    }
-    __syncwarp();
+  cluster_sync();
+  if (role == kRoleMma) {
     tc_fence_after();
-    tmem_dealloc(tmem, kTmemCols);
+    tmem_dealloc2(tmem, kTmemCols);
   }
+  cluster_sync();
 }
 
 // ---------------------------------------------------------------------------
 // host side
 // ---------------------------------------------------------------------------
-int k_tiles(const polyq_dev_layer* L, GmBlock* blk) {
+int k_tiles(const polyq_dev_layer* L, int bk, GmBlock* blk) {
   int kt = 0;
   for (int i = 0; i < L->n_blocks; ++i) {
     const polyq_block& b = L->blocks[i];
@@ -890,22 +1425,204 @@ int k_tiles(const polyq_dev_layer* L, GmBlock* blk) {
     g.grp_off = b.grp_off;
     g.n_grp = b.n_grp;
     g.kt0 = kt;
-    g.n_kt = (b.n_ch + BK - 1) / BK;  // half groups
+    g.n_kt = (b.n_ch + bk - 1) / bk;
     kt += g.n_kt;
     if (blk) blk[i] = g;
   }
   return kt;
 }
 
-// Workspace: Xg (16 KB blocks, M rounded up to a pair of M tiles) fp16, the
-// row scales [M] fp32, then 256 bytes holding the status word; each part
-// starts on a 256-byte boundary.
+// Workspace: Xg fp16 (M rounded up to a token tile of any kernel that may
+// take it, K slots padded to 64 per block), the row scales [M] fp32, then 256
+// bytes holding the status word; each part starts on a 256-byte boundary.
+// Grows with M, so that a workspace made for M serves fewer rows too.
 size_t gemm_xg_bytes(const polyq_dev_layer* L, int64_t M) {
-  const size_t Mp = (size_t)((M + MT * BM - 1) / (MT * BM)) * (MT * BM);
-  return (Mp * k_tiles(L, nullptr) * BK * 2 + 255) / 256 * 256;
+  size_t Mp = 32;
+  while (Mp < 512 && Mp < (size_t)M) Mp *= 2;
+  if (Mp == 512) Mp = ((size_t)M + 511) / 512 * 512;
+  return Mp * k_tiles(L, 64, nullptr) * 64 * 2;
 }
 size_t gemm_workspace(const polyq_dev_layer* L, int64_t M) {
   return gemm_xg_bytes(L, M) + ((size_t)M * 4 + 255) / 256 * 256 + 256;
+}
+
+// CTA pairs resident at once for a kernel (per device, queried once), after
+// its shared-memory limit has been raised.
+constexpr int kMaxDevices = 64;
+template <class C>
+int resident_pairs(int dev, int* pairs) {
+  static std::atomic<int> cached[kMaxDevices];
+  int n = cached[dev].load(std::memory_order_acquire);
+  if (n == 0) {
+    cudaError_t e = cudaFuncSetAttribute(gemm_main<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)C::kSmem);
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = 2;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2);
+    cfg.blockDim = dim3(C::kThreads);
+    cfg.dynamicSmemBytes = C::kSmem;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    if (e == cudaSuccess) e = cudaOccupancyMaxActiveClusters(&n, gemm_main<C>, &cfg);
+    if (e != cudaSuccess || n < 1)
+      return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: %d CTA pairs fit: %s", n,
+                             cudaGetErrorString(e));
+    cached[dev].store(n, std::memory_order_release);
+  }
+  *pairs = n;
+  return POLYQ_OK;
+}
+
+// Modelled time (s) of a kernel on this problem and the K split it would use.
+// A unit's K tile takes `stage` seconds of a pair; a piece costs `piece` more
+// (pipeline fill, draining the accumulator) and splitting adds the zeroing of
+// Y.  Uniform split into k ranges: whole waves of units.  Stream-K: one
+// pair's equal share plus the pieces it touches.  Near ties go to the simpler
+// choice.
+struct Split {
+  double t;
+  int ksplit, streamk;
+};
+Split plan_split(int64_t M, int64_t N, int T, int KT, int bk, int pairs, double stage,
+                 double piece) {
+  const long long mn = ((M + T - 1) / T) * ((N + kRowsN - 1) / kRowsN);
+  const double zero = (double)M * N * 4.0 / kZeroBytesPerS;
+  Split s = {1e300, 1, 0};
+  const int kmax = std::max(1, std::min(64, KT * bk / 512));
+  for (int k = 1; k <= kmax; ++k) {
+    const long long waves = (mn * k + pairs - 1) / pairs;
+    const double t = waves * ((double)KT / k * stage + piece) + (k > 1 ? zero : 0.0);
+    if (t < 0.98 * s.t) s = {t, k, 0};
+  }
+  const double share = std::ceil((double)mn * KT / pairs);
+  const double t_sk = share * stage + piece * (std::ceil(share / KT) + 1.0) + zero;
+  if (mn * KT >= pairs && mn * KT < (1ll << 31) && t_sk < 0.98 * s.t) s = {t_sk, 1, 1};
+  return s;
+}
+
+template <class C>
+int launch_main(GmParams& P, const Split& sp, int pairs, cudaStream_t st) {
+  cudaLaunchAttribute at[2];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  at[1].id = cudaLaunchAttributeClusterDimension;
+  at[1].val.clusterDim.x = 2;
+  at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 2;
+  cfg.gridDim = dim3((unsigned)(2 * (sp.streamk ? pairs : std::min(P.units, pairs))));
+  cfg.blockDim = dim3(C::kThreads);
+  cfg.dynamicSmemBytes = C::kSmem;
+  cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_main<C>, P, gv::kMagic);
+  if (e != cudaSuccess)
+    return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: launch: %s", cudaGetErrorString(e));
+  return POLYQ_OK;
+}
+
+int launch_prep(GmParams& P, int sms, int dev, cudaStream_t st) {
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.stream = st;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  cfg.blockDim = dim3(kPrepThreads);
+  const int Kp = P.KT * P.bk;
+  const int Mp = P.units_m << (P.r_log2 + 1);
+  static std::atomic<bool> attr_done[kMaxDevices];
+  if (!attr_done[dev].load(std::memory_order_acquire)) {
+    cudaError_t ea = cudaFuncSetAttribute(gemm_prep, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                          kPrepMaxSmem);
+    if (ea == cudaSuccess)
+      ea = cudaFuncSetAttribute(gemm_prep_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                kSmallMaxK * 2);
+    if (ea != cudaSuccess)
+      return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep smem attribute: %s",
+                             cudaGetErrorString(ea));
+    attr_done[dev].store(true, std::memory_order_release);
+  }
+  cudaError_t e;
+  if (P.M <= 512 && P.K <= kSmallMaxK) {
+    // about four CTAs per SM, each with one to kSmallQuads quads per thread
+    const int quads = Kp / 4;
+    const int lo = (quads + kSmallQuads * kPrepThreads - 1) / (kSmallQuads * kPrepThreads);
+    const int hi = (quads + kPrepThreads - 1) / kPrepThreads;
+    P.prep_seg = std::max(lo, std::min(hi, 4 * sms / Mp));
+    P.prep_rows = Mp * P.prep_seg;
+    int n_zero = 0;
+    if (P.ksplit > 1 || P.streamk)  // eight float4 per thread, at most two CTAs per SM
+      n_zero = (int)std::min<long long>(2 * sms, ((long long)P.M * P.N + 32 * kPrepThreads - 1) /
+                                                     (32 * kPrepThreads));
+    cfg.gridDim = dim3((unsigned)(P.prep_rows + n_zero));
+    cfg.dynamicSmemBytes = ((size_t)P.K * 2 + 15) / 16 * 16;
+    e = cudaLaunchKernelEx(&cfg, gemm_prep_small, P);
+  } else {
+    const size_t smem = prep_smem_bytes(P.K, Kp, P.xscale != nullptr);
+    P.prep_staged = smem > 0;
+    // as many CTAs as are resident at once (registers and shared memory),
+    // each taking rows m = b, b + grid, ...
+    int per_sm = 0;
+    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemm_prep, kPrepThreads, smem);
+    if (e != cudaSuccess || per_sm < 1)
+      return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep occupancy: %s",
+                             cudaGetErrorString(e));
+    per_sm = std::min(8, per_sm);
+    cfg.gridDim = dim3((unsigned)std::min<long long>(P.M, (long long)sms * per_sm));
+    cfg.dynamicSmemBytes = smem;
+    e = cudaLaunchKernelEx(&cfg, gemm_prep, P);
+  }
+  if (e != cudaSuccess)
+    return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep launch: %s", cudaGetErrorString(e));
+  return POLYQ_OK;
+}
+
+// One kernel's candidacy: its modelled time and split.
+struct Choice {
+  int cfg, pairs;
+  Split split;
+};
+template <class C>
+int consider(const polyq_dev_layer* L, int64_t M, int dev, int id, double stage, double piece,
+             Choice* best) {
+  int pairs = 0;
+  int rc = resident_pairs<C>(dev, &pairs);
+  if (rc) return rc;
+  const Split s = plan_split(M, L->N, C::T, k_tiles(L, C::BK, nullptr), C::BK, pairs, stage, piece);
+  if (best->cfg < 0 || s.t < 0.98 * best->split.t) *best = {id, pairs, s};
+  return POLYQ_OK;
+}
+
+template <class C>
+int run(const polyq_dev_layer* L, GmParams& P, const Choice& ch, int sms, int dev,
+        cudaStream_t st) {
+  P.bk = C::BK;
+  P.KT = k_tiles(L, C::BK, P.blk);
+  P.r_log2 = 0;
+  while ((1 << P.r_log2) < C::R) ++P.r_log2;
+  P.units_m = (P.M + C::T - 1) / C::T;
+  P.units_n = (P.N + kRowsN - 1) / kRowsN;
+  P.ksplit = ch.split.ksplit;
+  P.streamk = ch.split.streamk;
+  P.units = P.units_m * P.units_n * P.ksplit;
+  if (P.streamk) {
+    const int total = P.units * P.KT;  // below 2^31, see plan_split
+    P.sk_share = total / ch.pairs;
+    P.sk_extra = total % ch.pairs;
+  }
+  int rc = launch_prep(P, sms, dev, st);
+  if (rc) return rc;
+  // The main kernel may launch while the pre-pass runs (programmatic
+  // dependent launch): its set-up overlaps the pre-pass, and its producer
+  // waits for the pre-pass before the first load of Xg.  It allocates all of
+  // an SM's tensor memory, which is safe because two of its CTAs (more than
+  // half of an SM's shared memory each) never share an SM.
+  return launch_main<C>(P, ch.split, ch.pairs, st);
 }
 
 }  // namespace
@@ -965,14 +1682,10 @@ extern "C" int polyq_linear_gemm(const polyq_dev_layer* L, const void* X, int64_
 
   GmParams P;
   memset(&P, 0, sizeof P);
-  const int KT = k_tiles(L, P.blk);
   P.n_blocks = L->n_blocks;
   P.M = (int)M;
   P.N = (int)L->N;
   P.K = (int)L->K;
-  P.KT = KT;
-  P.units_m = (int)((M + MT * BM - 1) / (MT * BM));
-  P.units_n = (int)((L->N + BN - 1) / BN);
   P.x = (const __nv_bfloat16*)X;
   P.gather = L->gather;
   P.xscale = L->xscale;
@@ -981,112 +1694,44 @@ extern "C" int polyq_linear_gemm(const polyq_dev_layer* L, const void* X, int64_
   P.y = Y;
   P.status = (int*)((uint8_t*)workspace + need - 256);
   rc = polyq_tensor_map_2d(&P.tm_codes, L->packed, 1, (uint64_t)L->row_stride, (uint64_t)L->N,
-                           (uint64_t)L->row_stride, kCodeBox, BN);
+                           (uint64_t)L->row_stride, kCodeBox, kRowsCta);
   if (rc) return rc;
   rc = polyq_tensor_map_2d(&P.tm_w16, L->packed, 2, (uint64_t)L->row_stride / 2, (uint64_t)L->N,
-                           (uint64_t)L->row_stride, BK, BN, 64);
+                           (uint64_t)L->row_stride, kSlots, kRowsCta, 64);
   if (rc) return rc;
   if (L->n_groups > 0) {
     rc = polyq_tensor_map_2d(&P.tm_meta, L->meta, 4, (uint64_t)L->meta_stride, (uint64_t)L->N,
-                             (uint64_t)L->meta_stride * 4, 4, BN);
+                             (uint64_t)L->meta_stride * 4, 4, kRowsCta);
     if (rc) return rc;
     P.has_meta = 1;
   }
 
   cudaStream_t st = (cudaStream_t)stream;
-  int sms = 0;
+  int sms = 0, dev = 0;
   rc = polyq_sm_count(&sms);
   if (rc) return rc;
-  // Split K when the (M, N) tiles fill the SMs poorly.  The modelled time, in
-  // K-tile stages of one CTA, is for a uniform split into k ranges: whole
-  // waves of units times (K tiles per unit + a per-piece cost for filling the
-  // pipeline and adding the tile into Y); for stream-K: the K tiles of one
-  // CTA's equal share plus the per-piece cost of the (at most three) pieces
-  // it touches.  Both add the zeroing of Y when they split.  Each uniform
-  // split keeps at least 16 K tiles; near ties go to the simpler choice.
-  {
-    const int mn = P.units_m * P.units_n;
-    const bool can_split = (P.N % 4) == 0;  // zeroing writes float4
-    const double zero = (double)M * P.N * 4.0 / kZeroBytesPerS / kStageSeconds;
-    int ks = 1;
-    double best = 1e300;
-    const int kmax = can_split ? std::max(1, std::min(64, KT / 16)) : 1;
-    for (int k = 1; k <= kmax; ++k) {
-      const long long waves = ((long long)mn * k + sms - 1) / sms;
-      const double t = (double)waves * ((double)KT / k + kUnitCostTiles) + (k > 1 ? zero : 0.0);
-      if (t < 0.98 * best) {
-        best = t;
-        ks = k;
-      }
-    }
-    const double share = std::ceil((double)mn * KT / sms);
-    const double t_sk = share + kUnitCostTiles * (std::ceil(share / KT) + 1.0) + zero;
-    if (can_split && (long long)mn * KT >= sms && t_sk < 0.98 * best) {
-      P.streamk = 1;
-      P.ksplit = 1;
-      P.units = mn;
-    } else {
-      P.ksplit = ks;
-      P.units = mn * ks;
-    }
-  }
-  static bool attr_done[8] = {false};
-  int dev = 0;
   cudaGetDevice(&dev);
-  const size_t smem = (size_t)kStagesG * kStageG + 1024;
-  if (!attr_done[dev & 7]) {
-    cudaError_t e = cudaFuncSetAttribute(gemm_main, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         (int)smem);
-    if (e != cudaSuccess)
-      return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: smem attribute: %s",
-                             cudaGetErrorString(e));
-    attr_done[dev & 7] = true;
+  if (dev < 0 || dev >= kMaxDevices)
+    return polyq_set_error(POLYQ_EUNSUPPORTED, "polyq_linear_gemm: device %d >= %d", dev,
+                           kMaxDevices);
+  // The smallest token tile that holds M (a wider one would multiply padding:
+  // 13824 x 5120 takes 26 / 30 / 38 us at M = 16 / 96 / 256, and took 53 us at
+  // each with 256), or for more than 256 tokens the cheaper of 256 and 512 by
+  // the model (stage and piece times measured).
+  Choice ch = {-1, 0, {}};
+  if (M <= 32) rc = consider<Cfg32>(L, M, dev, 32, kStage32, kPiece32, &ch);
+  else if (M <= 64) rc = consider<Cfg64>(L, M, dev, 64, kStage64, kPiece64, &ch);
+  else if (M <= 128) rc = consider<Cfg128>(L, M, dev, 128, kStage128, kPiece128, &ch);
+  else {
+    rc = consider<Cfg256>(L, M, dev, 256, kStage256, kPiece256, &ch);
+    if (!rc && M > 256) rc = consider<Cfg512>(L, M, dev, 512, kStage512, kPiece512, &ch);
   }
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at[0].val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg = {};
-  cfg.stream = st;
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  const size_t prep_smem = prep_smem_bytes(P.K, KT * BK, P.xscale != nullptr);
-  P.prep_staged = prep_smem > 0;
-  static bool prep_attr_done[8] = {false};
-  if (!prep_attr_done[dev & 7]) {
-    cudaError_t ea = cudaFuncSetAttribute(gemm_prep, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          kPrepMaxSmem);
-    if (ea != cudaSuccess)
-      return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep smem attribute: %s",
-                             cudaGetErrorString(ea));
-    prep_attr_done[dev & 7] = true;
+  if (rc) return rc;
+  switch (ch.cfg) {
+    case 32: return run<Cfg32>(L, P, ch, sms, dev, st);
+    case 64: return run<Cfg64>(L, P, ch, sms, dev, st);
+    case 128: return run<Cfg128>(L, P, ch, sms, dev, st);
+    case 256: return run<Cfg256>(L, P, ch, sms, dev, st);
+    default: return run<Cfg512>(L, P, ch, sms, dev, st);
   }
-  {
-    // as many CTAs as are resident at once (registers and shared memory),
-    // each taking rows m = b, b + grid, ...
-    int per_sm = 0;
-    cudaError_t eo =
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemm_prep, kPrepThreads, prep_smem);
-    if (eo != cudaSuccess || per_sm < 1)
-      return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep occupancy: %s",
-                             cudaGetErrorString(eo));
-    per_sm = std::min(8, per_sm);
-    cfg.gridDim = dim3((unsigned)std::min<long long>(M, (long long)sms * per_sm));
-  }
-  cfg.blockDim = dim3(kPrepThreads);
-  cfg.dynamicSmemBytes = prep_smem;
-  cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_prep, P);
-  if (e != cudaSuccess)
-    return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep launch: %s", cudaGetErrorString(e));
-  // The main kernel may launch while the pre-pass runs (programmatic
-  // dependent launch): its set-up overlaps the pre-pass, and its producer
-  // waits for the pre-pass before the first load of Xg.  It allocates all of
-  // an SM's tensor memory, which is safe because two of its CTAs (197 KB of
-  // shared memory each) never share an SM.
-  cfg.gridDim = dim3((unsigned)(P.streamk ? sms : std::min(P.units, sms)));
-  cfg.blockDim = dim3(kThreadsG);
-  cfg.dynamicSmemBytes = smem;
-  e = cudaLaunchKernelEx(&cfg, gemm_main, P);
-  if (e != cudaSuccess)
-    return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: launch: %s", cudaGetErrorString(e));
-  return POLYQ_OK;
 }

@@ -122,3 +122,27 @@ def test_gemm_rows_too_wide_to_stage(polyq_lib):
     Y = polyq_lib.linear_gemm(dev, _x_dev(Xb))
     torch.cuda.synchronize()
     check_tolerance(Y.cpu().numpy(), O.linear(ref, X), X, K)
+
+
+@pytest.mark.parametrize("M", [5, 16, 17, 32, 33, 64, 65, 128, 129, 256, 257, 512, 513, 1025])
+@pytest.mark.parametrize("N,K,seed", [
+    (258, 3001, 64),   # one and a bit tiles of weight rows, ragged K, all five widths
+    (129, 70, 65),     # fewer K tiles than pipeline stages
+])
+def test_gemm_token_tile_edges(polyq_lib, M, N, K, seed):
+    """Each number of tokens at the edge of a kernel's token tile (32 to 512),
+    on a workspace that a larger call left dirty."""
+    W, a = synth.layer_weights(N, K, seed)
+    bits = synth.random_codes_layer_bits(K, seed)
+    Xb, X = synth.activations(a, M, seed)
+    host = polyq_lib.HostLayer.pack(W, a, 3.0, forced_bits=bits)
+    dev = polyq_lib.DeviceLayer(host, "cuda")
+    need = polyq_lib.gemm_workspace_bytes(dev, M)
+    assert need <= polyq_lib.gemm_workspace_bytes(dev, M + 1)  # a workspace serves fewer rows too
+    ws = torch.full((need,), 255, dtype=torch.uint8, device="cuda")
+    Y = torch.full((M, N), float("nan"), device="cuda")
+    polyq_lib.linear_gemm(dev, _x_dev(Xb), Y=Y, workspace=ws)
+    torch.cuda.synchronize()
+    assert polyq_lib.workspace_status(ws[-256:]) == 0
+    ref = O.pack_layer(W, a, 3.0, bits=bits)
+    check_tolerance(Y.cpu().numpy(), O.linear(ref, X), X, K)
