@@ -6,7 +6,7 @@
 // The contraction runs over K tiles of 32 or 64 (half or all of a quantisation
 // group); every tile lies inside one bit block (Section 4.2) and one group, so
 // each weight row of a tile has one (scale, zero).
-//  1. A pre-pass (gemm_prep, or gemm_prep_small for a few rows) gathers X
+//  1. A pre-pass (gemm_prep_rows, or gemm_prep_small for a few rows) gathers X
 //     through `gather` into a clustered fp16 matrix Xg (workspace),
 //     zero-padded at block ends, with the K order inside each tile permuted
 //     the same way the dequantiser emits codes.  Xg is stored as the
@@ -207,7 +207,6 @@ struct GmParams {
   int streamk;  // 1: each pair takes an equal contiguous range of (unit, K tile) pairs:
   int sk_share, sk_extra;  // sk_share of them, the first sk_extra pairs one more
   int has_meta;
-  int prep_staged;  // 1: the pre-pass stages each row of X in shared memory
   int prep_seg;     // gemm_prep_small: CTAs per row
   int prep_rows;    // gemm_prep_small: CTAs that gather rows (the others zero Y)
   const __nv_bfloat16* x;
@@ -450,7 +449,7 @@ __host__ __device__ inline int slot_code(int bits, int s) {
 // Shared copy of the block table and of slot_code for every width.
 struct PrepTables {
   GmBlock blk[POLYQ_MAX_BLOCKS];
-  uint8_t code[5][kSlots];
+  alignas(8) uint8_t code[5][kSlots];
 };
 __device__ __forceinline__ int width_index(int bits) {
   return bits <= 4 ? bits - 2 : (bits == 8 ? 3 : 4);
@@ -483,9 +482,11 @@ constexpr int kRowExp = 14;       // a row's largest magnitude becomes [2^14, 2^
 constexpr int kRowExpMin = -126;  // 2^e stays a normal float
 constexpr int kPrepThreads = 256;
 constexpr int kPrepMaxSmem = 200 * 1024;
-constexpr int kRowVec = 8;  // 16-byte pieces of a row a thread holds (rows up to 16384 wide)
 constexpr int kSmallQuads = 4;                // 4-slot quads per thread of gemm_prep_small
 constexpr int kSmallMaxK = 32768;             // widest row it stages
+constexpr int kSmallMaxM = 128;               // most rows it is used for (K = 13824: 34 us for the
+                                              // call at M = 128, 37 with gemm_prep_rows; K = 5120,
+                                              // M = 256: 40 and 37)
 
 // Element offset of Xg(m, k) in the blocked layout: block (m / R, k / 32) of
 // R rows x 32 fp16, row m % R at 64 bytes each, its 16-byte chunks in the
@@ -522,194 +523,263 @@ __device__ __forceinline__ void zero_y(const GmParams& P, int cta, int n_cta) {
 __device__ __forceinline__ int row_exp(uint32_t mx) {
   return mx ? max((int)(mx >> 23) - 127 - kRowExp, kRowExpMin) : 0;
 }
-__device__ __forceinline__ uint32_t bf16x8_max(const uint4& v, uint32_t mx) {
-  const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-  for (int q = 0; q < 4; ++q) mx = max(mx, max(w[q] & 0x7FFFu, (w[q] >> 16) & 0x7FFFu));
-  return mx;
+// Largest magnitudes of the low and of the high halves of eight bf16 (their bit
+// patterns without the sign order as integers), and the larger of the two.
+__device__ __forceinline__ uint32_t bf16x8_max(const uint4& v, uint32_t mx2) {
+  constexpr uint32_t kAbs = 0x7FFF7FFFu;
+  return __vmaxu2(__vmaxu2(__vmaxu2(mx2, v.x & kAbs), v.y & kAbs),
+                  __vmaxu2(v.z & kAbs, v.w & kAbs));
+}
+__device__ __forceinline__ uint32_t max_halves(uint32_t mx2) {
+  return max(mx2 & 0xFFFFu, mx2 >> 16);
 }
 
-// Shared memory of the staged pre-pass: the slot -> source map (int32 [Kp]),
-// the slot factors (fp32 [Kp], scaled layers only) and one row of X (bf16
-// [K]); 0 when it does not fit.
-size_t prep_smem_bytes(int K, int Kp, bool xscale) {
-  const size_t b = (size_t)Kp * 4 * (xscale ? 2 : 1) + ((size_t)K * 2 + 15) / 16 * 16;
-  return b <= (size_t)kPrepMaxSmem ? b : 0;
+// Many rows, RW (1, 2 or 4) at a time: a CTA stages RW rows of X in shared
+// memory interleaved, one word of RW bf16 values per channel, and gathers from
+// there, so that one index read and one word read serve RW values.  Bound by
+// shared-memory wavefronts (62-75% of the pipe) and issue (60%); one row at a
+// time, with an index, a value, a test and 64-bit address arithmetic per
+// element, it was bound by 25 to 34 instructions an element.  K = 5120, M =
+// 8192: 49 -> 37 us; K = 13824, M = 2048: 48 -> 31 us (cold cache).  16-byte pieces of RW words lie in planes, so that the staging stores of a
+// warp are contiguous; the slot map holds positions in that layout and is
+// built, from static layer data, before the wait for the previous kernel.
+constexpr int kRowsThreads = 512;
+constexpr int kRowsMaxK = 65520;  // staged positions and the zero word fit 16 bits
+
+// Words (of RW bf16) per 16-byte piece.
+template <int RW>
+__host__ __device__ constexpr int piece_words() {
+  return 8 / RW;
+}
+// Position of channel k among the staged words: the 8 channels of a 16-byte
+// piece of X fill RW staged pieces, one in each of RW planes of n8.  The words
+// after them, from 8 n8 on, are zero: the source of slots past a block's end.
+template <int RW>
+__device__ __forceinline__ uint32_t staged_pos(int k, int n8) {
+  constexpr int PW = piece_words<RW>();
+  return (uint32_t)(((k & 7) / PW * n8 + (k >> 3)) * PW + (k & (PW - 1)));
+}
+template <int RW>
+__host__ __device__ constexpr size_t rows_smem(int K, int Kp, bool xscale) {
+  return (size_t)((K + 7) / 8) * 16 * RW + 16 + (size_t)Kp * 2 + (xscale ? (size_t)Kp * 4 : 0);
 }
 
-// Many rows: each CTA first builds, in shared memory, the map from a clustered
-// slot to the source channel it reads (and its activation factor); then, one
-// row at a time, it copies the row of X into shared memory with 16-byte loads
-// (finding the row's largest magnitude on the way) and gathers from there.
-// Rows up to 16384 wide are held in registers, the next row's loads in flight
-// while the current row is gathered.  Global reads and writes are so coalesced
-// whatever the permutation.  Layers too wide for shared memory (see
-// prep_smem_bytes) gather from global memory instead.  Y is zeroed when the K
-// range is split over CTAs.
-__global__ void __launch_bounds__(kPrepThreads) gemm_prep(const __grid_constant__ GmParams P) {
+template <int RW, bool XS>  // XS: scaled layer
+__global__ void __launch_bounds__(kRowsThreads) gemm_prep_rows(const __grid_constant__ GmParams P) {
   extern __shared__ __align__(16) uint8_t psm[];
+  constexpr int PW = piece_words<RW>();
+  pdl_trigger();
+  __shared__ PrepTables S;
+  __shared__ uint32_t s_max[2][RW];
+  load_tables(P, &S);
+  if (threadIdx.x < 2 * RW) s_max[threadIdx.x / RW][threadIdx.x % RW] = 0;
+  __syncthreads();
+  const int Kp = P.KT * P.bk, ks = Kp / kSlots, n8 = (P.K + 7) / 8;
+  uint4* s_x = reinterpret_cast<uint4*>(psm);
+  uint16_t* s_map = reinterpret_cast<uint16_t*>(psm + (size_t)n8 * 16 * RW + 16);
+  float* s_fac = reinterpret_cast<float*>(s_map + Kp);
+  {
+    // a thread takes 8 consecutive slots (of one block and half group), so
+    // that finding them costs 11 instructions a slot and not 60
+    for (int k = 8 * threadIdx.x; k < Kp; k += 8 * kRowsThreads) {
+      const GmBlock& B = S.blk[find_kblock(S.blk, P.n_blocks, P.bk == 64 ? k >> 6 : k >> 5)];
+      const int o = k - B.kt0 * P.bk;
+      const uint2 c8 = *reinterpret_cast<const uint2*>(&S.code[width_index(B.bits)][o & (kSlots - 1)]);
+      const int base = o & ~(kSlots - 1);
+      int src[8];
+      float fac[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const int w = base + (int)(((u < 4 ? c8.x : c8.y) >> (8 * (u & 3))) & 0xFFu);
+        const int p = B.pos0 + w;
+        const bool in = w < B.n_ch;
+        src[u] = !in ? -1 : (P.gather ? __ldg(P.gather + p) : p);
+        fac[u] = (XS && in) ? __ldg(P.xscale + p) : 0.f;
+      }
+      uint32_t m[4];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) {
+        const uint32_t v = src[u] < 0 ? 8u * n8 : staged_pos<RW>(src[u], n8);
+        m[u >> 1] = (u & 1) ? m[u >> 1] | (v << 16) : v;
+        if (XS) s_fac[k + u] = fac[u];
+      }
+      *reinterpret_cast<uint4*>(s_map + k) = make_uint4(m[0], m[1], m[2], m[3]);
+    }
+    if (threadIdx.x == 0) s_x[n8 * RW] = make_uint4(0u, 0u, 0u, 0u);
+  }
+  pdl_wait();  // X comes from the previous kernel; Y and the workspace may still be in use
+  if (blockIdx.x == 0 && threadIdx.x == 0) *P.status = 0;
+  if (P.ksplit > 1 || P.streamk) zero_y(P, blockIdx.x, gridDim.x);
+  const int lane = threadIdx.x & 31;
+  const int Mp = P.units_m << (P.r_log2 + 1);  // rows past M are zero: their MMA columns must be finite
+  const bool vec = (P.K & 7) == 0 && (reinterpret_cast<uintptr_t>(P.x) & 15) == 0;
+  const uint16_t* x = reinterpret_cast<const uint16_t*>(P.x);
+  int it = 0;
+  for (int m0 = blockIdx.x * RW; m0 < Mp; m0 += gridDim.x * RW, it ^= 1) {
+    uint32_t mx[RW];
+#pragma unroll
+    for (int r = 0; r < RW; ++r) mx[r] = 0;
+    constexpr int U = 4 / RW;  // pieces of a thread in flight: four 16-byte loads
+    for (int i0 = threadIdx.x; i0 < n8; i0 += U * kRowsThreads) {
+      uint4 v[U][RW];  // 8 channels of each row
+#pragma unroll
+      for (int u = 0; u < U; ++u)
+#pragma unroll
+        for (int r = 0; r < RW; ++r) {
+          const int i = i0 + u * kRowsThreads;
+          v[u][r] = make_uint4(0u, 0u, 0u, 0u);
+          if (m0 + r < P.M && i < n8) {
+            const size_t o = (size_t)(m0 + r) * P.K + 8 * i;
+            if (vec) {
+              v[u][r] = __ldcg(reinterpret_cast<const uint4*>(x + o));
+            } else {
+              uint32_t e[8];
+#pragma unroll
+              for (int c = 0; c < 8; ++c) e[c] = 8 * i + c < P.K ? (uint32_t)__ldcg(x + o + c) : 0u;
+              v[u][r] = make_uint4(e[0] | e[1] << 16, e[2] | e[3] << 16, e[4] | e[5] << 16,
+                                   e[6] | e[7] << 16);
+            }
+          }
+        }
+#pragma unroll
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * kRowsThreads;
+        if (i >= n8) break;
+        uint32_t w[RW][4];
+#pragma unroll
+        for (int r = 0; r < RW; ++r) {
+          mx[r] = bf16x8_max(v[u][r], mx[r]);
+          w[r][0] = v[u][r].x; w[r][1] = v[u][r].y; w[r][2] = v[u][r].z; w[r][3] = v[u][r].w;
+        }
+#pragma unroll
+        for (int j = 0; j < RW; ++j) {  // piece j: channels j * PW.., row-fastest
+          uint32_t o[4];
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            if (RW == 1) {
+              o[q] = w[0][q];
+            } else {
+              const int c = j * PW + (2 * q) / RW, r = (2 * q) % RW;
+              o[q] = __byte_perm(w[r][c >> 1], w[r + (RW > 1)][c >> 1], (c & 1) ? 0x7632 : 0x5410);
+            }
+          }
+          s_x[j * n8 + i] = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+      }
+    }
+    if (!XS) {  // without factors the largest |X| of the raw row, as the gather is a permutation
+#pragma unroll
+      for (int r = 0; r < RW; ++r) {
+        const uint32_t v = __reduce_max_sync(0xffffffffu, max_halves(mx[r])) << 16;  // bf16 -> fp32
+        if (lane == 0) atomicMax(&s_max[it][r], v);
+      }
+    }
+    __syncthreads();  // the rows (and, on the first pass, the map) are complete
+    // the RW values of a slot
+    auto values = [&](uint32_t pos, float (&v)[RW]) {
+      if constexpr (RW == 4) {
+        const uint2 a = reinterpret_cast<const uint2*>(s_x)[pos];
+        v[0] = bf16_lo(a.x); v[1] = bf16_hi(a.x); v[2] = bf16_lo(a.y); v[3] = bf16_hi(a.y);
+      } else if constexpr (RW == 2) {
+        const uint32_t a = reinterpret_cast<const uint32_t*>(s_x)[pos];
+        v[0] = bf16_lo(a); v[1] = bf16_hi(a);
+      } else {
+        v[0] = bf16_lo(reinterpret_cast<const uint16_t*>(s_x)[pos]);
+      }
+    };
+    if (XS) {
+#pragma unroll
+      for (int r = 0; r < RW; ++r) mx[r] = 0;
+      for (int k = threadIdx.x; k < Kp; k += kRowsThreads) {
+        float v[RW];
+        values(s_map[k], v);
+#pragma unroll
+        for (int r = 0; r < RW; ++r) mx[r] = max(mx[r], __float_as_uint(fabsf(v[r] * s_fac[k])));
+      }
+#pragma unroll
+      for (int r = 0; r < RW; ++r) {
+        const uint32_t v = __reduce_max_sync(0xffffffffu, mx[r]);
+        if (lane == 0) atomicMax(&s_max[it][r], v);
+      }
+      __syncthreads();
+    }
+    float inv[RW];
+#pragma unroll
+    for (int r = 0; r < RW; ++r) {
+      const int e = row_exp(s_max[it][r]);
+      if ((int)threadIdx.x == r && m0 + r < P.M) P.rowscale[m0 + r] = __int_as_float((127 + e) << 23);
+      inv[r] = __int_as_float((127 - e) << 23);
+    }
+    if (threadIdx.x < RW) s_max[it ^ 1][threadIdx.x] = 0;  // for the next pass
+    // rows m0.. of one block of R rows: addresses as in xg_off
+    __half* dst = P.xg + xg_off(m0, 0, ks, P.r_log2);  // its swizzle undone below
+    const int r0 = m0 & ((1 << P.r_log2) - 1);
+    dst -= ((r0 >> 1) & 3) << 3;
+    for (int i = threadIdx.x; i < Kp / 4; i += kRowsThreads) {
+      const uint2 mp = reinterpret_cast<const uint2*>(s_map)[i];
+      const uint32_t pos[4] = {mp.x & 0xFFFFu, mp.x >> 16, mp.y & 0xFFFFu, mp.y >> 16};
+      float v[4][RW];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) values(pos[e], v[e]);
+      if (XS) {
+        const float4 f = reinterpret_cast<const float4*>(s_fac)[i];
+        const float fac[4] = {f.x, f.y, f.z, f.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+#pragma unroll
+          for (int r = 0; r < RW; ++r) v[e][r] *= fac[e];
+      }
+      const uint32_t at = ((uint32_t)(i >> 3) << (P.r_log2 + 5)) + 4 * (i & 1);
+      const int c = (i >> 1) & 3;
+#pragma unroll
+      for (int r = 0; r < RW; ++r) {
+        const __half2 a = __floats2half2_rn(v[0][r] * inv[r], v[1][r] * inv[r]);
+        const __half2 b = __floats2half2_rn(v[2][r] * inv[r], v[3][r] * inv[r]);
+        *reinterpret_cast<uint2*>(dst + at + (r * kSlots + ((c ^ (((r0 + r) >> 1) & 3)) << 3))) =
+            make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+      }
+    }
+    __syncthreads();  // the staged rows are replaced by the next pass
+  }
+}
+
+// Layers too wide to stage a row (see rows_smem): gathered from global memory.
+__global__ void __launch_bounds__(kPrepThreads) gemm_prep_wide(const __grid_constant__ GmParams P) {
   pdl_trigger();
   __shared__ PrepTables S;
   __shared__ uint32_t s_wmax[kPrepThreads / 32];
   load_tables(P, &S);
   __syncthreads();
-  const int Kp = P.KT * P.bk, half = Kp / 2;  // slots and fp16 pairs per row of Xg
-  const int ks = Kp / kSlots;
-  const bool staged = P.prep_staged != 0;
-  int* s_src = reinterpret_cast<int*>(psm);
-  float* s_fac = reinterpret_cast<float*>(psm + (size_t)Kp * 4);
-  uint16_t* s_row = reinterpret_cast<uint16_t*>(psm + (size_t)Kp * 4 * (P.xscale ? 2 : 1));
-  if (staged) {
-    // static layer data, built before the wait for the previous kernel; a
-    // thread's loads of 16 slots are issued together
-    constexpr int U = 16;
-    for (int k0 = threadIdx.x; k0 < Kp; k0 += kPrepThreads * U) {
-      int pos[U], src[U];
-      float fac[U];
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int k = k0 + u * kPrepThreads;
-        pos[u] = k < Kp ? slot_pos(S, P.n_blocks, P.bk, k) : -1;
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        src[u] = pos[u] < 0 ? -1 : (P.gather ? __ldg(P.gather + pos[u]) : pos[u]);
-        fac[u] = (P.xscale && pos[u] >= 0) ? __ldg(P.xscale + pos[u]) : 0.f;
-      }
-#pragma unroll
-      for (int u = 0; u < U; ++u) {
-        const int k = k0 + u * kPrepThreads;
-        if (k < Kp) {
-          s_src[k] = src[u];
-          if (P.xscale) s_fac[k] = fac[u];
-        }
-      }
-    }
-  }
+  const int Kp = P.KT * P.bk, ks = Kp / kSlots;
   pdl_wait();  // X comes from the previous kernel; Y and the workspace may still be in use
   if (blockIdx.x == 0 && threadIdx.x == 0) *P.status = 0;
   if (P.ksplit > 1 || P.streamk) zero_y(P, blockIdx.x, gridDim.x);
-  // the value at clustered slot k of row m
-  auto value = [&](int m, int k) -> float {
-    int src;
-    float f = 1.f;
-    if (staged) {
-      src = s_src[k];
-      if (src < 0) return 0.f;
-      if (P.xscale) f = s_fac[k];
-    } else {
-      const int p = slot_pos(S, P.n_blocks, P.bk, k);
+  const int Mp = P.units_m << (P.r_log2 + 1);
+  for (int m = blockIdx.x; m < Mp; m += gridDim.x) {
+    auto value = [&](int k) -> float {  // at clustered slot k
+      const int p = m < P.M ? slot_pos(S, P.n_blocks, P.bk, k) : -1;
       if (p < 0) return 0.f;
-      src = P.gather ? __ldg(P.gather + p) : p;
-      if (P.xscale) f = __ldg(P.xscale + p);
-    }
-    const uint16_t b = staged ? s_row[src]
-                              : __ldcg(reinterpret_cast<const uint16_t*>(P.x) + (size_t)m * P.K + src);
-    return __uint_as_float((uint32_t)b << 16) * f;
-  };
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  // The rows of the last token tile past M are zero (their MMA columns are
-  // not stored, but they must be finite).
-  auto zero_pad_rows = [&]() {
-    const int Mp = P.units_m << (P.r_log2 + 1);
-    for (int m = P.M + blockIdx.x; m < Mp; m += gridDim.x)
-      for (int i = threadIdx.x; i < Kp / 4; i += kPrepThreads)
-        *reinterpret_cast<uint2*>(P.xg + xg_off(m, 4 * i, ks, P.r_log2)) = make_uint2(0u, 0u);
-  };
-  // Row scale of row m from its largest magnitude bits mx (fp32 bit pattern,
-  // per thread).  Returns 2^-e_m.
-  auto row_scale = [&](int m, uint32_t mx) -> float {
-    if (P.xscale) {
-      mx = 0;
-      for (int k = threadIdx.x; k < Kp; k += kPrepThreads)
-        mx = max(mx, __float_as_uint(fabsf(value(m, k))));
-    }
+      const int src = P.gather ? __ldg(P.gather + p) : p;
+      const uint16_t b = __ldcg(reinterpret_cast<const uint16_t*>(P.x) + (size_t)m * P.K + src);
+      const float v = __uint_as_float((uint32_t)b << 16);
+      return P.xscale ? v * __ldg(P.xscale + p) : v;
+    };
+    uint32_t mx = 0;
+    for (int k = threadIdx.x; k < Kp; k += kPrepThreads)
+      mx = max(mx, __float_as_uint(fabsf(value(k))));
     mx = __reduce_max_sync(0xffffffffu, mx);
-    if (lane == 0) s_wmax[warp] = mx;
+    if ((threadIdx.x & 31) == 0) s_wmax[threadIdx.x >> 5] = mx;
     __syncthreads();
 #pragma unroll
     for (int w = 0; w < kPrepThreads / 32; ++w) mx = max(mx, s_wmax[w]);
     const int e = row_exp(mx);
-    if (threadIdx.x == 0) P.rowscale[m] = __int_as_float((127 + e) << 23);
-    return __int_as_float((127 - e) << 23);
-  };
-  const int n8 = P.K / 8;  // 16-byte pieces of a row
-  const bool vec = staged && (P.K & 7) == 0 && (reinterpret_cast<uintptr_t>(P.x) & 15) == 0 &&
-                   n8 <= kRowVec * kPrepThreads;
-  if (vec) {
-    // A thread holds its pieces of a row in registers: the next row's loads
-    // are issued before the current row is gathered, so they are in flight
-    // meanwhile.
-    auto load_row = [&](int m, uint4 (&v)[kRowVec]) {
-      const uint4* row = reinterpret_cast<const uint4*>(P.x) + (size_t)m * n8;
-#pragma unroll
-      for (int u = 0; u < kRowVec; ++u) {
-        const int i = threadIdx.x + u * kPrepThreads;
-        v[u] = i < n8 ? __ldcg(row + i) : make_uint4(0u, 0u, 0u, 0u);
-      }
-    };
-    uint4 v[kRowVec];
-    if ((int)blockIdx.x < P.M) load_row(blockIdx.x, v);
-    for (int m = blockIdx.x; m < P.M; m += gridDim.x) {
-      uint32_t mx = 0;
-#pragma unroll
-      for (int u = 0; u < kRowVec; ++u) {
-        const int i = threadIdx.x + u * kPrepThreads;
-        if (i < n8) {
-          reinterpret_cast<uint4*>(s_row)[i] = v[u];
-          mx = bf16x8_max(v[u], mx);
-        }
-      }
-      mx <<= 16;  // bf16 magnitude bits -> fp32 bits
-      __syncthreads();  // the staged row (and, on the first row, the map) is complete
-      const float inv = row_scale(m, mx);
-      if (m + (int)gridDim.x < P.M) load_row(m + gridDim.x, v);
-      // four consecutive slots per thread and 8-byte store (with eight, the
-      // row reads of a warp's threads collide in shared-memory banks more)
-      for (int i = threadIdx.x; i < Kp / 4; i += kPrepThreads) {
-        uint32_t w[2];
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-          const __half2 h = __halves2half2(__float2half_rn(value(m, 4 * i + 2 * q) * inv),
-                                           __float2half_rn(value(m, 4 * i + 2 * q + 1) * inv));
-          w[q] = *reinterpret_cast<const uint32_t*>(&h);
-        }
-        *reinterpret_cast<uint2*>(P.xg + xg_off(m, 4 * i, ks, P.r_log2)) = make_uint2(w[0], w[1]);
-      }
-      __syncthreads();  // the row buffer and s_wmax are reused by the next row
-    }
-    zero_pad_rows();
-    return;
-  }
-  for (int m = blockIdx.x; m < P.M; m += gridDim.x) {
-    // largest magnitude of the row's values (bit patterns of non-negative
-    // floats order as integers); without activation factors that is the
-    // largest |X[m][k]| over the raw row, since the gather is a permutation
-    const uint16_t* row = reinterpret_cast<const uint16_t*>(P.x) + (size_t)m * P.K;
-    uint32_t mx = 0;
-    if ((P.K & 7) == 0 && (reinterpret_cast<uintptr_t>(row) & 15) == 0) {
-      for (int i = threadIdx.x; i < P.K / 8; i += kPrepThreads) {
-        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(row) + i);
-        if (staged) reinterpret_cast<uint4*>(s_row)[i] = v;
-        mx = bf16x8_max(v, mx);
-      }
-    } else {
-      for (int i = threadIdx.x; i < P.K; i += kPrepThreads) {
-        const uint16_t v = __ldcg(row + i);
-        if (staged) s_row[i] = v;
-        mx = max(mx, (uint32_t)(v & 0x7FFFu));
-      }
-    }
-    mx <<= 16;  // bf16 magnitude bits -> fp32 bits
-    __syncthreads();  // the staged row (and, on the first row, the map) is complete
-    const float inv = row_scale(m, mx);
-    for (int i = threadIdx.x; i < half; i += kPrepThreads)
+    if (threadIdx.x == 0 && m < P.M) P.rowscale[m] = __int_as_float((127 + e) << 23);
+    const float inv = __int_as_float((127 - e) << 23);
+    for (int i = threadIdx.x; i < Kp / 2; i += kPrepThreads)
       *reinterpret_cast<__half2*>(P.xg + xg_off(m, 2 * i, ks, P.r_log2)) =
-          __halves2half2(__float2half_rn(value(m, 2 * i) * inv),
-                         __float2half_rn(value(m, 2 * i + 1) * inv));
-    __syncthreads();  // the row buffer and s_wmax are reused by the next row
+          __floats2half2_rn(value(2 * i) * inv, value(2 * i + 1) * inv);
+    __syncthreads();  // s_wmax is reused by the next row
   }
-  zero_pad_rows();
 }
 
 // A few rows: prep_seg CTAs per row (of all rows of the token tiles), each
@@ -765,7 +835,7 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep_small(const __grid_con
         mx = max(mx, (uint32_t)(v & 0x7FFFu));
       }
     }
-    mx <<= 16;  // bf16 magnitude bits -> fp32 bits
+    mx = max_halves(mx) << 16;  // bf16 magnitude bits -> fp32 bits
     __syncthreads();
     if (P.xscale) {  // the largest |x * t| over the whole row
       mx = 0;
@@ -1524,6 +1594,35 @@ int launch_main(GmParams& P, const Split& sp, int pairs, cudaStream_t st) {
   return POLYQ_OK;
 }
 
+// The row-staging pre-pass with RW rows at a time: as many CTAs as are resident
+// at once.
+template <int RW, bool XS>
+int launch_prep_rows(const GmParams& P, int sms, int dev, cudaLaunchConfig_t cfg) {
+  static std::atomic<bool> attr_done[kMaxDevices];
+  if (!attr_done[dev].load(std::memory_order_acquire)) {
+    cudaError_t e = cudaFuncSetAttribute(gemm_prep_rows<RW, XS>,
+                                         cudaFuncAttributeMaxDynamicSharedMemorySize, kPrepMaxSmem);
+    if (e != cudaSuccess)
+      return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep smem attribute: %s",
+                             cudaGetErrorString(e));
+    attr_done[dev].store(true, std::memory_order_release);
+  }
+  cfg.blockDim = dim3(kRowsThreads);
+  cfg.dynamicSmemBytes = rows_smem<RW>(P.K, P.KT * P.bk, P.xscale != nullptr);
+  int per_sm = 0;
+  cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemm_prep_rows<RW, XS>,
+                                                                kRowsThreads, cfg.dynamicSmemBytes);
+  if (e != cudaSuccess || per_sm < 1)
+    return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep occupancy: %s",
+                           cudaGetErrorString(e));
+  const int Mp = P.units_m << (P.r_log2 + 1);
+  cfg.gridDim = dim3((unsigned)std::min<long long>(Mp / RW, (long long)sms * per_sm));
+  e = cudaLaunchKernelEx(&cfg, gemm_prep_rows<RW, XS>, P);
+  if (e != cudaSuccess)
+    return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep launch: %s", cudaGetErrorString(e));
+  return POLYQ_OK;
+}
+
 int launch_prep(GmParams& P, int sms, int dev, cudaStream_t st) {
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1532,23 +1631,19 @@ int launch_prep(GmParams& P, int sms, int dev, cudaStream_t st) {
   cfg.stream = st;
   cfg.attrs = at;
   cfg.numAttrs = 1;
-  cfg.blockDim = dim3(kPrepThreads);
   const int Kp = P.KT * P.bk;
   const int Mp = P.units_m << (P.r_log2 + 1);
-  static std::atomic<bool> attr_done[kMaxDevices];
-  if (!attr_done[dev].load(std::memory_order_acquire)) {
-    cudaError_t ea = cudaFuncSetAttribute(gemm_prep, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                          kPrepMaxSmem);
-    if (ea == cudaSuccess)
-      ea = cudaFuncSetAttribute(gemm_prep_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                kSmallMaxK * 2);
-    if (ea != cudaSuccess)
-      return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep smem attribute: %s",
-                             cudaGetErrorString(ea));
-    attr_done[dev].store(true, std::memory_order_release);
-  }
   cudaError_t e;
-  if (P.M <= 512 && P.K <= kSmallMaxK) {
+  if (P.M <= kSmallMaxM && P.K <= kSmallMaxK) {
+    static std::atomic<bool> attr_done[kMaxDevices];
+    if (!attr_done[dev].load(std::memory_order_acquire)) {
+      e = cudaFuncSetAttribute(gemm_prep_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               kSmallMaxK * 2);
+      if (e != cudaSuccess)
+        return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep smem attribute: %s",
+                               cudaGetErrorString(e));
+      attr_done[dev].store(true, std::memory_order_release);
+    }
     // about four CTAs per SM, each with one to kSmallQuads quads per thread
     const int quads = Kp / 4;
     const int lo = (quads + kSmallQuads * kPrepThreads - 1) / (kSmallQuads * kPrepThreads);
@@ -1560,23 +1655,33 @@ int launch_prep(GmParams& P, int sms, int dev, cudaStream_t st) {
       n_zero = (int)std::min<long long>(2 * sms, ((long long)P.M * P.N + 32 * kPrepThreads - 1) /
                                                      (32 * kPrepThreads));
     cfg.gridDim = dim3((unsigned)(P.prep_rows + n_zero));
+    cfg.blockDim = dim3(kPrepThreads);
     cfg.dynamicSmemBytes = ((size_t)P.K * 2 + 15) / 16 * 16;
     e = cudaLaunchKernelEx(&cfg, gemm_prep_small, P);
-  } else {
-    const size_t smem = prep_smem_bytes(P.K, Kp, P.xscale != nullptr);
-    P.prep_staged = smem > 0;
-    // as many CTAs as are resident at once (registers and shared memory),
-    // each taking rows m = b, b + grid, ...
-    int per_sm = 0;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, gemm_prep, kPrepThreads, smem);
-    if (e != cudaSuccess || per_sm < 1)
-      return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep occupancy: %s",
+    if (e != cudaSuccess)
+      return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep launch: %s",
                              cudaGetErrorString(e));
-    per_sm = std::min(8, per_sm);
-    cfg.gridDim = dim3((unsigned)std::min<long long>(P.M, (long long)sms * per_sm));
-    cfg.dynamicSmemBytes = smem;
-    e = cudaLaunchKernelEx(&cfg, gemm_prep, P);
+    return POLYQ_OK;
   }
+  // Four rows at a time when two CTAs of that size share an SM and the rows
+  // then still fill the GPU twice, else two, else one (K = 5120, M = 768: 81 us
+  // for the whole call at two, 85 at four).
+  const bool xs = P.xscale != nullptr;
+  const size_t half_sm = 112 * 1024;
+  if (P.K <= kRowsMaxK) {
+    if (rows_smem<4>(P.K, Kp, xs) <= half_sm && Mp / 4 >= 2 * sms)
+      return xs ? launch_prep_rows<4, true>(P, sms, dev, cfg)
+                : launch_prep_rows<4, false>(P, sms, dev, cfg);
+    if (rows_smem<2>(P.K, Kp, xs) <= half_sm && Mp / 2 >= sms)
+      return xs ? launch_prep_rows<2, true>(P, sms, dev, cfg)
+                : launch_prep_rows<2, false>(P, sms, dev, cfg);
+    if (rows_smem<1>(P.K, Kp, xs) <= (size_t)kPrepMaxSmem)
+      return xs ? launch_prep_rows<1, true>(P, sms, dev, cfg)
+                : launch_prep_rows<1, false>(P, sms, dev, cfg);
+  }
+  cfg.gridDim = dim3((unsigned)std::min<long long>(Mp, 8ll * sms));
+  cfg.blockDim = dim3(kPrepThreads);
+  e = cudaLaunchKernelEx(&cfg, gemm_prep_wide, P);
   if (e != cudaSuccess)
     return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep launch: %s", cudaGetErrorString(e));
   return POLYQ_OK;
