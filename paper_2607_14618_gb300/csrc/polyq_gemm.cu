@@ -154,7 +154,10 @@ constexpr double kStage512 = 0.27e-6, kPiece512 = 5.5e-6;
 //   CODES   code slots: packed codes and meta, free again once a dequantiser
 //           holds them in registers, so that the copies of the packed weights
 //           run CODES stages ahead whatever the MMAs do
-//   GROUPS  dequantiser groups of four warps (CODES a multiple of it)
+//   GROUPS  dequantiser groups (CODES and OPS multiples of it): the twelve warps as three of
+//           four, a weight row per thread, or as six of two, two rows per thread.  Two rows
+//           share a stage's waits, fence and arrivals (M = 16: 26.0 -> 24.7 us for 13824 x
+//           5120, M = 96: 30.2 -> 29.4); with 512 tokens the MMAs set the pace either way
 //   EPI     epilogue warps (a multiple of four)
 template <int TN_, int NACC_, int BK_, int OPS_, int XS_, int CODES_, int GROUPS_, int EPI_>
 struct Cfg {
@@ -169,18 +172,19 @@ struct Cfg {
   static constexpr int kCodes = HALVES * kBoxBytes;
   static constexpr int kCode = kCodes + kMetaBytes;
   static constexpr int kCodeProd = 2;  // producer warps of the codes
+  static constexpr int kDqGroup = 12 / GROUPS, kDqRows = kRowsCta / (32 * kDqGroup);  // warps, rows a thread
   static constexpr int kEpiWarp = 16, kWarps = kEpiWarp + EPI;
   static constexpr int kThreads = 32 * kWarps;
   static constexpr int kXOff = OPS * kA, kCodeOff = kXOff + XS * kX;  // in shared memory
   static constexpr size_t kSmem = (size_t)kCodeOff + CODES * kCode + 1024;
   static constexpr uint32_t kIdesc = umma_idesc_f16(kRowsN, TN);
   static_assert(kX % 1024 == 0 && kSmem <= 225 * 1024 + 512 && NACC * NBUF * TN <= (int)kTmemCols, "");
-  static_assert(GROUPS == 3 && CODES % GROUPS == 0 && OPS % GROUPS == 0 && kCodeProd <= CODES, "");
+  static_assert((GROUPS == 3 || GROUPS == 6) && CODES % GROUPS == 0 && OPS % GROUPS == 0 && kCodeProd <= CODES, "");
 };
-using Cfg32 = Cfg<32, 1, 64, 6, 16, 9, 3, 4>;
-using Cfg64 = Cfg<64, 1, 64, 6, 8, 9, 3, 4>;
-using Cfg128 = Cfg<128, 1, 64, 6, 6, 6, 3, 4>;
-using Cfg256 = Cfg<256, 1, 64, 6, 4, 6, 3, 4>;
+using Cfg32 = Cfg<32, 1, 64, 6, 16, 6, 6, 4>;
+using Cfg64 = Cfg<64, 1, 64, 6, 8, 6, 6, 4>;
+using Cfg128 = Cfg<128, 1, 64, 6, 6, 6, 6, 4>;
+using Cfg256 = Cfg<256, 1, 64, 6, 4, 6, 6, 4>;
 using Cfg512 = Cfg<256, 2, 32, 6, 7, 9, 3, 8>;
 // Warps 0, 4, 8 and 12, which share a scheduler, are the lone-thread roles
 // (two code producers, the X producer, the MMA issuer), the other twelve of
@@ -1027,13 +1031,13 @@ __device__ __forceinline__ void store_chunk(float* __restrict__ y, uint32_t N, b
 
 // What bounds it, by token tile (13824 x 5120 at B = 3, one call): with 512
 // tokens the tensor core: a stage of 32 K takes 507 cycles of the MMAs' 512,
-// an accumulator drain 9400 cycles per 95000 of a unit (M = 2048: 277 -> 177
-// us; M = 4096: 529 -> 354 us, 1640 TFLOP/s).  With 256 and fewer the latency
-// of a stage of 64 K through its rings, 540 to 620 cycles (M = 256: 53.6 -> 38
-// us, M = 96: 54 -> 30 us, M = 16: 53 -> 26 us): the copy of 128 code rows and
-// 128 meta rows (325 cycles of the TMA unit, which takes a row a cycle and 32
-// bytes across a 32-byte boundary as two), dequantisation, the arrival at the
-// leader and the commit back.  "Before" is one CTA per tile of 256 x 256
+// an accumulator drain 9400 cycles per 95000 of a unit (M = 2048: 277 -> 171
+// us; M = 4096: 529 -> 349 us, 1660 TFLOP/s).  With 256 and fewer the latency
+// of a stage of 64 K through its rings, 440 to 590 cycles (M = 256: 53.6 -> 37
+// us, M = 96: 54 -> 28 us, M = 16: 53 -> 24 us): the arrival at the leader
+// (1300 cycles of a weight slot's turn of 2640), the commit back (400), and
+// dequantisation; the copy of 128 code rows and 128 meta rows takes 325 cycles
+// of the TMA unit (a row a cycle, 32 bytes across a 32-byte boundary two).  "Before" is one CTA per tile of 256 x 256
 // whatever M, which dequantised every weight once per SM and 256 tokens.
 template <class C>
 __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constant__ GmParams P,
@@ -1066,10 +1070,10 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
     s_abort = 0;
     for (int s = 0; s < C::CODES; ++s) {
       mbar_init(smem_u32(&bar_cfull[s]), 1);
-      mbar_init(smem_u32(&bar_cfree[s]), 4);  // one group of four warps
+      mbar_init(smem_u32(&bar_cfree[s]), C::kDqGroup);
     }
     for (int s = 0; s < C::OPS; ++s) {
-      mbar_init(smem_u32(&bar_bready[s]), 2 * 4);  // a group of each CTA
+      mbar_init(smem_u32(&bar_bready[s]), 2 * C::kDqGroup);  // a group of each CTA
       mbar_init(smem_u32(&bar_sfree[s]), 1);
     }
     for (int s = 0; s < C::XS; ++s) {
@@ -1304,8 +1308,9 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
     // wait cannot tell a phase from the last but one: a code slot always
     // belongs to one group, as GROUPS divides CODES.)
     const int dq = (warp >> 2) * 3 + (warp & 3) - 1;  // 0..11
-    const int grp = dq >> 2;
-    const int r = (dq & 3) * 32 + lane;
+    constexpr int RW = C::kDqRows, kRowStep = 32 * C::kDqGroup;
+    const int grp = dq / C::kDqGroup;
+    const int r = dq % C::kDqGroup * 32 + lane;  // the thread's rows: r, r + kRowStep
     const uint32_t code_row = smem_u32(smem_codes) + r * kCodeBox;
     const uint32_t meta_row = smem_u32(smem_codes) + C::kCodes + r * 16;
     // 16-byte chunk c of operand row r lies at (c XOR bits 7..8 of the row's
@@ -1329,33 +1334,56 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
         const bool free = mbar_test(smem_u32(&bar_sfree[s]), sph);
         B.advance(sblk, nblk, kt);
         const int tb = kt - B.kt0;
+        bool early = false;  // the code slot has been released
         const uint32_t op = op_row + s * C::kA;
         const uint32_t codes = code_row + sc * C::kCode;
         auto dequant = [&](auto bits) {
           constexpr int BITS = decltype(bits)::value;
-          const uint32_t meta =
-              lds32(meta_row + sc * C::kCode + ((B.grp_off + tb * C::BK / 64) & 3) * 4);
-          CodeWords<BITS, C::HALVES> cw;
-          cw.load(codes, (B.seg_off + (C::BK / 8) * BITS * tb) & 15);
-          const __half s16 = __ushort_as_half((uint16_t)(meta & 0xFFFFu));
-          const __half z16 = __ushort_as_half((uint16_t)(meta >> 16));
-          const __half2 ss = __halves2half2(s16, s16), zz = __halves2half2(z16, z16);
+          const uint32_t ma = meta_row + sc * C::kCode + ((B.grp_off + tb * C::BK / 64) & 3) * 4;
+          const int off = (B.seg_off + (C::BK / 8) * BITS * tb) & 15;
+          CodeWords<BITS, C::HALVES> cw[RW];
+          __half2 ss[RW], zz[RW];
+#pragma unroll
+          for (int i = 0; i < RW; ++i) {
+            const uint32_t meta = lds32(ma + i * kRowStep * 16);
+            cw[i].load(codes + i * kRowStep * kCodeBox, off);
+            const __half s16 = __ushort_as_half((uint16_t)(meta & 0xFFFFu));
+            const __half z16 = __ushort_as_half((uint16_t)(meta >> 16));
+            ss[i] = __halves2half2(s16, s16);
+            zz[i] = __halves2half2(z16, z16);
+          }
 #pragma unroll 1  // one copy of the code for both halves
           for (int h = 0;;) {
-            uint32_t p[16];
-            dequant_half<BITS>(cw.w, zz, ss, magic, p);
+            uint32_t p[RW][16];
+#pragma unroll
+            for (int i = 0; i < RW; ++i) dequant_half<BITS>(cw[i].w, zz[i], ss[i], magic, p[i]);
             if (h == 0 && !free) {
               w = wait_ab(smem_u32(&bar_sfree[s]), sph, &s_abort);
               if (w != kWaitOk) break;
             }
 #pragma unroll
-            for (int c = 0; c < 4; ++c) sts128((op + h * kHalfTile) ^ (c << 4), p + 4 * c);
-            if (++h == C::HALVES) break;
-            if constexpr (BITS == 8) {
-              cw.load(codes + kBoxBytes, 0);
-            } else if constexpr (C::HALVES == 2) {
+            for (int i = 0; i < RW; ++i)
 #pragma unroll
-              for (int k = 0; k < BITS; ++k) cw.w[k] = cw.w[k + BITS];
+              for (int c = 0; c < 4; ++c)
+                sts128((op + h * kHalfTile + i * kRowStep * 64) ^ (c << 4), p[i] + 4 * c);
+            if (++h == C::HALVES) break;
+            if constexpr (BITS != 8) {
+              // every code word is in registers (the stores above follow the
+              // reads in the shared-memory pipe): the slot is free half a tile
+              // early, which the ring of six needs (its turn, 2930 cycles with
+              // the slot held to the tile's end, set the stage)
+              __syncwarp();
+              if (lane == 0) mbar_arrive(smem_u32(&bar_cfree[sc]));
+              early = true;
+            }
+#pragma unroll
+            for (int i = 0; i < RW; ++i) {
+              if constexpr (BITS == 8) {
+                cw[i].load(codes + kBoxBytes + i * kRowStep * kCodeBox, 0);
+              } else if constexpr (C::HALVES == 2) {
+#pragma unroll
+                for (int k = 0; k < BITS; ++k) cw[i].w[k] = cw[i].w[k + BITS];
+              }
             }
           }
           fence_proxy_async_smem();
@@ -1387,13 +1415,14 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
         }
 #ifdef POLYQ_DEBUG
         for (int h = 0; h < C::HALVES; ++h)
-          dbg_row(smem + s * C::kA + h * kHalfTile, r, un * kRowsN + (int)rank * kRowsCta + r, P.N,
-                  sblk[B.bi], tb * C::HALVES + h);
+          for (int q = r; q < kRowsCta; q += kRowStep)
+            dbg_row(smem + s * C::kA + h * kHalfTile, q, un * kRowsN + (int)rank * kRowsCta + q, P.N,
+                    sblk[B.bi], tb * C::HALVES + h);
 #endif
         __syncwarp();
         if (lane == 0) {
           mbar_arrive_cluster(bready0 + 8 * s);
-          mbar_arrive(smem_u32(&bar_cfree[sc]));
+          if (!early) mbar_arrive(smem_u32(&bar_cfree[sc]));
         }
         sc += C::GROUPS;
         if (sc >= C::CODES) {
@@ -1820,7 +1849,7 @@ extern "C" int polyq_linear_gemm(const polyq_dev_layer* L, const void* X, int64_
     return polyq_set_error(POLYQ_EUNSUPPORTED, "polyq_linear_gemm: device %d >= %d", dev,
                            kMaxDevices);
   // The smallest token tile that holds M (a wider one would multiply padding:
-  // 13824 x 5120 takes 26 / 30 / 38 us at M = 16 / 96 / 256, and took 53 us at
+  // 13824 x 5120 takes 24 / 28 / 37 us at M = 16 / 96 / 256, and took 53 us at
   // each with 256), or for more than 256 tokens the cheaper of 256 and 512 by
   // the model (stage and piece times measured).
   Choice ch = {-1, 0, {}};
