@@ -303,34 +303,30 @@ __global__ void __launch_bounds__(kPrepThreads) gemv_prep(const __grid_constant_
     return;
   }
   __shared__ GvShared S;
-  __shared__ uint32_t s_p3[16];  // 3-bit pair schedule
+  __shared__ uint32_t s_pair[kPairEntries];
   load_shared(P, &S);
-  if (threadIdx.x < 16) {
-    const PairDef d = pair3(threadIdx.x);
-    s_p3[threadIdx.x] = (uint32_t)d.lo | ((uint32_t)d.hi << 8) | ((uint32_t)(d.win + 16) << 16);
-  }
+  load_pairs(s_pair);
   __syncthreads();
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int r = blockIdx.x;
   int l, bi, j;
   rec_pos(S, P.n_layers, r, &l, &bi, &j);
-  int src[2][2];
-  float fac[2][2];
+  RecSlots<kPrepWarps> R;
   const XIn in = xin_of(P, l);
-  rec_sources<NB, kPrepWarps>(in, S.blk[l][bi], j, warp, lane, s_p3, src, fac);  // static layer data
+  rec_sources<NB>(in, S.blk[l][bi], j, warp, lane, s_pair, R);  // static layer data
   if (P.xkind == POLYQ_X_RMSNORM) rms_prefetch(P.xa, P.L[0].K, P.batch);
   pdl_wait();  // x comes from the previous kernel; the records and y may still be in use
   // The streaming kernel writes the status only after its own wait for this
   // grid, so clearing it here cannot lose one of its reports.
   if (P.clear_status && blockIdx.x == 0 && threadIdx.x == 0) *P.status = 0;
-  float ra[2][2], rb[2][2];
-  rec_load<NB, kPrepWarps>(in, S.blk[l][bi], j, warp, lane, s_p3, src, ra, rb);
+  float ra[R.N][2], rb[R.N][2];
+  rec_load(in, R, ra, rb);
   __shared__ float s_rnorm[4];
   __shared__ float s_part[4][kPrepWarps];
   if (P.xkind == POLYQ_X_RMSNORM)
     rms_rnorm<kPrepWarps>(P.xa, P.L[0].K, P.batch, P.eps, s_part, s_rnorm);
-  rec_store<NB, kPrepWarps>(in, S.blk[l][bi], j, warp, lane, s_p3, src, fac, ra, rb, s_rnorm,
-                            reinterpret_cast<uint32_t*>(P.rec + (size_t)r * rec_bytes(NB)));
+  rec_store<NB>(in, S.blk[l][bi].bits, warp, lane, R, ra, rb, s_rnorm,
+                reinterpret_cast<uint32_t*>(P.rec + (size_t)r * rec_bytes(NB)));
 }
 
 template <int NB>

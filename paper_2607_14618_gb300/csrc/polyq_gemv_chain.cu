@@ -180,17 +180,17 @@ __device__ __forceinline__ XIn chain_xin(const ChShared& S, int l, int batch) {
 
 // One activation record of the phase (flat index f) into global memory.
 template <int NB>
-__device__ __noinline__ void build_record(const ChShared& S, int f, int batch, const uint32_t* p3,
+__device__ __noinline__ void build_record(const ChShared& S, int f, int batch, const uint32_t* pairs,
                                           const float* s_rnorm, uint8_t* dst) {
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   int l, bi, j;
   rec_where(S, f, &l, &bi, &j);
   const XIn in = chain_xin(S, l, batch);
-  int src[2][2];
-  float fac[2][2], ra[2][2], rb[2][2];
-  rec_sources<NB>(in, S.blk[l][bi], j, warp, lane, p3, src, fac);
-  rec_load<NB>(in, S.blk[l][bi], j, warp, lane, p3, src, ra, rb);
-  rec_store<NB>(in, S.blk[l][bi], j, warp, lane, p3, src, fac, ra, rb, s_rnorm,
+  RecSlots<kWarps> R;
+  float ra[R.N][2], rb[R.N][2];
+  rec_sources<NB>(in, S.blk[l][bi], j, warp, lane, pairs, R);
+  rec_load(in, R, ra, rb);
+  rec_store<NB>(in, S.blk[l][bi].bits, warp, lane, R, ra, rb, s_rnorm,
                 reinterpret_cast<uint32_t*>(dst));
 }
 
@@ -217,7 +217,7 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
   uint32_t* zeros = reinterpret_cast<uint32_t*>(smem + kStages * kStageBytes);
   uint64_t* bars = reinterpret_cast<uint64_t*>(zeros + 64);
   __shared__ ChShared S;
-  __shared__ uint32_t s_p3[16];
+  __shared__ uint32_t s_pair[kPairEntries];
   __shared__ float s_rnorm[4];
   __shared__ float s_part[4][kWarps];
   __shared__ volatile int s_abort;
@@ -237,10 +237,7 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
     mbar_fence_init();
   }
   if (threadIdx.x < 64) zeros[threadIdx.x] = 0u;
-  if (threadIdx.x < 16) {
-    const PairDef d = pair3(threadIdx.x);
-    s_p3[threadIdx.x] = (uint32_t)d.lo | ((uint32_t)d.hi << 8) | ((uint32_t)(d.win + 16) << 16);
-  }
+  load_pairs(s_pair);
   __syncthreads();
 
   if (warp == kWarps) {
@@ -438,7 +435,7 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
       if (S.kind == POLYQ_X_RMSNORM) rms_rnorm(S.xa, S.K[0], P.batch, S.eps, s_part, s_rnorm);
       int built = 0;
       for (int f = blockIdx.x; f < S.recs; f += G, ++built)
-        build_record<NB>(S, f, P.batch, s_p3, s_rnorm, P.rec + (size_t)f * RB);
+        build_record<NB>(S, f, P.batch, s_pair, s_rnorm, P.rec + (size_t)f * RB);
       consumer_sync();
       if (threadIdx.x == 0) {
         __threadfence();

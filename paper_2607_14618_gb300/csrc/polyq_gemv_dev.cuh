@@ -34,74 +34,73 @@ __device__ __forceinline__ uint32_t pack_half2(__half lo, __half hi) {
 // ---------------------------------------------------------------------------
 // activation records (consumer warps, shared memory)
 // ---------------------------------------------------------------------------
-// Which activation values one consumer thread contributes to a record.  A
-// record has at most two slots per thread:
-//  * b < 16: slot s is the (batch, chunk) pair bc = warp + 4s of the step;
-//    lane q of the warp makes the q-th of the chunk's 32 lane pairs.
-//  * 16-bit: slot s is entry e = tid + 128s of the [batch][lane][16] pairs.
-struct SlotGeom {
-  bool valid;
-  int bb, c, t, jp;
-  int ch[2];  // channels (inside the block) of the pair's low and high half
-  int p[2];   // power-of-two scale exponents of the two halves
-};
-
-// NW warps build a record: a thread has slots s < rec_slots(NW).
+// Which activation values one thread contributes to a record: slot s of
+//  * b < 16: the (batch row, chunk) pair bc = warp + NW s of the step; lane q
+//    of the warp makes the q-th of the chunk's 32 lane pairs;
+//  * 16-bit: entry e = tid + 32 NW s of the [batch][lane][16] pairs.
+// NW warps build a record; a thread has slots s < rec_slots(NW).
 __host__ __device__ constexpr int rec_slots(int nw) { return nw >= 8 ? 1 : 2; }
 
-template <int NB, int BITS, int NW>
-__device__ __forceinline__ SlotGeom slot_geom_t(int warp, int lane, int tid, int s, int j,
-                                                const uint32_t* p3) {
-  SlotGeom g;
-  if constexpr (BITS == 16) {
-    const int e = tid + 32 * NW * s;
-    g.valid = e < NB * 64;
-    g.bb = e / 64;
-    g.t = (e / 16) % 4;
-    g.jp = e % 16;
-    g.c = 0;
-    g.ch[0] = j * 128 + lane_weight16(g.t, 2 * g.jp);
-    g.ch[1] = j * 128 + lane_weight16(g.t, 2 * g.jp + 1);
-    g.p[0] = g.p[1] = 0;
-  } else {
-    constexpr int U = step_units(BITS, NB), NGS = U / 64;
-    constexpr int GP = group_pairs(BITS), GU = group_units(BITS);
-    const int bc = warp + NW * s;
-    g.valid = bc < NB * NGS;
-    g.bb = bc / NGS;
-    g.c = bc - g.bb * NGS;
-    chunk_pair(BITS, NB, g.c, lane, &g.t, &g.jp);
-    const int jj = g.jp % GP, base = (g.jp / GP) * GU;
-    int lo, hi;
-    if constexpr (BITS == 3) {
-      const uint32_t e = p3[jj];  // lo | hi << 8 | (win + 16) << 16
-      lo = (int)(e & 0xFF);
-      hi = (int)((e >> 8) & 0xFF);
-      const int win = (int)(e >> 16) - 16;
-      g.p[0] = 3 * lo - win;
-      g.p[1] = 3 * hi - win - 16;
-    } else {
-      const PairDef d = pair_def(BITS, jj);
-      lo = d.lo;
-      hi = d.hi;
-      g.p[0] = d.plo;
-      g.p[1] = d.phi;
-    }
-    g.ch[0] = j * U + lane_unit(BITS, NB, g.t, base + lo);
-    g.ch[1] = j * U + lane_unit(BITS, NB, g.t, base + hi);
+template <int NW>
+struct RecSlots {
+  static constexpr int N = rec_slots(NW);
+  // Held across the grid-dependency wait, so packed: word of the record that
+  // takes the pair, entry of the chunk's sums (batch row major), the two
+  // halves' power-of-two scale exponents and the batch row, in 12, 4, 4, 4 and
+  // 2 bits; -1: no slot.
+  int geom[N];
+  int src[N][2];    // source channels, -1: none
+  float fac[N][2];  // activation factors
+  __device__ __forceinline__ void set(int s, int at, int sum, int p0, int p1, int row) {
+    geom[s] = at | (sum << 12) | (p0 << 16) | (p1 << 20) | (row << 24);
   }
-  return g;
+  __device__ __forceinline__ bool valid(int s) const { return geom[s] >= 0; }
+  __device__ __forceinline__ int at(int s) const { return geom[s] & 0xFFF; }
+  __device__ __forceinline__ int sum(int s) const { return (geom[s] >> 12) & 0xF; }
+  __device__ __forceinline__ int p(int s, int h) const { return (geom[s] >> (16 + 4 * h)) & 0xF; }
+  __device__ __forceinline__ int row(int s) const { return (geom[s] >> 24) & 0x3; }
+};
+
+// The decoder's pairs (lo | hi << 8 | plo << 16 | phi << 24 of each) of widths
+// 2, 3, 4 and 8, for rec_sources: 8, 16, 4 and 4 of them.  (Two pre-pass CTAs
+// fit beside three streaming CTAs on an SM with this table at 128 bytes and
+// not with 256: the step of the Qwen3-32B linears at batch 4, whose records
+// take more CTAs than there are SMs, 110 us instead of 93.)
+constexpr int kPairEntries = 32;
+__host__ __device__ __forceinline__ int pair_entry0(int bits) {
+  return bits == 2 ? 0 : bits == 3 ? 8 : bits == 4 ? 24 : 28;
+}
+__device__ __forceinline__ void load_pairs(uint32_t* s_pair) {
+  const int i = threadIdx.x;
+  if (i < kPairEntries) {
+    const int bits = i < 8 ? 2 : i < 24 ? 3 : i < 28 ? 4 : 8;
+    const PairDef d = pair_def(bits, i - pair_entry0(bits));
+    s_pair[i] = (uint32_t)d.lo | ((uint32_t)d.hi << 8) | ((uint32_t)d.plo << 16) |
+                ((uint32_t)d.phi << 24);
+  }
 }
 
-template <int NB, int NW>
-__device__ __forceinline__ SlotGeom slot_geom(int bits, int warp, int lane, int tid, int s,
-                                              int j, const uint32_t* p3) {
-  switch (bits) {
-    case 2: return slot_geom_t<NB, 2, NW>(warp, lane, tid, s, j, p3);
-    case 3: return slot_geom_t<NB, 3, NW>(warp, lane, tid, s, j, p3);
-    case 4: return slot_geom_t<NB, 4, NW>(warp, lane, tid, s, j, p3);
-    case 8: return slot_geom_t<NB, 8, NW>(warp, lane, tid, s, j, p3);
-    default: return slot_geom_t<NB, 16, NW>(warp, lane, tid, s, j, p3);
+// Units (inside the step) and scale exponents of the pair that lane `lane` of
+// the warp holding chunk c makes, and the pair's lane t and index jp: the
+// layout's chunk_pair, pair_units and lane_unit with the width as a value, by
+// shifts, so that one short path serves all widths.
+__host__ __device__ __forceinline__ void chunk_pair_units(int bits, int nb, int c, int lane,
+                                                          const uint32_t* pairs, int* t, int* jp,
+                                                          int (&unit)[2], int (&p)[2]) {
+  const int lu = nb == 4 ? 7 : (nb == 2 || bits == 8) ? 8 : 9;       // log2 of the step's units
+  const int lnbx = (nb == 1 || (nb == 2 && bits == 8)) ? 1 : 0;      // boxes
+  const int lper = lu - 2 - lnbx, lcpb = lu - lnbx - 6;              // lane's units, chunks per box
+  const int lgp = bits == 2 ? 3 : bits == 3 ? 4 : 2;                 // pairs per decoder group
+  const int h = c >> lcpb, cb = c - (h << lcpb);
+  *t = (cb << (6 - lper)) + (lane >> (lper - 1));
+  *jp = (h << (lper - 1)) + (lane & ((1 << (lper - 1)) - 1));
+  const uint32_t e = pairs[pair_entry0(bits) + (*jp & ((1 << lgp) - 1))];
+  const int base = (*jp >> lgp) << (lgp + 1);
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const int i = base + (int)((e >> (8 * k)) & 0xFFu);  // unit of the lane
+    unit[k] = ((i >> lper) << (lu - lnbx)) + (*t << lper) + (i & ((1 << lper) - 1));
+    p[k] = (int)((e >> (16 + 8 * k)) & 0xFFu);
   }
 }
 
@@ -122,37 +121,56 @@ __device__ __forceinline__ void prefetch_l2(const void* p) {
   asm volatile("prefetch.global.L2 [%0];" ::"l"(p));
 }
 
-// Pass 1 of a record: the gather indices and activation factors (static
-// layer data, so this may run before the grid-dependency wait), and an L2
-// prefetch of the activations the record will read.  L2 is where writes of
+// Pass 1 of a record: its geometry, gather indices and activation factors
+// (static layer data, so this may run before the grid-dependency wait; the
+// geometry, one width switch per pass before, is found here once, and the
+// Llama2-13B step went from 49.9 to 48.0 us at batch 1), and an
+// L2 prefetch of the activations the record will read.  L2 is where writes of
 // earlier kernels land, so prefetching before their completion is safe: the
 // loads after the wait still see the final values.
-template <int NB, int NW = kWarps>
+template <int NB, int NW>
 __device__ __forceinline__ void rec_sources(const XIn& in, const GvBlock& B, int j, int warp,
-                                            int lane, const uint32_t* p3, int (&src)[2][2],
-                                            float (&fac)[2][2]) {
+                                            int lane, const uint32_t* pairs, RecSlots<NW>& R) {
+  constexpr int LW = rec_lane_words(NB);
   const int32_t* gather = in.gather;
 #pragma unroll
-  for (int s = 0; s < 2; ++s) {
-    src[s][0] = src[s][1] = -1;
-    fac[s][0] = fac[s][1] = 1.f;
-    if (s >= rec_slots(NW)) continue;
-    const SlotGeom g = slot_geom<NB, NW>(B.bits, warp, lane, threadIdx.x, s, j, p3);
-    if (g.valid && g.bb < in.batch) {
+  for (int s = 0; s < R.N; ++s) {
+    int t, jp, unit[2], p[2] = {0, 0}, c = 0, row;
+    bool valid;
+    if (B.bits == 16) {
+      const int e = threadIdx.x + 32 * NW * s;
+      valid = e < NB * 64;
+      row = e / 64;
+      t = (e / 16) % 4;
+      jp = e % 16;
+      unit[0] = lane_weight16(t, 2 * jp);
+      unit[1] = lane_weight16(t, 2 * jp + 1);
+    } else {
+      const int lngs = 31 - __clz(B.units >> 6), bc = warp + NW * s;  // chunks per step: 2^lngs
+      valid = bc < (NB << lngs);
+      row = bc >> lngs;
+      c = bc - (row << lngs);
+      chunk_pair_units(B.bits, NB, c, lane, pairs, &t, &jp, unit, p);
+    }
+    R.set(s, (row * 4 + t) * LW + jp, row * (8 / NB) + c, p[0], p[1], row);
+    if (!valid) R.geom[s] = -1;
 #pragma unroll
-      for (int h = 0; h < 2; ++h)
-        if (g.ch[h] < B.n_ch) {
-          const int p = B.pos0 + g.ch[h];
-          src[s][h] = gather ? __ldg(gather + p) : p;
-          if (in.xscale) fac[s][h] = __ldg(in.xscale + p);
-          const size_t o = (size_t)g.bb * in.K + src[s][h];
-          if (in.kind == POLYQ_X_BF16) {
-            prefetch_l2(in.x + o);
-          } else {
-            prefetch_l2(in.xa + o);
-            if (in.kind == POLYQ_X_SILU_MUL) prefetch_l2(in.xb + o);
-          }
+    for (int h = 0; h < 2; ++h) {
+      R.src[s][h] = -1;
+      R.fac[s][h] = 1.f;
+      const int ch = j * B.units + unit[h];
+      if (valid && row < in.batch && ch < B.n_ch) {
+        const int q = B.pos0 + ch;
+        R.src[s][h] = gather ? __ldg(gather + q) : q;
+        if (in.xscale) R.fac[s][h] = __ldg(in.xscale + q);
+        const size_t o = (size_t)row * in.K + R.src[s][h];
+        if (in.kind == POLYQ_X_BF16) {
+          prefetch_l2(in.x + o);
+        } else {
+          prefetch_l2(in.xa + o);
+          if (in.kind == POLYQ_X_SILU_MUL) prefetch_l2(in.xb + o);
         }
+      }
     }
   }
 }
@@ -225,19 +243,17 @@ __device__ __forceinline__ void rms_rnorm(const float* xa, int K, int batch, flo
 // Pass 2 of a record: load the thread's raw inputs (bf16 x, or the fp32
 // inputs of the transform).  Loads go through L2 (ld.global.cg) because in
 // the chained kernel the inputs are written during the same launch.
-template <int NB, int NW = kWarps>
-__device__ __forceinline__ void rec_load(const XIn& in, const GvBlock& B, int j, int warp,
-                                         int lane, const uint32_t* p3, const int (&src)[2][2],
-                                         float (&ra)[2][2], float (&rb)[2][2]) {
+template <int NW>
+__device__ __forceinline__ void rec_load(const XIn& in, const RecSlots<NW>& R,
+                                         float (&ra)[RecSlots<NW>::N][2],
+                                         float (&rb)[RecSlots<NW>::N][2]) {
 #pragma unroll
-  for (int s = 0; s < 2; ++s) {
-    ra[s][0] = ra[s][1] = rb[s][0] = rb[s][1] = 0.f;
-    if (s >= rec_slots(NW)) continue;
-    const SlotGeom g = slot_geom<NB, NW>(B.bits, warp, lane, threadIdx.x, s, j, p3);
+  for (int s = 0; s < R.N; ++s)
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      if (src[s][h] < 0) continue;
-      const size_t o = (size_t)g.bb * in.K + src[s][h];
+      ra[s][h] = rb[s][h] = 0.f;
+      if (R.src[s][h] < 0) continue;
+      const size_t o = (size_t)R.row(s) * in.K + R.src[s][h];
       if (in.kind == POLYQ_X_BF16) {
         ra[s][h] = __bfloat162float(__ushort_as_bfloat16(
             __ldcg(reinterpret_cast<const unsigned short*>(in.x) + o)));
@@ -246,30 +262,27 @@ __device__ __forceinline__ void rec_load(const XIn& in, const GvBlock& B, int j,
         if (in.kind == POLYQ_X_SILU_MUL) rb[s][h] = __ldcg(in.xb + o);
       }
     }
-  }
 }
 
 // Pass 3: apply the transform (the bf16 activation x), write the optional
 // bf16 copy, multiply by the activation factor, scale each value by the power
 // of two its code carries, round to fp16 and store the pairs and (b < 16)
 // the per-chunk sums C1 = 1024 * sum x' and X = sum x' * 2^p.
-template <int NB, int NW = kWarps>
-__device__ __forceinline__ void rec_store(const XIn& in, const GvBlock& B, int j, int warp,
-                                          int lane, const uint32_t* p3, const int (&src)[2][2],
-                                          const float (&fac)[2][2], const float (&ra)[2][2],
-                                          const float (&rb)[2][2], const float* rnorm,
-                                          uint32_t* rec) {
+template <int NB, int NW>
+__device__ __forceinline__ void rec_store(const XIn& in, int bits, int warp, int lane,
+                                          const RecSlots<NW>& R,
+                                          const float (&ra)[RecSlots<NW>::N][2],
+                                          const float (&rb)[RecSlots<NW>::N][2],
+                                          const float* rnorm, uint32_t* rec) {
   constexpr int LW = rec_lane_words(NB);
   constexpr int PW = rec_pair_words(NB);
   constexpr int NGM = 8 / NB;
-  constexpr int SL = rec_slots(NW);
-  float xv[2][2];
+  float xv[R.N][2];
 #pragma unroll
-  for (int s = 0; s < SL; ++s) {
-    const SlotGeom g = slot_geom<NB, NW>(B.bits, warp, lane, threadIdx.x, s, j, p3);
+  for (int s = 0; s < R.N; ++s) {
 #pragma unroll
     for (int h = 0; h < 2; ++h) {
-      if (src[s][h] < 0) {
+      if (R.src[s][h] < 0) {
         xv[s][h] = 0.f;
         continue;
       }
@@ -277,17 +290,19 @@ __device__ __forceinline__ void rec_store(const XIn& in, const GvBlock& B, int j
       float v;  // the bf16 activation, as a float
       switch (in.kind) {
         case POLYQ_X_F32: v = __bfloat162float(__float2bfloat16_rn(a)); break;
-        case POLYQ_X_RMSNORM: v = __bfloat162float(__float2bfloat16_rn(a * rnorm[g.bb])); break;
+        case POLYQ_X_RMSNORM:
+          v = __bfloat162float(__float2bfloat16_rn(a * rnorm[R.row(s)]));
+          break;
         case POLYQ_X_SILU_MUL:
           v = __bfloat162float(__float2bfloat16_rn(a / (1.f + expf(-a)) * rb[s][h]));
           break;
         default: v = a; break;
       }
       if (in.xout) {
-        const size_t o = (size_t)g.bb * in.K + src[s][h];
+        const size_t o = (size_t)R.row(s) * in.K + R.src[s][h];
         in.xout[o] = __bfloat16_as_ushort(__float2bfloat16_rn(v));  // exact: v is bf16
       }
-      xv[s][h] = v * fac[s][h];  // Section 3.4 factor (1 if none)
+      xv[s][h] = v * R.fac[s][h];  // Section 3.4 factor (1 if none)
     }
   }
   // Largest magnitude of each slot's values over the warp (the bit patterns of
@@ -295,53 +310,52 @@ __device__ __forceinline__ void rec_store(const XIn& in, const GvBlock& B, int j
   // exactly one chunk; a 16-bit batch row spans warps w and w ^ 1, which
   // exchange their maxima through shared memory (the width is uniform over
   // the record, so every consumer thread takes the same branch).
-  uint32_t mx[2] = {0u, 0u};
+  uint32_t mx[R.N];
 #pragma unroll
-  for (int s = 0; s < SL; ++s)
+  for (int s = 0; s < R.N; ++s)
     mx[s] = __reduce_max_sync(0xffffffffu, max(__float_as_uint(fabsf(xv[s][0])),
                                                __float_as_uint(fabsf(xv[s][1]))));
-  if (B.bits == 16) {
-    __shared__ uint32_t s_wmax[NW][2];
+  if (bits == 16) {
+    __shared__ uint32_t s_wmax[NW][R.N];
     consumer_sync<NW>();  // an earlier record's readers are done with s_wmax
     if (lane == 0) {
-      s_wmax[warp][0] = mx[0];
-      s_wmax[warp][1] = mx[1];
+#pragma unroll
+      for (int s = 0; s < R.N; ++s) s_wmax[warp][s] = mx[s];
     }
     consumer_sync<NW>();
-    mx[0] = max(mx[0], s_wmax[warp ^ 1][0]);
-    mx[1] = max(mx[1], s_wmax[warp ^ 1][1]);
+#pragma unroll
+    for (int s = 0; s < R.N; ++s) mx[s] = max(mx[s], s_wmax[warp ^ 1][s]);
   }
   float* recf = reinterpret_cast<float*>(rec);
 #pragma unroll
-  for (int s = 0; s < SL; ++s) {
-    const SlotGeom g = slot_geom<NB, NW>(B.bits, warp, lane, threadIdx.x, s, j, p3);
-    if (!g.valid) continue;  // uniform over the warp
+  for (int s = 0; s < R.N; ++s) {
+    if (!R.valid(s)) continue;  // uniform over the warp
     // e: floor(log2(max)) - kRecExp (an fp32 subnormal maximum counts as 2^-127)
     const int e = mx[s] ? max((int)(mx[s] >> 23) - 127 - kRecExp, kRecExpMin) : 0;
     // 2^(-p-e) lies in [2^-121, 2^126] (p <= 8, -126 <= e <= 113): a
     // normal float, so the products are exact scalings (rounded like any
     // product where they fall below the normal range)
-    const __half hlo = __float2half_rn(xv[s][0] * pow2i(-g.p[0] - e));
-    const __half hhi = __float2half_rn(xv[s][1] * pow2i(-g.p[1] - e));
-    rec[(g.bb * 4 + g.t) * LW + g.jp] = pack_half2(hlo, hhi);
-    if (B.bits != 16) {
+    const __half hlo = __float2half_rn(xv[s][0] * pow2i(-R.p(s, 0) - e));
+    const __half hhi = __float2half_rn(xv[s][1] * pow2i(-R.p(s, 1) - e));
+    rec[R.at(s)] = pack_half2(hlo, hhi);
+    if (bits != 16) {
       // X sums the values the MMA multiplies (fp16 times 2^p), so that the
       // zero-point term removes exactly what the codes' z adds; with
       // activation factors these differ from the fp32 products x * t
       float s1 = __half2float(hlo) + __half2float(hhi);
-      float s2 = __half2float(hlo) * pow2i(g.p[0]) + __half2float(hhi) * pow2i(g.p[1]);
+      float s2 = __half2float(hlo) * pow2i(R.p(s, 0)) + __half2float(hhi) * pow2i(R.p(s, 1));
 #pragma unroll
       for (int o = 16; o > 0; o >>= 1) {
         s1 += __shfl_xor_sync(0xffffffffu, s1, o);
         s2 += __shfl_xor_sync(0xffffffffu, s2, o);
       }
       if (lane == 0) {
-        recf[PW + g.bb * NGM + g.c] = kMagicF * s1;
-        recf[PW + NB * NGM + g.bb * NGM + g.c] = s2;
-        recf[PW + 2 * NB * NGM + g.bb * NGM + g.c] = pow2i(e);
+        recf[PW + R.sum(s)] = kMagicF * s1;
+        recf[PW + NB * NGM + R.sum(s)] = s2;
+        recf[PW + 2 * NB * NGM + R.sum(s)] = pow2i(e);
       }
-    } else if (g.jp == 0 && g.t == 0) {
-      recf[PW + 2 * NB * NGM + g.bb * NGM] = pow2i(e);
+    } else if (R.at(s) == R.row(s) * 4 * LW) {
+      recf[PW + 2 * NB * NGM + R.sum(s)] = pow2i(e);
     }
   }
 }
