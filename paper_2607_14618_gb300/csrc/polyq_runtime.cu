@@ -84,7 +84,11 @@ int polyq_tensor_map_2d(CUtensorMap* out, const void* base, int elem_bytes, uint
                    swizzle_bytes == 128  ? CU_TENSOR_MAP_SWIZZLE_128B
                    : swizzle_bytes == 64 ? CU_TENSOR_MAP_SWIZZLE_64B
                                          : CU_TENSOR_MAP_SWIZZLE_NONE,
-                   CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+                   // No L2 promotion: packed rows start anywhere in 16 bytes, and a
+                   // 128-byte box row then costs the copy unit 1.36 ns instead of
+                   // 1.70 with 256-byte promotion (Llama2-13B step 48.0 -> 47.7 us,
+                   // 13824 x 5120 at B = 6 14.2 -> 13.9 us).
+                   CU_TENSOR_MAP_L2_PROMOTION_NONE, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS)
     return polyq_set_error(POLYQ_ECUDA, "cuTensorMapEncodeTiled failed (%d)", (int)r);
   if (g_maps.size() > 4096) g_maps.clear();
