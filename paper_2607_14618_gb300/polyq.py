@@ -355,7 +355,7 @@ def _require(t, name, dtype, shape, device):
     `device`: the library reads and writes through raw pointers, so a wrong
     buffer would otherwise reach the GPU."""
     import torch
-    if (not isinstance(t, torch.Tensor) or t.dtype != dtype or tuple(t.shape) != tuple(shape)
+    if (not isinstance(t, torch.Tensor) or t.dtype != dtype or t.shape != shape
             or t.device != device or not t.is_contiguous()):
         raise ValueError(f"{name} must be a contiguous {dtype} tensor {list(shape)} on {device}")
 
@@ -368,16 +368,31 @@ def _cuda_input(x, name, dtype, K):
     if (not isinstance(x, torch.Tensor) or x.dtype != dtype or not x.is_cuda or x.dim() != 2
             or x.shape[1] != K):
         raise ValueError(f"{name} must be a CUDA {dtype} tensor [rows][{K}]")
-    if x.device.index != torch.cuda.current_device():
-        raise ValueError(f"{name} is on {x.device}, not on the current device "
+    dev = x.device
+    if dev.index != torch.cuda.current_device():
+        raise ValueError(f"{name} is on {dev}, not on the current device "
                          f"cuda:{torch.cuda.current_device()}")
-    return x.device
+    return dev
 
 
 def _stream_ptr(stream):
+    """The cudaStream_t of `stream` (default: the current device's current
+    stream, whose handle is asked for directly: a torch.cuda.Stream object made
+    only to read it takes 3.2 us, a fifth of a small call's host time)."""
     import torch
-    s = torch.cuda.current_stream() if stream is None else stream
-    return C.c_void_p(s.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+
+
+def _workspace_of(workspace, need, zeros, dev):
+    """The caller's workspace, checked, or a new one of need() bytes.  The
+    library checks the size of a given one itself."""
+    import torch
+    if workspace is None:
+        return (torch.zeros if zeros else torch.empty)(need(), dtype=torch.uint8, device=dev)
+    _require(workspace, "workspace", torch.uint8, (workspace.numel(),), dev)
+    return workspace
 
 
 def gemv_workspace_bytes(layer: DeviceLayer, batch: int) -> int:
@@ -398,17 +413,11 @@ def linear_gemv(layer: DeviceLayer, x, y=None, residual=None, workspace=None, st
     _require(y, "y", torch.float32, (batch, layer.N), dev)
     if residual is not None:
         _require(residual, "residual", torch.float32, (batch, layer.N), dev)
-    ws_need = gemv_workspace_bytes(layer, batch)
-    if workspace is None and ws_need:
-        # the status word must start at zero; every call rewrites the records
-        workspace = torch.zeros(ws_need, dtype=torch.uint8, device=dev)
-    if workspace is not None:
-        _require(workspace, "workspace", torch.uint8, (workspace.numel(),), dev)
-    ws_ptr = workspace.data_ptr() if workspace is not None else None
-    ws_len = workspace.numel() if workspace is not None else 0
+    # the status word must start at zero; every call rewrites the records
+    workspace = _workspace_of(workspace, lambda: gemv_workspace_bytes(layer, batch), True, dev)
     _check(_lib.polyq_linear_gemv(C.byref(layer.desc), x.data_ptr(), batch, y.data_ptr(),
                                   residual.data_ptr() if residual is not None else None,
-                                  ws_ptr, ws_len, _stream_ptr(stream)))
+                                  workspace.data_ptr(), workspace.numel(), _stream_ptr(stream)))
     return y
 
 
@@ -488,10 +497,7 @@ def linear_gemv_group(layers, xs, ys=None, residuals=None, workspace=None, strea
     if ys is None:
         ys = [torch.empty((batch, l.N), dtype=torch.float32, device=dev) for l in layers]
     _check_outputs(layers, batch, ys, residuals, dev)
-    need = gemv_group_workspace_bytes(layers, batch)
-    if workspace is None:
-        workspace = torch.zeros(need, dtype=torch.uint8, device=dev)
-    _require(workspace, "workspace", torch.uint8, (workspace.numel(),), dev)
+    workspace = _workspace_of(workspace, lambda: gemv_group_workspace_bytes(layers, batch), True, dev)
     xa = (C.c_void_p * n)(*[x.data_ptr() for x in xs])
     ya = (C.c_void_p * n)(*[y.data_ptr() for y in ys])
     ra = None
@@ -524,10 +530,7 @@ def linear_gemv_input(layers, kind, a, b=None, eps=1e-6, ys=None, residuals=None
     if ys is None:
         ys = [torch.empty((batch, l.N), dtype=torch.float32, device=dev) for l in layers]
     _check_outputs(layers, batch, ys, residuals, dev)
-    need = gemv_group_workspace_bytes(layers, batch)
-    if workspace is None:
-        workspace = torch.zeros(need, dtype=torch.uint8, device=dev)
-    _require(workspace, "workspace", torch.uint8, (workspace.numel(),), dev)
+    workspace = _workspace_of(workspace, lambda: gemv_group_workspace_bytes(layers, batch), True, dev)
     inp = GemvInput(kind, eps, a.data_ptr(), b.data_ptr() if b is not None else None,
                     x_out.data_ptr() if x_out is not None else None)
     ya = (C.c_void_p * n)(*[y.data_ptr() for y in ys])
@@ -556,15 +559,9 @@ def linear_gemm(layer: DeviceLayer, X, Y=None, workspace=None, stream=None):
     if Y is None:
         Y = torch.empty((M, layer.N), dtype=torch.float32, device=dev)
     _require(Y, "Y", torch.float32, (M, layer.N), dev)
-    ws_need = gemm_workspace_bytes(layer, M)
-    if workspace is None and ws_need:
-        workspace = torch.empty(ws_need, dtype=torch.uint8, device=dev)
-    if workspace is not None:
-        _require(workspace, "workspace", torch.uint8, (workspace.numel(),), dev)
-    ws_ptr = workspace.data_ptr() if workspace is not None else None
-    ws_len = workspace.numel() if workspace is not None else 0
+    workspace = _workspace_of(workspace, lambda: gemm_workspace_bytes(layer, M), False, dev)
     _check(_lib.polyq_linear_gemm(C.byref(layer.desc), X.data_ptr(), M, Y.data_ptr(),
-                                  ws_ptr, ws_len, _stream_ptr(stream)))
+                                  workspace.data_ptr(), workspace.numel(), _stream_ptr(stream)))
     return Y
 
 
