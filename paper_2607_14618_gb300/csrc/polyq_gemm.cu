@@ -486,11 +486,12 @@ constexpr int kRowExp = 14;       // a row's largest magnitude becomes [2^14, 2^
 constexpr int kRowExpMin = -126;  // 2^e stays a normal float
 constexpr int kPrepThreads = 256;
 constexpr int kPrepMaxSmem = 200 * 1024;
-constexpr int kSmallQuads = 4;                // 4-slot quads per thread of gemm_prep_small
+constexpr int kSmallOcts = 2;                 // 8-slot pieces per thread of gemm_prep_small
 constexpr int kSmallMaxK = 32768;             // widest row it stages
-constexpr int kSmallMaxM = 128;               // most rows it is used for (K = 13824: 34 us for the
-                                              // call at M = 128, 37 with gemm_prep_rows; K = 5120,
-                                              // M = 256: 40 and 37)
+// Most rows it is used for: 13824 x 5120 / 5120 x 13824 at M = 256 36.1 / 40.1
+// us for the call, 37.1 / 45.8 with gemm_prep_rows; at M = 512 59.4 / 66.2 and
+// 60.3 / 58.6.
+constexpr int kSmallMaxM = 256;
 
 // Element offset of Xg(m, k) in the blocked layout: block (m / R, k / 32) of
 // R rows x 32 fp16, row m % R at 64 bytes each, its 16-byte chunks in the
@@ -509,6 +510,27 @@ __device__ __forceinline__ int slot_pos(const PrepTables& S, int nblk, int bk, i
   const int o = k - B.kt0 * bk;
   const int w = (o & ~(kSlots - 1)) + S.code[width_index(B.bits)][o & (kSlots - 1)];
   return w < B.n_ch ? B.pos0 + w : -1;
+}
+
+// Source channels (-1 past the end of the block) and, for a scaled layer,
+// activation factors of the 8 slots from k on (k a multiple of 8: they lie in
+// one block and half group, so that finding them takes 11 instructions a slot
+// and not the 60 of slot_pos).
+template <bool XS>
+__device__ __forceinline__ void slot_sources(const GmParams& P, const PrepTables& S, int k,
+                                             int (&src)[8], float (&fac)[8]) {
+  const GmBlock& B = S.blk[find_kblock(S.blk, P.n_blocks, P.bk == 64 ? k >> 6 : k >> 5)];
+  const int o = k - B.kt0 * P.bk;
+  const uint2 c8 = *reinterpret_cast<const uint2*>(&S.code[width_index(B.bits)][o & (kSlots - 1)]);
+  const int base = o & ~(kSlots - 1);
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int w = base + (int)(((u < 4 ? c8.x : c8.y) >> (8 * (u & 3))) & 0xFFu);
+    const int p = B.pos0 + w;
+    const bool in = w < B.n_ch;
+    src[u] = !in ? -1 : (P.gather ? __ldg(P.gather + p) : p);
+    fac[u] = (XS && in) ? __ldg(P.xscale + p) : 0.f;
+  }
 }
 
 // Y = 0 by CTA `cta` of `n_cta` (Y is 16-byte aligned).
@@ -583,23 +605,10 @@ __global__ void __launch_bounds__(kRowsThreads) gemm_prep_rows(const __grid_cons
   uint16_t* s_map = reinterpret_cast<uint16_t*>(psm + (size_t)n8 * 16 * RW + 16);
   float* s_fac = reinterpret_cast<float*>(s_map + Kp);
   {
-    // a thread takes 8 consecutive slots (of one block and half group), so
-    // that finding them costs 11 instructions a slot and not 60
     for (int k = 8 * threadIdx.x; k < Kp; k += 8 * kRowsThreads) {
-      const GmBlock& B = S.blk[find_kblock(S.blk, P.n_blocks, P.bk == 64 ? k >> 6 : k >> 5)];
-      const int o = k - B.kt0 * P.bk;
-      const uint2 c8 = *reinterpret_cast<const uint2*>(&S.code[width_index(B.bits)][o & (kSlots - 1)]);
-      const int base = o & ~(kSlots - 1);
       int src[8];
       float fac[8];
-#pragma unroll
-      for (int u = 0; u < 8; ++u) {
-        const int w = base + (int)(((u < 4 ? c8.x : c8.y) >> (8 * (u & 3))) & 0xFFu);
-        const int p = B.pos0 + w;
-        const bool in = w < B.n_ch;
-        src[u] = !in ? -1 : (P.gather ? __ldg(P.gather + p) : p);
-        fac[u] = (XS && in) ? __ldg(P.xscale + p) : 0.f;
-      }
+      slot_sources<XS>(P, S, k, src, fac);
       uint32_t m[4];
 #pragma unroll
       for (int u = 0; u < 8; ++u) {
@@ -790,7 +799,11 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep_wide(const __grid_cons
 // gathering a segment of the row's slots, so that even one row is spread over
 // the GPU; further CTAs zero Y.  Every CTA stages the whole row in shared
 // memory and finds its largest magnitude itself.  A thread's gather indices
-// (and factors) are loaded before the wait for the previous kernel.
+// (and factors) are loaded before the wait for the previous kernel.  Bound by
+// latency and by the instructions of the slot look-up: with eight slots a look-
+// up and 16-byte stores the call takes 25.8 instead of 28.1 us at 13824 x 5120,
+// M = 96, 27.0 instead of 30.7 at 5120 x 13824.
+template <bool XS>
 __global__ void __launch_bounds__(kPrepThreads) gemm_prep_small(const __grid_constant__ GmParams P) {
   extern __shared__ __align__(16) uint8_t psm[];
   pdl_trigger();
@@ -804,74 +817,87 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep_small(const __grid_con
   load_tables(P, &S);
   __syncthreads();
   const int m = blockIdx.x / P.prep_seg, seg = blockIdx.x % P.prep_seg;
-  const int quads = P.KT * P.bk / 4, ks = P.KT * P.bk / kSlots;
-  const int q_lo = (int)((long long)seg * quads / P.prep_seg);
-  const int q_hi = (int)((long long)(seg + 1) * quads / P.prep_seg);
-  int src[kSmallQuads][4];
-  float fac[kSmallQuads][4];
+  const int octs = P.KT * P.bk / 8, ks = P.KT * P.bk / kSlots;
+  const int o_lo = (int)((long long)seg * octs / P.prep_seg);
+  const int o_hi = (int)((long long)(seg + 1) * octs / P.prep_seg);
+  int src[kSmallOcts][8];
+  float fac[kSmallOcts][8];
 #pragma unroll
-  for (int u = 0; u < kSmallQuads; ++u) {
-    const int i = q_lo + u * kPrepThreads + threadIdx.x;
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int p = i < q_hi && m < P.M ? slot_pos(S, P.n_blocks, P.bk, 4 * i + e) : -1;
-      src[u][e] = p < 0 ? -1 : (P.gather ? __ldg(P.gather + p) : p);
-      fac[u][e] = (P.xscale && p >= 0) ? __ldg(P.xscale + p) : 1.f;
-    }
+  for (int u = 0; u < kSmallOcts; ++u) {
+    const int i = o_lo + u * kPrepThreads + threadIdx.x;
+    if (i < o_hi && m < P.M) slot_sources<XS>(P, S, 8 * i, src[u], fac[u]);
   }
   pdl_wait();  // X comes from the previous kernel; the workspace may still be in use
   if (blockIdx.x == 0 && threadIdx.x == 0) *P.status = 0;
-  float inv = 0.f;
-  const uint16_t* s_row = reinterpret_cast<const uint16_t*>(psm);
-  if (m < P.M) {
-    const uint16_t* row = reinterpret_cast<const uint16_t*>(P.x) + (size_t)m * P.K;
-    uint32_t mx = 0;
-    if ((P.K & 7) == 0 && (reinterpret_cast<uintptr_t>(row) & 15) == 0) {
-      for (int i = threadIdx.x; i < P.K / 8; i += kPrepThreads) {
-        const uint4 v = __ldcg(reinterpret_cast<const uint4*>(row) + i);
-        reinterpret_cast<uint4*>(psm)[i] = v;
-        mx = bf16x8_max(v, mx);
-      }
-    } else {
-      for (int i = threadIdx.x; i < P.K; i += kPrepThreads) {
-        const uint16_t v = __ldcg(row + i);
-        reinterpret_cast<uint16_t*>(psm)[i] = v;
-        mx = max(mx, (uint32_t)(v & 0x7FFFu));
-      }
-    }
-    mx = max_halves(mx) << 16;  // bf16 magnitude bits -> fp32 bits
-    __syncthreads();
-    if (P.xscale) {  // the largest |x * t| over the whole row
-      mx = 0;
-      for (int p = threadIdx.x; p < P.K; p += kPrepThreads) {
-        const int c = P.gather ? __ldg(P.gather + p) : p;
-        mx = max(mx, __float_as_uint(fabsf(__uint_as_float((uint32_t)s_row[c] << 16) *
-                                           __ldg(P.xscale + p))));
-      }
-    }
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    if ((threadIdx.x & 31) == 0) s_wmax[threadIdx.x >> 5] = mx;
-    __syncthreads();
-#pragma unroll
-    for (int w = 0; w < kPrepThreads / 32; ++w) mx = max(mx, s_wmax[w]);
-    const int e = row_exp(mx);
-    if (seg == 0 && threadIdx.x == 0) P.rowscale[m] = __int_as_float((127 + e) << 23);
-    inv = __int_as_float((127 - e) << 23);
+  if (m >= P.M) {  // a row that pads the token tile: its MMA columns must be finite
+    for (int i = o_lo + threadIdx.x; i < o_hi; i += kPrepThreads)
+      *reinterpret_cast<uint4*>(P.xg + xg_off(m, 8 * i, ks, P.r_log2)) = make_uint4(0u, 0u, 0u, 0u);
+    return;
   }
+  const uint16_t* s_row = reinterpret_cast<const uint16_t*>(psm);
+  const uint16_t* row = reinterpret_cast<const uint16_t*>(P.x) + (size_t)m * P.K;
+  uint32_t mx = 0;
+  if ((P.K & 7) == 0 && (reinterpret_cast<uintptr_t>(row) & 15) == 0) {
+    constexpr int U = 4;  // a thread's 16-byte loads in flight
+    const int n8 = P.K / 8;
+    for (int i0 = threadIdx.x; i0 < n8; i0 += U * kPrepThreads) {
+      uint4 v[U];
 #pragma unroll
-  for (int u = 0; u < kSmallQuads; ++u) {
-    const int i = q_lo + u * kPrepThreads + threadIdx.x;
-    if (i >= q_hi) break;
-    float v[4];
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * kPrepThreads;
+        v[u] = i < n8 ? __ldcg(reinterpret_cast<const uint4*>(row) + i) : make_uint4(0u, 0u, 0u, 0u);
+      }
 #pragma unroll
-    for (int e = 0; e < 4; ++e)
-      v[e] = src[u][e] < 0
-                 ? 0.f
-                 : __uint_as_float((uint32_t)s_row[src[u][e]] << 16) * fac[u][e] * inv;
-    const __half2 a = __halves2half2(__float2half_rn(v[0]), __float2half_rn(v[1]));
-    const __half2 b = __halves2half2(__float2half_rn(v[2]), __float2half_rn(v[3]));
-    *reinterpret_cast<uint2*>(P.xg + xg_off(m, 4 * i, ks, P.r_log2)) =
-        make_uint2(*reinterpret_cast<const uint32_t*>(&a), *reinterpret_cast<const uint32_t*>(&b));
+      for (int u = 0; u < U; ++u) {
+        const int i = i0 + u * kPrepThreads;
+        if (i < n8) reinterpret_cast<uint4*>(psm)[i] = v[u];
+        mx = bf16x8_max(v[u], mx);
+      }
+    }
+  } else {
+    for (int i = threadIdx.x; i < P.K; i += kPrepThreads) {
+      const uint16_t v = __ldcg(row + i);
+      reinterpret_cast<uint16_t*>(psm)[i] = v;
+      mx = max(mx, (uint32_t)(v & 0x7FFFu));
+    }
+  }
+  mx = max_halves(mx) << 16;  // bf16 magnitude bits -> fp32 bits
+  __syncthreads();
+  if (XS) {  // the largest |x * t| over the whole row
+    mx = 0;
+    for (int p = threadIdx.x; p < P.K; p += kPrepThreads) {
+      const int c = P.gather ? __ldg(P.gather + p) : p;
+      mx = max(mx, __float_as_uint(fabsf(__uint_as_float((uint32_t)s_row[c] << 16) *
+                                         __ldg(P.xscale + p))));
+    }
+  }
+  mx = __reduce_max_sync(0xffffffffu, mx);
+  if ((threadIdx.x & 31) == 0) s_wmax[threadIdx.x >> 5] = mx;
+  __syncthreads();
+#pragma unroll
+  for (int w = 0; w < kPrepThreads / 32; ++w) mx = max(mx, s_wmax[w]);
+  const int e = row_exp(mx);
+  if (seg == 0 && threadIdx.x == 0) P.rowscale[m] = __int_as_float((127 + e) << 23);
+  const float inv = __int_as_float((127 - e) << 23);
+#pragma unroll
+  for (int u = 0; u < kSmallOcts; ++u) {
+    const int i = o_lo + u * kPrepThreads + threadIdx.x;
+    if (i >= o_hi) break;
+    uint32_t w[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float v[2];
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        const int c = src[u][2 * q + h];
+        const float x = c < 0 ? 0.f : __uint_as_float((uint32_t)s_row[c] << 16);
+        v[h] = (XS ? x * fac[u][2 * q + h] : x) * inv;
+      }
+      const __half2 p = __floats2half2_rn(v[0], v[1]);
+      w[q] = *reinterpret_cast<const uint32_t*>(&p);
+    }
+    *reinterpret_cast<uint4*>(P.xg + xg_off(m, 8 * i, ks, P.r_log2)) =
+        make_uint4(w[0], w[1], w[2], w[3]);
   }
 }
 
@@ -1652,6 +1678,40 @@ int launch_prep_rows(const GmParams& P, int sms, int dev, cudaLaunchConfig_t cfg
   return POLYQ_OK;
 }
 
+// The pre-pass of a few rows: about two CTAs per SM, each with half to
+// kSmallOcts pieces per thread, and CTAs that zero Y.  (Four per SM: the same
+// up to M = 64, M = 128 0.3 us slower; eight 0.8 to 2.6 us slower.)
+template <bool XS>
+int launch_prep_small(GmParams& P, int sms, int dev, cudaLaunchConfig_t cfg) {
+  static std::atomic<bool> attr_done[kMaxDevices];
+  cudaError_t e;
+  if (!attr_done[dev].load(std::memory_order_acquire)) {
+    e = cudaFuncSetAttribute(gemm_prep_small<XS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             kSmallMaxK * 2);
+    if (e != cudaSuccess)
+      return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep smem attribute: %s",
+                             cudaGetErrorString(e));
+    attr_done[dev].store(true, std::memory_order_release);
+  }
+  const int Mp = P.units_m << (P.r_log2 + 1);
+  const int octs = P.KT * P.bk / 8;
+  const int lo = (octs + kSmallOcts * kPrepThreads - 1) / (kSmallOcts * kPrepThreads);
+  const int hi = (2 * octs + kPrepThreads - 1) / kPrepThreads;  // half of the threads at work
+  P.prep_seg = std::max(lo, std::min(hi, 2 * sms / Mp));
+  P.prep_rows = Mp * P.prep_seg;
+  int n_zero = 0;
+  if (P.ksplit > 1 || P.streamk)  // eight float4 per thread, at most two CTAs per SM
+    n_zero = (int)std::min<long long>(2 * sms, ((long long)P.M * P.N + 32 * kPrepThreads - 1) /
+                                                   (32 * kPrepThreads));
+  cfg.gridDim = dim3((unsigned)(P.prep_rows + n_zero));
+  cfg.blockDim = dim3(kPrepThreads);
+  cfg.dynamicSmemBytes = ((size_t)P.K * 2 + 15) / 16 * 16;
+  e = cudaLaunchKernelEx(&cfg, gemm_prep_small<XS>, P);
+  if (e != cudaSuccess)
+    return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep launch: %s", cudaGetErrorString(e));
+  return POLYQ_OK;
+}
+
 int launch_prep(GmParams& P, int sms, int dev, cudaStream_t st) {
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1663,35 +1723,9 @@ int launch_prep(GmParams& P, int sms, int dev, cudaStream_t st) {
   const int Kp = P.KT * P.bk;
   const int Mp = P.units_m << (P.r_log2 + 1);
   cudaError_t e;
-  if (P.M <= kSmallMaxM && P.K <= kSmallMaxK) {
-    static std::atomic<bool> attr_done[kMaxDevices];
-    if (!attr_done[dev].load(std::memory_order_acquire)) {
-      e = cudaFuncSetAttribute(gemm_prep_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                               kSmallMaxK * 2);
-      if (e != cudaSuccess)
-        return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep smem attribute: %s",
-                               cudaGetErrorString(e));
-      attr_done[dev].store(true, std::memory_order_release);
-    }
-    // about four CTAs per SM, each with one to kSmallQuads quads per thread
-    const int quads = Kp / 4;
-    const int lo = (quads + kSmallQuads * kPrepThreads - 1) / (kSmallQuads * kPrepThreads);
-    const int hi = (quads + kPrepThreads - 1) / kPrepThreads;
-    P.prep_seg = std::max(lo, std::min(hi, 4 * sms / Mp));
-    P.prep_rows = Mp * P.prep_seg;
-    int n_zero = 0;
-    if (P.ksplit > 1 || P.streamk)  // eight float4 per thread, at most two CTAs per SM
-      n_zero = (int)std::min<long long>(2 * sms, ((long long)P.M * P.N + 32 * kPrepThreads - 1) /
-                                                     (32 * kPrepThreads));
-    cfg.gridDim = dim3((unsigned)(P.prep_rows + n_zero));
-    cfg.blockDim = dim3(kPrepThreads);
-    cfg.dynamicSmemBytes = ((size_t)P.K * 2 + 15) / 16 * 16;
-    e = cudaLaunchKernelEx(&cfg, gemm_prep_small, P);
-    if (e != cudaSuccess)
-      return polyq_set_error(POLYQ_ECUDA, "polyq_linear_gemm: prep launch: %s",
-                             cudaGetErrorString(e));
-    return POLYQ_OK;
-  }
+  if (P.M <= kSmallMaxM && P.K <= kSmallMaxK)
+    return P.xscale ? launch_prep_small<true>(P, sms, dev, cfg)
+                    : launch_prep_small<false>(P, sms, dev, cfg);
   // Four rows at a time when two CTAs of that size share an SM and the rows
   // then still fill the GPU twice, else two, else one (K = 5120, M = 768: 81 us
   // for the whole call at two, 85 at four).
