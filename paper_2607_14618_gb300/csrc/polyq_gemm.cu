@@ -138,11 +138,15 @@ constexpr double kZeroBytesPerS = 5e12;  // the pre-pass zeroing Y
 constexpr uint32_t kTmemCols = 512;
 // Cost model of the split of K (plan_split), seconds: one stage of a pair and
 // the overhead of a piece, by token tile.
-constexpr double kStage32 = 0.27e-6, kPiece32 = 2.5e-6;
-constexpr double kStage64 = 0.27e-6, kPiece64 = 2.5e-6;
-constexpr double kStage128 = 0.29e-6, kPiece128 = 3e-6;
-constexpr double kStage256 = 0.31e-6, kPiece256 = 4.5e-6;
-constexpr double kStage512 = 0.27e-6, kPiece512 = 5.5e-6;
+// (Stages as traced; pieces set so that the model picks the faster of both
+// splits and both tiles on 5120 x 5120, 13824 x 5120 and 5120 x 13824 from M =
+// 16 to 4096, to 2%: 5120 x 5120, M = 512 34.5 us with 4.5 and 5.5, 32.2 with
+// 3.5 and 6.5; 13824 x 5120, M = 256 36.3 and 34.4.)
+constexpr double kStage32 = 0.23e-6, kPiece32 = 1.5e-6;
+constexpr double kStage64 = 0.24e-6, kPiece64 = 1.5e-6;
+constexpr double kStage128 = 0.26e-6, kPiece128 = 2e-6;
+constexpr double kStage256 = 0.31e-6, kPiece256 = 3.5e-6;
+constexpr double kStage512 = 0.27e-6, kPiece512 = 6.5e-6;
 
 // One kernel per token count T of a work unit.
 //   TN      tokens per MMA (its N); CTA r of the pair holds TN / 2 of them
