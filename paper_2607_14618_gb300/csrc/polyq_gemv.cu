@@ -348,8 +348,10 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) gemv_main(const __grid_c
     int rec_a[kStages], rec_b[kStages];  // records of each stage's steps (-1: none)
     // Weights of a stage: one item, or at batch 2-4 two consecutive steps of
     // one block and tile whose codes take one box each.  A stage is planned
-    // (its descriptor and copy coordinates, from the shared layer tables)
-    // before the wait for its slot, and issued after it.
+    // (its descriptor and copy coordinates, from the shared layer tables) and
+    // issued after the wait for its slot.  (Planning the next one before the
+    // wait was worth 4% at batch 4 while lane 0 of a whole warp did this; an
+    // elected thread is 7% faster than that, and 1% more without.)
     struct Plan {
       uint4 d;
 #ifdef POLYQ_DEBUG
@@ -434,30 +436,21 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) gemv_main(const __grid_c
                 full0 + 8 * slot);
     };
     int ks = 0;  // stages issued
-    if (lane == 0) {
-      for (int l = 0; l < nl; ++l) {
-        for (int b = 0; b < S.n_blocks[l]; ++b) prefetch_tmap(&P.L[l].tm_codes[b]);
-        prefetch_tmap(&P.L[l].tm_meta);
-      }
-      if (item < hi) {
-        Plan p0;
-        plan_stage(p0);
-        issue_stage(ks++, p0);
-      }
+    if (!elect_one()) return;
+    for (int l = 0; l < nl; ++l) {
+      for (int b = 0; b < S.n_blocks[l]; ++b) prefetch_tmap(&P.L[l].tm_codes[b]);
+      prefetch_tmap(&P.L[l].tm_meta);
+    }
+    if (item < hi) {
+      Plan p0;
+      plan_stage(p0);
+      issue_stage(ks++, p0);
     }
     pdl_wait();  // the records come from the pre-pass of this call
     fence_proxy_async_global();  // it wrote them through the generic proxy
-    if (lane != 0) return;
     if (ks > 0) issue_records(0);
-    // At batch 2-4, where the producer's per-stage work is on the ring's
-    // critical path, the next stage is planned while its slot is still in
-    // use; at batch 1 after the wait (measured 0.7% faster there).
-    constexpr bool kPlanAhead = NB > 1;
     bool ok = true;
-    Plan pn;
-    bool have = item < hi;
-    if (kPlanAhead && have) plan_stage(pn);
-    while (have) {
+    while (item < hi) {
       const int slot = ks % kStages;
       if (ks >= kStages && !wait_or_abort(empty0 + 8 * slot, ((ks / kStages) - 1) & 1, &s_abort)) {
         if (!s_abort) atomicExch(P.status, kStatusTimeoutEmpty);
@@ -465,12 +458,11 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) gemv_main(const __grid_c
         ok = false;
         break;
       }
-      if (!kPlanAhead) plan_stage(pn);
+      Plan pn;
+      plan_stage(pn);
       issue_stage(ks, pn);
       issue_records(ks);
       ++ks;
-      have = item < hi;
-      if (kPlanAhead && have) plan_stage(pn);
     }
     // wait (bounded) for the copies still in flight, then mark the end of
     // the items in the next stage

@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
     // Weights are issued as soon as a stage is free, across phase
     // boundaries; an item's activation record is issued once its phase's
     // records are all built (a counter per phase, summed over launches).
-    if (lane != 0) return;
+    if (!elect_one()) return;
     const unsigned epoch = s_epoch;
     int kg = 0, kr = 0;           // items whose weights / records were issued
     int ready_phase = -1;         // phases whose records are known to be built
