@@ -178,22 +178,6 @@ __device__ __forceinline__ XIn chain_xin(const ChShared& S, int l, int batch) {
   return in;
 }
 
-// One activation record of the phase (flat index f) into global memory.
-template <int NB>
-__device__ __noinline__ void build_record(const ChShared& S, int f, int batch, const uint32_t* pairs,
-                                          const float* s_rnorm, uint8_t* dst) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  int l, bi, j;
-  rec_where(S, f, &l, &bi, &j);
-  const XIn in = chain_xin(S, l, batch);
-  RecSlots<kWarps> R;
-  float ra[R.N][2], rb[R.N][2];
-  rec_sources<NB>(in, S.blk[l][bi], j, warp, lane, pairs, R);
-  rec_load(in, R, ra, rb);
-  rec_store<NB>(in, S.blk[l][bi].bits, warp, lane, R, ra, rb, s_rnorm,
-                reinterpret_cast<uint32_t*>(dst));
-}
-
 // Outputs of a phase start as the residual (or zero); grid-stride over all
 // consumer threads of the launch.
 __device__ void init_outputs(const ChPhase* ph, int batch) {
@@ -397,13 +381,17 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
   // of consumer_sync() calls whatever happens, so a wait that gives up never
   // strands a warp at a barrier; decisions that steer control flow are taken
   // by thread 0 and read by all after a consumer_sync().
-  auto grid_sync = [&]() -> bool {
+  auto grid_arrive = [&]() {
     consumer_sync();  // this CTA's atomic additions are issued
+    if (threadIdx.x == 0 && !s_abort) {
+      __threadfence();
+      atomicAdd(P.bar, 1u);
+    }
+  };
+  auto grid_wait = [&]() -> bool {
     if (threadIdx.x == 0) {
       bool ok = !s_abort;
       if (ok) {
-        __threadfence();
-        atomicAdd(P.bar, 1u);
         const unsigned target = (gen + 1) * (unsigned)G;
         uint32_t it = 0;
         while (ld_acquire_gpu(P.bar) < target) {
@@ -424,18 +412,42 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
     return s_ok;
   };
 
-  init_outputs(P.ph, P.batch);
-  bool alive = grid_sync();
-  for (int p = 0; p < P.n_phases && alive; ++p) {
-    const ChPhase* ph = P.ph + p;
-    load_phase(ph, &S);
+  // Between arriving at the barrier before phase p and waiting there: the
+  // phase's tables and, for this CTA's first record, everything that does not
+  // depend on the previous phase (geometry, gather indices, factors).
+  RecSlots<kWarps> R;
+  XIn in;
+  int rec_bits = 0;
+  auto record_of = [&](int f) {
+    int l, bi, j;
+    rec_where(S, f, &l, &bi, &j);
+    in = chain_xin(S, l, P.batch);
+    rec_bits = S.blk[l][bi].bits;
+    rec_sources<NB>(in, S.blk[l][bi], j, warp, lane, s_pair, R);
+  };
+  auto prepare = [&](int p) {
+    load_phase(P.ph + p, &S);  // grid_arrive's first sync ended this CTA's use of the last one's
     consumer_sync();
+    if (blockIdx.x < S.recs) record_of(blockIdx.x);
+  };
+
+  init_outputs(P.ph, P.batch);
+  grid_arrive();
+  prepare(0);
+  bool alive = grid_wait();
+  for (int p = 0; p < P.n_phases && alive; ++p) {
     // this CTA's share of the phase's records (the inputs are complete)
     if (blockIdx.x < S.recs) {
       if (S.kind == POLYQ_X_RMSNORM) rms_rnorm(S.xa, S.K[0], P.batch, S.eps, s_part, s_rnorm);
       int built = 0;
-      for (int f = blockIdx.x; f < S.recs; f += G, ++built)
-        build_record<NB>(S, f, P.batch, s_pair, s_rnorm, P.rec + (size_t)f * RB);
+#pragma unroll 1
+      for (int f = blockIdx.x; f < S.recs; f += G, ++built) {
+        if (built) record_of(f);
+        float ra[R.N][2], rb[R.N][2];
+        rec_load(in, R, ra, rb);
+        rec_store<NB>(in, rec_bits, warp, lane, R, ra, rb, s_rnorm,
+                      reinterpret_cast<uint32_t*>(P.rec + (size_t)f * RB));
+      }
       consumer_sync();
       if (threadIdx.x == 0) {
         __threadfence();
@@ -482,7 +494,11 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
         phase ^= 1u;
       }
     }
-    if (p + 1 < P.n_phases) alive = grid_sync();
+    if (p + 1 < P.n_phases) {
+      grid_arrive();
+      prepare(p + 1);
+      alive = grid_wait();
+    }
   }
   // the last CTA to finish clears the barrier counters and counts the launch
   consumer_sync();
