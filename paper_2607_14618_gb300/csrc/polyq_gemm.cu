@@ -47,75 +47,12 @@
 #include <algorithm>
 #include <atomic>
 #include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
-#include <atomic>
-#include <cstring>
 
 #include "polyq.h"
 #ifdef POLYQ_DEBUG
 #include "polyq_debug.h"
 #endif
 #include "polyq_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
-#include "polyq_gemv_dev.cuh"
 #include "polyq_gemv_dev.cuh"
 #include "polyq_internal.h"
 
@@ -562,9 +499,10 @@ __device__ __forceinline__ uint32_t max_halves(uint32_t mx2) {
 // shared-memory wavefronts (62-75% of the pipe) and issue (60%); one row at a
 // time, with an index, a value, a test and 64-bit address arithmetic per
 // element, it was bound by 25 to 34 instructions an element.  K = 5120, M =
-// 8192: 49 -> 37 us; K = 13824, M = 2048: 48 -> 31 us (cold cache).  16-byte pieces of RW words lie in planes, so that the staging stores of a
-// warp are contiguous; the slot map holds positions in that layout and is
-// built, from static layer data, before the wait for the previous kernel.
+// 8192: 49 -> 37 us; K = 13824, M = 2048: 48 -> 31 us (cold cache).  16-byte
+// pieces of RW words lie in planes, so that the staging stores of a warp are
+// contiguous; the slot map holds positions in that layout and is built, from
+// static layer data, before the wait for the previous kernel.
 constexpr int kRowsThreads = 512;
 constexpr int kRowsMaxK = 65520;  // staged positions and the zero word fit 16 bits
 

@@ -146,3 +146,30 @@ def test_gemm_token_tile_edges(polyq_lib, M, N, K, seed):
     assert polyq_lib.workspace_status(ws[-256:]) == 0
     ref = O.pack_layer(W, a, 3.0, bits=bits)
     check_tolerance(Y.cpu().numpy(), O.linear(ref, X), X, K)
+
+
+# One shape on each side of every line of the pre-pass's dispatch (rows, and the
+# shared memory that a staged row takes).
+PREP_EDGES = [
+    (256, 40, 32768, 66),   # most rows and widest row of the pre-pass of a few rows
+    (257, 40, 3003, 67),    # two rows at a time, ragged K
+    (257, 40, 20011, 68),   # rows too wide for two at a time
+    (1, 40, 32769, 69),     # a single row, staged by the pre-pass of many
+    (1281, 40, 2049, 70),   # four rows at a time
+    (1281, 40, 16008, 71),  # enough rows for four at a time, which do not fit
+    (3, 40, 70001, 72),     # not staged
+]
+
+
+@pytest.mark.parametrize("M,N,K,seed", PREP_EDGES)
+def test_gemm_prepass_edges(polyq_lib, M, N, K, seed):
+    W, a = synth.layer_weights(N, K, seed)
+    bits = synth.random_codes_layer_bits(K, seed)
+    Xb, X = synth.activations(a, M, seed)
+    dev = polyq_lib.DeviceLayer(polyq_lib.HostLayer.pack(W, a, 3.0, forced_bits=bits), "cuda")
+    ws = torch.full((polyq_lib.gemm_workspace_bytes(dev, M),), 255, dtype=torch.uint8,
+                    device="cuda")
+    Y = polyq_lib.linear_gemm(dev, _x_dev(Xb), workspace=ws)
+    torch.cuda.synchronize()
+    assert polyq_lib.workspace_status(ws[-256:]) == 0
+    check_tolerance(Y.cpu().numpy(), O.linear(O.pack_layer(W, a, 3.0, bits=bits), X), X, K)

@@ -102,3 +102,21 @@ def test_scaled_gemm_matches_oracle(polyq_lib, M, N, K, seed, forced):
     Y = polyq_lib.linear_gemm(dev, _x_dev(Xb))
     torch.cuda.synchronize()
     check_tolerance(Y.cpu().numpy(), O.linear_scaled(ref, X), X, K)
+
+
+@pytest.mark.parametrize("M,N,K,seed", [
+    (256, 40, 3005, 64),    # the pre-pass of a few rows
+    (257, 40, 2999, 65),    # two rows at a time
+    (257, 40, 14003, 66),   # one row at a time
+    (1281, 40, 1030, 67),   # four rows at a time
+    (5, 40, 40001, 68),     # not staged
+])
+def test_scaled_gemm_prepass_edges(polyq_lib, M, N, K, seed):
+    """One shape for each kernel that the pre-pass of a scaled layer may take."""
+    W, a = synth.layer_weights(N, K, seed)
+    host, ref = _scaled_pair(polyq_lib, W, a, 3.0, synth.random_codes_layer_bits(K, seed))
+    dev = polyq_lib.DeviceLayer(host, "cuda")
+    Xb, X = synth.activations(a, M, seed)
+    Y = polyq_lib.linear_gemm(dev, _x_dev(Xb))
+    torch.cuda.synchronize()
+    check_tolerance(Y.cpu().numpy(), O.linear_scaled(ref, X), X, K)
