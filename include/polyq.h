@@ -427,7 +427,7 @@ int polyq_linear_gemv_input(const polyq_dev_layer* const* layers, int n,
  * CTAs meet at a grid-wide barrier (phase p+1 reads what phase p wrote),
  * then build the phase's activation records in the workspace, one per CTA.
  * Work items of a phase are (layer, 64-row tile, step) in tile-major order,
- * split into contiguous ranges of equal modelled cost; each tile piece adds
+ * split into contiguous ranges of equal length; each tile piece adds
  * its rows into y with fp32 atomics (the order of those additions varies
  * from run to run).  Every device-side wait is bounded; on a timeout the
  * kernel records a status and returns. */
@@ -460,7 +460,7 @@ int polyq_gemv_chain_create(const polyq_gemv_phase* phases, int n_phases, int ba
                             polyq_gemv_chain** out);
 
 /* Bytes of device memory the chain's plan needs (tensor maps, block tables
- * and per-CTA work ranges for the current device). */
+ * and work shares for the current device). */
 /* Bytes of the workspace a launch of the chain needs: a status word, the
  * grid-barrier and launch counters, one record-ready counter per phase and
  * the activation records of the largest phase. */

@@ -10,17 +10,19 @@
 //    (a per-phase counter in the workspace).
 //  * Warps 0-3 (16 rows each) run the phases in order.  A grid-wide barrier
 //    (an arrival counter) separates phases, because phase p+1 reads what
-//    phase p wrote.  After it, CTA b builds record b (b+G, ...) of the phase
+//    phase p wrote.  After it (in the first phase, at once), CTA b builds record b (b+G, ...) of the phase
 //    into the workspace: gather, transform (RMSNorm, SiLU * up, rounding to
 //    bf16), activation factor, fp16 rounding, per-chunk sums.  The warps then
 //    set the next phase's outputs to its residual (or zero) and decode and
 //    multiply their items exactly as the per-call kernel does, adding each
 //    tile piece's rows into y with fp32 atomics.
 // Items of a phase are (layer, tile, step) in tile-major order, split into
-// contiguous ranges of equal modelled cost, so each CTA streams the rows of
-// a few tiles from start to end.  Every wait is bounded; a wait that gives
-// up records a status, makes the CTA skip the rest, waits (bounded) for its
-// own copies in flight and returns.
+// contiguous ranges of equal length, so each CTA streams the rows of a few
+// tiles from start to end.  (At batch 1 an item takes 0.6 to 0.8 us whatever
+// its width; ranges of equal bytes had the last CTA of q/k/v 8 us behind the
+// median one, these 5.)  Every wait is bounded; a wait that gives up records a
+// status, makes the CTA skip the rest, waits (bounded) for its own copies in
+// flight and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -48,7 +50,6 @@ constexpr int kChMaxGrid = 1024;
 // sleeps at least 128-256 ns and reads L2): about a second, against waits of
 // microseconds in a working launch.
 constexpr uint32_t kGridWaitLimit = 1u << 21;
-constexpr int kItemFixedCost = 2048;  // per-item overhead in the cost model, bytes
 // workspace: status word at 0; barrier arrivals, CTAs done and the launch
 // count at 64; per-phase record-ready counters from 256; then the records
 constexpr size_t kWsCounters = 64;
@@ -70,6 +71,7 @@ struct ChPhase {
   ChLayer L[POLYQ_MAX_GROUP];
   int n_layers, items, recs, kind;
   float eps;
+  int share, extra;  // items of a CTA, and the CTAs that take one more
   int pad0;
   const float* xa;
   const float* xb;
@@ -78,8 +80,8 @@ struct ChPhase {
 
 struct ChParams {
   const ChPhase* ph;
-  const int* ranges;  // [n_phases][gridDim.x + 1] item boundaries
   int n_phases, batch;
+  int init0;  // CTAs that initialise the first phase's outputs
   uint32_t magic;
   int* status;
   unsigned int* bar;    // [0] barrier arrivals, [1] CTAs done, [2] launches completed
@@ -178,17 +180,26 @@ __device__ __forceinline__ XIn chain_xin(const ChShared& S, int l, int batch) {
   return in;
 }
 
-// Outputs of a phase start as the residual (or zero); grid-stride over all
-// consumer threads of the launch.
-__device__ void init_outputs(const ChPhase* ph, int batch) {
+// The items [lo, hi) of this CTA in a phase.  (With the one more that some take
+// going to the last CTAs, which build no record, the 13B-shaped layer took 0.3
+// us longer.)
+__device__ __forceinline__ void item_range(const ChPhase* ph, int* lo, int* hi) {
+  const int b = blockIdx.x, share = ph->share, extra = ph->extra;
+  *lo = b * share + min(b, extra);
+  *hi = *lo + share + (b < extra ? 1 : 0);
+}
+
+// Outputs of a phase start as the residual (or zero): the share of the
+// consumer threads of CTA `cta` of `n_cta`.
+__device__ void init_outputs(const ChPhase* ph, int batch, int cta, int n_cta) {
   const int nl = ph->n_layers;
-  const int stride = gridDim.x * kConsumers;
+  const int stride = n_cta * kConsumers;
   for (int l = 0; l < nl; ++l) {
     float* y = ph->L[l].y;
     const float* res = ph->L[l].residual;
     if (y == res) continue;
     const int total = batch * ph->L[l].N;
-    for (int i = blockIdx.x * kConsumers + threadIdx.x; i < total; i += stride)
+    for (int i = cta * kConsumers + threadIdx.x; i < total; i += stride)
       y[i] = res ? __ldcg(res + i) : 0.f;
   }
 }
@@ -236,9 +247,9 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
     const uint8_t* rsrc[kStages]; // record source of each pending item, by slot
     int rphase[kStages];
     auto wait_ready = [&](int p) -> bool {
-      // the counter grows by recs per launch and wraps after 2^32 / recs
-      // launches: compare by signed difference
-      const unsigned target = (epoch + 1u) * (unsigned)P.ph[p].recs;
+      // the counter grows by recs (and for the first phase init0) per launch
+      // and wraps: compare by signed difference
+      const unsigned target = (epoch + 1u) * (unsigned)(P.ph[p].recs + (p == 0 ? P.init0 : 0));
       uint32_t it = 0;
       while ((int)(target - ld_acquire_gpu(P.ready + p)) > 0) {
         if (++it > kGridWaitLimit || s_abort) return false;
@@ -267,8 +278,8 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
     bool go = true;
     for (int p = 0; p < P.n_phases && go; ++p) {
       const ChPhase* ph = P.ph + p;
-      const int lo = __ldg(P.ranges + p * (G + 1) + blockIdx.x);
-      const int hi = __ldg(P.ranges + p * (G + 1) + blockIdx.x + 1);
+      int lo, hi;
+      item_range(ph, &lo, &hi);
       if (lo >= hi) continue;
       const int nl = ph->n_layers;
       for (int q = 0; q < nl; ++q) {
@@ -431,32 +442,38 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
     if (blockIdx.x < S.recs) record_of(blockIdx.x);
   };
 
-  init_outputs(P.ph, P.batch);
-  grid_arrive();
+  // No barrier before the first phase: its inputs are complete, and its outputs
+  // are initialised by CTAs that its record counter waits for too (the last
+  // ones, which build no record unless there is one for every CTA).  The first
+  // stage is complete 8.5 us after the launch instead of 10.5.
+  const int init_i = G - 1 - (int)blockIdx.x;
+  if (init_i < P.init0) init_outputs(P.ph, P.batch, init_i, P.init0);
   prepare(0);
-  bool alive = grid_wait();
+  bool alive = true;
   for (int p = 0; p < P.n_phases && alive; ++p) {
     // this CTA's share of the phase's records (the inputs are complete)
-    if (blockIdx.x < S.recs) {
-      if (S.kind == POLYQ_X_RMSNORM) rms_rnorm(S.xa, S.K[0], P.batch, S.eps, s_part, s_rnorm);
+    const bool init = p == 0 && init_i < P.init0;
+    if (blockIdx.x < S.recs || init) {
       int built = 0;
 #pragma unroll 1
       for (int f = blockIdx.x; f < S.recs; f += G, ++built) {
         if (built) record_of(f);
         float ra[R.N][2], rb[R.N][2];
         rec_load(in, R, ra, rb);
+        if (built == 0 && S.kind == POLYQ_X_RMSNORM)  // its reads overlap the record's
+          rms_rnorm(S.xa, S.K[0], P.batch, S.eps, s_part, s_rnorm);
         rec_store<NB>(in, rec_bits, warp, lane, R, ra, rb, s_rnorm,
                       reinterpret_cast<uint32_t*>(P.rec + (size_t)f * RB));
       }
       consumer_sync();
       if (threadIdx.x == 0) {
         __threadfence();
-        atomicAdd(P.ready + p, (unsigned)built);
+        atomicAdd(P.ready + p, (unsigned)(built + init));
       }
     }
-    if (p + 1 < P.n_phases) init_outputs(P.ph + p + 1, P.batch);
-    const int lo = __ldg(P.ranges + p * (G + 1) + blockIdx.x);
-    const int hi = __ldg(P.ranges + p * (G + 1) + blockIdx.x + 1);
+    if (p + 1 < P.n_phases) init_outputs(P.ph + p + 1, P.batch, blockIdx.x, G);
+    int lo, hi;
+    item_range(P.ph + p, &lo, &hi);
     for (int it = lo; it < hi; ++it) {
       bool ok = false;
       for (uint32_t w = 0; w < kWaitLimit && !s_abort; ++w)
@@ -536,9 +553,9 @@ Span span(const void* p, size_t bytes) {
 
 struct polyq_gemv_chain {
   int n_phases = 0, batch = 0, nb = 1, grid = 0;
+  int init0 = 0;
   std::vector<ChPhase> ph;
-  std::vector<int> ranges;
-  size_t ranges_off = 0, plan_bytes = 0;
+  size_t plan_bytes = 0;
   size_t rec_off = 0, ws_bytes = 0;  // workspace: records region, total
   void* plan_dev = nullptr;
 };
@@ -651,33 +668,6 @@ int fill_phase(const polyq_gemv_phase& P, int nb, ChPhase* C) {
   return POLYQ_OK;
 }
 
-// Contiguous item ranges of equal modelled cost (bytes streamed plus a fixed
-// per-item cost) for `grid` CTAs; items are (layer, tile, step) tile-major.
-void split_phase(const ChPhase& C, int nb, int grid, int* out) {
-  std::vector<long long> prefix(1, 0);  // cost of items [0, i)
-  prefix.reserve((size_t)C.items + 1);
-  for (int l = 0; l < C.n_layers; ++l) {
-    const ChLayer& L = C.L[l];
-    std::vector<long long> per;
-    for (int b = 0; b < L.n_blocks; ++b) {
-      const GvBlock& B = L.blk[b];
-      const long long c = (long long)kRows * step_bytes(B.bits, nb) +
-                          (B.bits < 16 ? kRows * 4LL * (B.units / 64) : 0) + kItemFixedCost;
-      for (int j = 0; j < B.n_steps; ++j) per.push_back(c);
-    }
-    for (int t = 0; t < L.tiles; ++t)
-      for (long long c : per) prefix.push_back(prefix.back() + c);
-  }
-  const long long total = prefix.back();
-  int item = 0;
-  for (int b = 0; b <= grid; ++b) {
-    const long long goal = (long long)((__int128)total * b / grid);
-    while (item < C.items && prefix[item + 1] <= goal) ++item;
-    out[b] = item;
-  }
-  out[grid] = C.items;
-}
-
 template <int NB>
 int launch_chain(const polyq_gemv_chain* ch, void* ws, cudaStream_t st) {
   static bool attr_done[64] = {false};
@@ -699,9 +689,9 @@ int launch_chain(const polyq_gemv_chain* ch, void* ws, cudaStream_t st) {
   }
   ChParams P;
   P.ph = static_cast<const ChPhase*>(ch->plan_dev);
-  P.ranges = reinterpret_cast<const int*>(static_cast<const char*>(ch->plan_dev) + ch->ranges_off);
   P.n_phases = ch->n_phases;
   P.batch = ch->batch;
+  P.init0 = ch->init0;
   P.magic = kMagic;
   P.status = static_cast<int*>(ws);
   P.bar = reinterpret_cast<unsigned int*>(static_cast<char*>(ws) + kWsCounters);
@@ -778,7 +768,6 @@ extern "C" int polyq_gemv_chain_create(const polyq_gemv_phase* phases, int n_pha
     ch->nb = nb_of_batch(batch);
     ch->grid = std::max(1, std::min(kChCtasPerSm * sms, kChMaxGrid));
     ch->ph.resize(n_phases);
-    ch->ranges.assign((size_t)n_phases * (ch->grid + 1), 0);
     for (int p = 0; p < n_phases; ++p) {
       rc = fill_phase(phases[p], ch->nb, &ch->ph[p]);
       if (rc) {
@@ -789,14 +778,18 @@ extern "C" int polyq_gemv_chain_create(const polyq_gemv_phase* phases, int n_pha
         delete ch;
         return polyq_set_error(POLYQ_EUNSUPPORTED, "%s: phase %d has too many items", who, p);
       }
-      split_phase(ch->ph[p], ch->nb, ch->grid, ch->ranges.data() + (size_t)p * (ch->grid + 1));
+      ch->ph[p].share = ch->ph[p].items / ch->grid;
+      ch->ph[p].extra = ch->ph[p].items % ch->grid;
     }
   } catch (const std::bad_alloc&) {
     delete ch;
     return polyq_set_error(POLYQ_ENOMEM, "%s: out of host memory", who);
   }
-  ch->ranges_off = (size_t)n_phases * sizeof(ChPhase);
-  ch->plan_bytes = ch->ranges_off + ch->ranges.size() * sizeof(int);
+  ch->plan_bytes = (size_t)n_phases * sizeof(ChPhase);
+  int64_t out0 = 0;  // four outputs per thread
+  for (int i = 0; i < phases[0].n_layers; ++i)
+    if (phases[0].residuals[i] != phases[0].ys[i]) out0 += (int64_t)batch * phases[0].layers[i]->N;
+  ch->init0 = (int)std::min<int64_t>(ch->grid, (out0 + 4 * kConsumers - 1) / (4 * kConsumers));
   int max_recs = 0;
   for (const ChPhase& c : ch->ph) max_recs = std::max(max_recs, c.recs);
   ch->rec_off = (kWsReady + 4 * (size_t)n_phases + 255) / 256 * 256;
@@ -832,14 +825,11 @@ extern "C" int polyq_gemv_chain_upload(polyq_gemv_chain* ch, void* plan_dev, siz
     return polyq_set_error(POLYQ_EINVAL, "%s: plan memory must be %zu-byte aligned", who,
                            alignof(ChPhase));
   cudaStream_t st = (cudaStream_t)stream;
-  cudaError_t e = cudaMemcpyAsync(plan_dev, ch->ph.data(), ch->ranges_off,
+  cudaError_t e = cudaMemcpyAsync(plan_dev, ch->ph.data(), ch->plan_bytes,
                                   cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyAsync(static_cast<char*>(plan_dev) + ch->ranges_off, ch->ranges.data(),
-                        ch->ranges.size() * sizeof(int), cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess)
     return polyq_set_error(POLYQ_ECUDA, "%s: copy: %s", who, cudaGetErrorString(e));
-  // the host plan must outlive the asynchronous copies from pageable memory
+  // the host plan must outlive the asynchronous copy from pageable memory
   e = cudaStreamSynchronize(st);
   if (e != cudaSuccess)
     return polyq_set_error(POLYQ_ECUDA, "%s: %s", who, cudaGetErrorString(e));
