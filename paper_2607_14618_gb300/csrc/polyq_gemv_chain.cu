@@ -242,10 +242,10 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
     // records are all built (a counter per phase, summed over launches).
     if (!elect_one()) return;
     const unsigned epoch = s_epoch;
-    int kg = 0, kr = 0;           // items whose weights / records were issued
+    int kg = 0, kr = 0;           // stages whose weights / records were issued
     int ready_phase = -1;         // phases whose records are known to be built
-    const uint8_t* rsrc[kStages]; // record source of each pending item, by slot
-    int rphase[kStages];
+    const uint8_t* rsrc[kStages]; // record source of each pending stage, by slot
+    int rphase[kStages], rbytes[kStages];
     auto wait_ready = [&](int p) -> bool {
       // the counter grows by recs (and for the first phase init0) per launch
       // and wraps: compare by signed difference
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
       fence_proxy_async_global();  // the builders wrote through the generic proxy
       return true;
     };
-    // issue the records of items kr..upto (blocking until their phases are built)
+    // issue the records of stages kr..upto (blocking until their phases are built)
     auto issue_records = [&](int upto) -> bool {
       while (kr <= upto) {
         const int sl = kr % kStages;
@@ -270,7 +270,7 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
           }
           ready_phase = rphase[sl];
         }
-        bulk_load(smem_u32(stages + sl * kStageBytes + kRecOff), rsrc[sl], RB, full0 + 8 * sl);
+        bulk_load(smem_u32(stages + sl * kStageBytes + kRecOff), rsrc[sl], rbytes[sl], full0 + 8 * sl);
         ++kr;
       }
       return true;
@@ -286,28 +286,34 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
         for (int b = 0; b < ph->L[q].n_blocks; ++b) tmap_acquire(&ph->L[q].tm_codes[b]);
         tmap_acquire(&ph->L[q].tm_meta);
       }
-      // position of item lo: layer, tile, step (tile-major)
+      // position of item lo: layer, tile, block, step (tile-major); it and the
+      // block's table stay in registers from item to item
       int l = 0;
       while (l + 1 < nl && lo >= ph->L[l + 1].item0) ++l;
-      int steps = ph->L[l].steps;
-      int tile = (lo - ph->L[l].item0) / steps;
-      int s = lo - ph->L[l].item0 - tile * steps;
-      for (int it = lo; it < hi && go; ++it) {
+      const ChLayer* L = &ph->L[l];
+      int tile = (lo - L->item0) / L->steps, bi = 0;
+      int j = lo - L->item0 - tile * L->steps;
+      while (bi + 1 < L->n_blocks && j >= L->blk[bi + 1].step0) ++bi;
+      GvBlock B = L->blk[bi];
+      j -= B.step0;
+      for (int it = lo; it < hi && go;) {
         const int slot = kg % kStages;
         if (kg >= kStages) {
-          // the consumers free this stage only after the item it holds, so
-          // that item's record goes first
+          // the consumers free this stage only after the items it holds, so
+          // their records go first
           if (!issue_records(kg - kStages)) {
             go = false;
             break;
           }
           const uint32_t bar = empty0 + 8 * slot, par = ((kg / kStages) - 1) & 1;
           bool ok = false;
-          for (uint32_t w = 0; w < kWaitLimit && !s_abort; ++w)
+          for (uint32_t w = 0; w < kWaitLimit; ++w) {
             if (mbar_try_wait(bar, par)) {
               ok = true;
               break;
             }
+            if (s_abort) break;
+          }
           if (!ok) {
             if (!s_abort) atomicExch(P.status, kStatusTimeoutEmpty);
             s_abort = 1;
@@ -315,12 +321,6 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
             break;
           }
         }
-        const ChLayer& L = ph->L[l];
-        int bi = 0;
-        while (bi + 1 < L.n_blocks && s >= L.blk[bi + 1].step0) ++bi;
-        const GvBlock B = L.blk[bi];
-        const int j = s - B.step0;
-        const bool flush = s == steps - 1 || it == hi - 1;
         int sb, nbx, pitch;
         switch (B.bits) {
           case 2: sb = step_bytes(2, NB); nbx = nbox_of(2, NB); pitch = box_pitch(2, NB); break;
@@ -329,30 +329,40 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
           case 8: sb = step_bytes(8, NB); nbx = nbox_of(8, NB); pitch = box_pitch(8, NB); break;
           default: sb = step_bytes(16, NB); nbx = nbox_of(16, NB); pitch = box_pitch(16, NB); break;
         }
+        // batch 2-4: two consecutive steps of a block and tile whose codes take
+        // one box each share a stage, as in the per-call kernel
+        const bool pair = NB > 1 && nbx == 1 && it + 1 < hi && j + 1 < B.n_steps;
+        const int n = pair ? 2 : 1;
         uint8_t* st = stages + slot * kStageBytes;
         const uint32_t dst = smem_u32(st);
         const uint32_t bar = full0 + 8 * slot;
         {
+          const bool last = j + n == B.n_steps && bi + 1 == L->n_blocks;  // of the tile
           const int uvalid = min(B.units, B.n_ch - j * B.units);
           const int g0 = (B.grp_off + j * (B.units / 64)) & 3;
           uint4 d;
-          d.x = (uint32_t)B.bits | ((uint32_t)flush << 8) | ((uint32_t)l << 16);
+          d.x = (uint32_t)B.bits | ((uint32_t)(last || it + n == hi) << 8) |
+                ((uint32_t)pair << 10) | ((uint32_t)l << 16);
           d.y = (uint32_t)uvalid | ((uint32_t)g0 << 16);
           d.z = (uint32_t)tile;
           d.w = 0u;
           *reinterpret_cast<uint4*>(st + kDescOff) = d;
         }
-        uint32_t bytes = nbx * pitch * kRows + RB;
+        uint32_t bytes = n * (nbx * pitch * kRows + RB);
         if (B.bits < 16) bytes += kMetaBytes;
         mbar_expect_tx(bar, bytes);
         for (int h = 0; h < nbx; ++h)
-          tma_load_2d(dst + h * kRows * pitch, &L.tm_codes[bi], B.seg_off + j * sb + h * (sb / nbx),
+          tma_load_2d(dst + h * kRows * pitch, &L->tm_codes[bi], B.seg_off + j * sb + h * (sb / nbx),
                       tile * kRows, bar);
-        if (B.bits < 16) {
+        if (pair)
+          tma_load_2d(dst + kRows * pitch, &L->tm_codes[bi], B.seg_off + (j + 1) * sb, tile * kRows,
+                      bar);
+        if (B.bits < 16) {  // one box of kMetaBox groups covers both steps of a pair
           const int x0 = (B.grp_off + j * (B.units / 64)) & ~3;
-          tma_load_2d(dst + kCodesBytes, &L.tm_meta, x0, tile * kRows, bar);
+          tma_load_2d(dst + kCodesBytes, &L->tm_meta, x0, tile * kRows, bar);
         }
-        rsrc[slot] = P.rec + (size_t)(L.rec0 + s) * RB;
+        rsrc[slot] = P.rec + (size_t)(L->rec0 + B.step0 + j) * RB;
+        rbytes[slot] = n * RB;  // consecutive records
         rphase[slot] = p;
         ++kg;
         if (p <= ready_phase && !issue_records(kg - 1)) {
@@ -360,12 +370,18 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
           break;
         }
         // next item
-        if (++s == steps) {
-          s = 0;
-          if (++tile == L.tiles) {
-            tile = 0;
-            if (++l < nl) steps = ph->L[l].steps;
+        it += n;
+        j += n;
+        if (j == B.n_steps && it < hi) {
+          j = 0;
+          if (++bi == L->n_blocks) {
+            bi = 0;
+            if (++tile == L->tiles) {
+              tile = 0;
+              L = &ph->L[++l];
+            }
           }
+          B = L->blk[bi];
         }
       }
     }
@@ -375,7 +391,7 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
     // wait (bounded) for the copies in flight before leaving.
     for (; kr < kg; ++kr) {
       const int sl = kr % kStages;
-      bulk_load(smem_u32(stages + sl * kStageBytes + kRecOff), rsrc[sl], RB, full0 + 8 * sl);
+      bulk_load(smem_u32(stages + sl * kStageBytes + kRecOff), rsrc[sl], rbytes[sl], full0 + 8 * sl);
     }
     for (int k = max(0, kg - kStages); k < kg; ++k)
       mbar_wait(full0 + 8 * (k % kStages), (k / kStages) & 1);
@@ -474,37 +490,53 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
     if (p + 1 < P.n_phases) init_outputs(P.ph + p + 1, P.batch, blockIdx.x, G);
     int lo, hi;
     item_range(P.ph + p, &lo, &hi);
-    for (int it = lo; it < hi; ++it) {
+    for (int it = lo; it < hi;) {
       bool ok = false;
-      for (uint32_t w = 0; w < kWaitLimit && !s_abort; ++w)
+      for (uint32_t w = 0; w < kWaitLimit; ++w) {
         if (mbar_try_wait(full0 + 8 * slot, phase)) {
           ok = true;
           break;
         }
-      if (!ok && !s_abort) {
-        if (lane == 0) atomicExch(P.status, kStatusTimeoutFull);
-        s_abort = 1;
+        if (s_abort) break;
       }
-      if (ok) {
-        const uint8_t* stage = stages + slot * kStageBytes;
-        const uint32_t* rec = reinterpret_cast<const uint32_t*>(stage + kRecOff);
-        const uint4 desc = *reinterpret_cast<const uint4*>(stage + kDescOff);
-        const int bits = (int)(desc.x & 0xFFu);
-        const int uvalid = (int)(desc.y & 0xFFFFu), g0 = (int)(desc.y >> 16);
-        switch (bits) {
-          case 2: step_mma<NB, 2>(P.magic, P.batch, uvalid, g0, stage, stage, rec, zeros, warp, lane, acc); break;
-          case 3: step_mma<NB, 3>(P.magic, P.batch, uvalid, g0, stage, stage, rec, zeros, warp, lane, acc); break;
-          case 4: step_mma<NB, 4>(P.magic, P.batch, uvalid, g0, stage, stage, rec, zeros, warp, lane, acc); break;
-          case 8: step_mma<NB, 8>(P.magic, P.batch, uvalid, g0, stage, stage, rec, zeros, warp, lane, acc); break;
-          default: step_16<NB>(P.batch, uvalid, stage, rec, zeros, warp, lane, acc); break;
+      if (!__all_sync(0xffffffffu, ok)) {  // one decision for the warp
+        if (!s_abort && lane == 0) atomicExch(P.status, kStatusTimeoutFull);
+        s_abort = 1;
+        break;
+      }
+      const uint8_t* stage = stages + slot * kStageBytes;
+      const uint32_t* rec = reinterpret_cast<const uint32_t*>(stage + kRecOff);
+      const uint4 desc = *reinterpret_cast<const uint4*>(stage + kDescOff);
+      const int bits = (int)(desc.x & 0xFFu);
+      const int uvalid = (int)(desc.y & 0xFFFFu), g0 = (int)(desc.y >> 16);
+      const bool pair = NB > 1 && (desc.x & 0x400u);
+      it += pair ? 2 : 1;
+      if (pair) {
+        if constexpr (NB > 1) {
+          const uint32_t* rec2 = rec + RB / 4;
+          switch (bits) {
+            case 2: step_mma_pair<NB, 2>(P.magic, P.batch, g0, stage, stage + kRows * box_pitch(2, NB), stage, rec, rec2, zeros, warp, lane, acc); break;
+            case 3: step_mma_pair<NB, 3>(P.magic, P.batch, g0, stage, stage + kRows * box_pitch(3, NB), stage, rec, rec2, zeros, warp, lane, acc); break;
+            case 4: step_mma_pair<NB, 4>(P.magic, P.batch, g0, stage, stage + kRows * box_pitch(4, NB), stage, rec, rec2, zeros, warp, lane, acc); break;
+            default:
+              if constexpr (nbox_of(8, NB) == 1)
+                step_mma_pair<NB, 8>(P.magic, P.batch, g0, stage, stage + kRows * box_pitch(8, NB), stage, rec, rec2, zeros, warp, lane, acc);
+              break;
+          }
         }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(empty0 + 8 * slot);
-        if (desc.x & 0x100u) {
-          // add this warp's 16 rows of the tile piece into y
-          const int l = (int)(desc.x >> 16);
-          flush_rows<NB>(acc, S.y[l], S.N[l], P.batch, (int)desc.z * kRows + warp * 16, lane);
-        }
+      } else switch (bits) {
+        case 2: step_mma<NB, 2>(P.magic, P.batch, uvalid, g0, stage, stage, rec, zeros, warp, lane, acc); break;
+        case 3: step_mma<NB, 3>(P.magic, P.batch, uvalid, g0, stage, stage, rec, zeros, warp, lane, acc); break;
+        case 4: step_mma<NB, 4>(P.magic, P.batch, uvalid, g0, stage, stage, rec, zeros, warp, lane, acc); break;
+        case 8: step_mma<NB, 8>(P.magic, P.batch, uvalid, g0, stage, stage, rec, zeros, warp, lane, acc); break;
+        default: step_16<NB>(P.batch, uvalid, stage, rec, zeros, warp, lane, acc); break;
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(empty0 + 8 * slot);
+      if (desc.x & 0x100u) {
+        // add this warp's 16 rows of the tile piece into y
+        const int l = (int)(desc.x >> 16);
+        flush_rows<NB>(acc, S.y[l], S.N[l], P.batch, (int)desc.z * kRows + warp * 16, lane);
       }
       if (++slot == kStages) {
         slot = 0;

@@ -156,6 +156,29 @@ def test_independent_phases_match_oracle(polyq_lib, batch):
             check_tolerance(ys[name].cpu().numpy(), ref, xs[name][1], K)
 
 
+@pytest.mark.parametrize("batch", [2, 3, 4])
+def test_ranges_of_paired_steps(polyq_lib, batch):
+    """More items than CTAs, over two phases: a CTA's range starts and ends
+    inside the pairs of steps that share a stage at batch 2 to 4, in blocks of
+    all five widths with odd step counts and a ragged end."""
+    phases, want = [], []
+    for N, K, seed in ((5000, 1231, 3300), (2500, 3001, 3301)):
+        W, a = synth.layer_weights(N, K, seed)
+        bits = synth.random_codes_layer_bits(K, seed)
+        dev = polyq_lib.DeviceLayer(polyq_lib.HostLayer.pack(W, a, 3.0, forced_bits=bits), "cuda")
+        xb, x = synth.activations(a, batch, seed)
+        y = torch.full((batch, N), float("nan"), device="cuda")
+        phases.append(dict(layers=[dev], kind=polyq_lib.X_BF16, a=_x_dev(xb), ys=[y]))
+        want.append((y, O.linear(O.pack_layer(W, a, 3.0, bits=bits), x), x, K))
+    chain = polyq_lib.GemvChain(phases, batch=batch)
+    for _ in range(2):
+        chain.run()
+        torch.cuda.synchronize()
+        assert polyq_lib.workspace_status(chain.workspace) == 0
+        for y, ref, x, K in want:
+            check_tolerance(y.cpu().numpy(), ref, x, K)
+
+
 def test_phase_with_more_records_than_ctas(polyq_lib):
     # Four layers of 48 rows (one partial tile each) over K = 65536 channels
     # of all five widths at batch 4: 2048 records, so every CTA builds
