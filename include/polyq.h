@@ -427,7 +427,8 @@ int polyq_linear_gemv_input(const polyq_dev_layer* const* layers, int n,
  * CTAs meet at a grid-wide barrier (phase p+1 reads what phase p wrote),
  * then build the phase's activation records in the workspace, one per CTA.
  * Work items of a phase are (layer, 64-row tile, step) in tile-major order,
- * split into contiguous ranges of equal length; each tile piece adds
+ * split into contiguous ranges of equal length, with an eighth of a larger
+ * phase left in a pool that CTAs take from as they go; each tile piece adds
  * its rows into y with fp32 atomics (the order of those additions varies
  * from run to run).  Every device-side wait is bounded; on a timeout the
  * kernel records a status and returns. */

@@ -10,19 +10,19 @@
 //    (a per-phase counter in the workspace).
 //  * Warps 0-3 (16 rows each) run the phases in order.  A grid-wide barrier
 //    (an arrival counter) separates phases, because phase p+1 reads what
-//    phase p wrote.  After it (in the first phase, at once), CTA b builds record b (b+G, ...) of the phase
-//    into the workspace: gather, transform (RMSNorm, SiLU * up, rounding to
+//    phase p wrote.  After it (in the first phase, at once), CTA b
+//    builds record b (b+G, ...) of the phase into the workspace: gather, transform (RMSNorm, SiLU * up, rounding to
 //    bf16), activation factor, fp16 rounding, per-chunk sums.  The warps then
 //    set the next phase's outputs to its residual (or zero) and decode and
 //    multiply their items exactly as the per-call kernel does, adding each
 //    tile piece's rows into y with fp32 atomics.
-// Items of a phase are (layer, tile, step) in tile-major order, split into
-// contiguous ranges of equal length, so each CTA streams the rows of a few
-// tiles from start to end.  (At batch 1 an item takes 0.6 to 0.8 us whatever
-// its width; ranges of equal bytes had the last CTA of q/k/v 8 us behind the
-// median one, these 5.)  Every wait is bounded; a wait that gives up records a
-// status, makes the CTA skip the rest, waits (bounded) for its own copies in
-// flight and returns.
+// Items of a phase are (layer, tile, step) in tile-major order.  Each CTA takes
+// a contiguous range of equal length, so it streams the rows of a few tiles
+// from start to end, and then pieces of a pool (see share_out).  (At batch 1 an
+// item takes 0.6 to 0.8 us whatever its width; ranges of equal bytes had the
+// last CTA of q/k/v 8 us behind the median one, equal lengths 5.)  Every wait
+// is bounded; a wait that gives up records a status, makes the CTA skip the
+// rest, waits (bounded) for its own copies in flight and returns.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -51,7 +51,8 @@ constexpr int kChMaxGrid = 1024;
 // microseconds in a working launch.
 constexpr uint32_t kGridWaitLimit = 1u << 21;
 // workspace: status word at 0; barrier arrivals, CTAs done and the launch
-// count at 64; per-phase record-ready counters from 256; then the records
+// count at 64; per-phase record-ready and pool counters from 256; then the
+// records
 constexpr size_t kWsCounters = 64;
 constexpr size_t kWsReady = 256;
 
@@ -71,8 +72,9 @@ struct ChPhase {
   ChLayer L[POLYQ_MAX_GROUP];
   int n_layers, items, recs, kind;
   float eps;
-  int share, extra;  // items of a CTA, and the CTAs that take one more
-  int pad0;
+  int share;   // items that every CTA takes, in order
+  int extra;   // no pool: the first CTAs that take one more
+  int chunks;  // else pieces of the pool, the items from gridDim * share on
   const float* xa;
   const float* xb;
   uint16_t* xout;
@@ -86,6 +88,7 @@ struct ChParams {
   int* status;
   unsigned int* bar;    // [0] barrier arrivals, [1] CTAs done, [2] launches completed
   unsigned int* ready;  // [n_phases] records built, summed over launches
+  unsigned int* pool;   // [n_phases] pool pieces asked for, summed over launches
   uint8_t* rec;         // records of the current phase
 };
 
@@ -180,14 +183,14 @@ __device__ __forceinline__ XIn chain_xin(const ChShared& S, int l, int batch) {
   return in;
 }
 
-// The items [lo, hi) of this CTA in a phase.  (With the one more that some take
-// going to the last CTAs, which build no record, the 13B-shaped layer took 0.3
-// us longer.)
+// The items [lo, hi) that this CTA takes in a phase without asking.
 __device__ __forceinline__ void item_range(const ChPhase* ph, int* lo, int* hi) {
   const int b = blockIdx.x, share = ph->share, extra = ph->extra;
   *lo = b * share + min(b, extra);
   *hi = *lo + share + (b < extra ? 1 : 0);
 }
+// Items per piece of a phase's pool: what one stage holds.
+__host__ __device__ constexpr int chunk_items(int nb) { return nb == 1 ? 1 : 2; }
 
 // Outputs of a phase start as the residual (or zero): the share of the
 // consumer threads of CTA `cta` of `n_cta`.
@@ -286,17 +289,30 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
         for (int b = 0; b < ph->L[q].n_blocks; ++b) tmap_acquire(&ph->L[q].tm_codes[b]);
         tmap_acquire(&ph->L[q].tm_meta);
       }
-      // position of item lo: layer, tile, block, step (tile-major); it and the
-      // block's table stay in registers from item to item
-      int l = 0;
-      while (l + 1 < nl && lo >= ph->L[l + 1].item0) ++l;
-      const ChLayer* L = &ph->L[l];
-      int tile = (lo - L->item0) / L->steps, bi = 0;
-      int j = lo - L->item0 - tile * L->steps;
-      while (bi + 1 < L->n_blocks && j >= L->blk[bi + 1].step0) ++bi;
-      GvBlock B = L->blk[bi];
-      j -= B.step0;
-      for (int it = lo; it < hi && go;) {
+      // Position of an item: layer, tile, block, step (tile-major); it and the
+      // block's table stay in registers from item to item.
+      int l, tile, bi, j;
+      const ChLayer* L;
+      GvBlock B;
+      auto seek = [&](int item) {
+        l = 0;
+        while (l + 1 < nl && item >= ph->L[l + 1].item0) ++l;
+        L = &ph->L[l];
+        tile = (item - L->item0) / L->steps;
+        j = item - L->item0 - tile * L->steps;
+        bi = 0;
+        while (bi + 1 < L->n_blocks && j >= L->blk[bi + 1].step0) ++bi;
+        B = L->blk[bi];
+        j -= B.step0;
+      };
+      seek(lo);
+      // The next piece of the pool, asked for a piece ahead (the answer takes
+      // about as long as an item).  Every CTA asks until it is refused once, so
+      // a launch adds chunks + G to the phase's counter.
+      const unsigned chunks = (unsigned)ph->chunks;
+      auto ask = [&]() { return atomicAdd(P.pool + p, 1u) - epoch * (chunks + (unsigned)G); };
+      unsigned next = chunks ? ask() : 0u;
+      for (int it = lo; go;) {
         const int slot = kg % kStages;
         if (kg >= kStages) {
           // the consumers free this stage only after the items it holds, so
@@ -338,11 +354,13 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
         const uint32_t bar = full0 + 8 * slot;
         {
           const bool last = j + n == B.n_steps && bi + 1 == L->n_blocks;  // of the tile
+          const bool ends = it + n == hi;  // of this range
           const int uvalid = min(B.units, B.n_ch - j * B.units);
           const int g0 = (B.grp_off + j * (B.units / 64)) & 3;
           uint4 d;
-          d.x = (uint32_t)B.bits | ((uint32_t)(last || it + n == hi) << 8) |
-                ((uint32_t)pair << 10) | ((uint32_t)l << 16);
+          d.x = (uint32_t)B.bits | ((uint32_t)(last || ends) << 8) |
+                ((uint32_t)(ends && next >= chunks) << 9) | ((uint32_t)pair << 10) |
+                ((uint32_t)l << 16);
           d.y = (uint32_t)uvalid | ((uint32_t)g0 << 16);
           d.z = (uint32_t)tile;
           d.w = 0u;
@@ -372,7 +390,13 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
         // next item
         it += n;
         j += n;
-        if (j == B.n_steps && it < hi) {
+        if (it == hi) {
+          if (next >= chunks) break;
+          it = G * ph->share + (int)next * chunk_items(NB);
+          hi = min(it + chunk_items(NB), ph->items);
+          next = ask();
+          seek(it);
+        } else if (j == B.n_steps) {
           j = 0;
           if (++bi == L->n_blocks) {
             bi = 0;
@@ -490,7 +514,7 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
     if (p + 1 < P.n_phases) init_outputs(P.ph + p + 1, P.batch, blockIdx.x, G);
     int lo, hi;
     item_range(P.ph + p, &lo, &hi);
-    for (int it = lo; it < hi;) {
+    for (bool more = lo < hi; more;) {
       bool ok = false;
       for (uint32_t w = 0; w < kWaitLimit; ++w) {
         if (mbar_try_wait(full0 + 8 * slot, phase)) {
@@ -510,7 +534,7 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
       const int bits = (int)(desc.x & 0xFFu);
       const int uvalid = (int)(desc.y & 0xFFFFu), g0 = (int)(desc.y >> 16);
       const bool pair = NB > 1 && (desc.x & 0x400u);
-      it += pair ? 2 : 1;
+      more = !(desc.x & 0x200u);  // the producer marks the last stage of a phase
       if (pair) {
         if constexpr (NB > 1) {
           const uint32_t* rec2 = rec + RB / 4;
@@ -700,6 +724,25 @@ int fill_phase(const polyq_gemv_phase& P, int nb, ChPhase* C) {
   return POLYQ_OK;
 }
 
+// Seven eighths of a phase's items are dealt out evenly, so that their weights
+// can be requested before the phase begins; the rest is a pool that CTAs take
+// from as they go, because they are not equally fast (the third CTA of an SM
+// gets the least of its issue slots, the builders of the records start late:
+// without a pool the last CTA of a phase ended 2 to 6 us after the mean, with
+// it 1).  13B-shaped layer at batch 1 / 4: no pool 77.1 / 89.3 us, an eighth
+// 70.8 / 88.2, a quarter 71.2 / 91.2, half 71.5 / 94.2 (a piece of the pool is
+// one more partial sum of a tile to add into y).  A phase of fewer than two
+// items per CTA has no pool.
+void share_out(ChPhase* C, int nb, int grid) {
+  C->share = C->items / grid;
+  C->extra = C->items % grid;
+  C->chunks = 0;
+  if (C->share < 2) return;
+  C->share = C->items * 7LL / 8 / grid;
+  C->extra = 0;
+  C->chunks = (C->items - grid * C->share + chunk_items(nb) - 1) / chunk_items(nb);
+}
+
 template <int NB>
 int launch_chain(const polyq_gemv_chain* ch, void* ws, cudaStream_t st) {
   static bool attr_done[64] = {false};
@@ -728,6 +771,7 @@ int launch_chain(const polyq_gemv_chain* ch, void* ws, cudaStream_t st) {
   P.status = static_cast<int*>(ws);
   P.bar = reinterpret_cast<unsigned int*>(static_cast<char*>(ws) + kWsCounters);
   P.ready = reinterpret_cast<unsigned int*>(static_cast<char*>(ws) + kWsReady);
+  P.pool = P.ready + ch->n_phases;
   P.rec = static_cast<uint8_t*>(ws) + ch->rec_off;
   cudaLaunchAttribute at[1];
   at[0].id = cudaLaunchAttributeCooperative;
@@ -810,8 +854,7 @@ extern "C" int polyq_gemv_chain_create(const polyq_gemv_phase* phases, int n_pha
         delete ch;
         return polyq_set_error(POLYQ_EUNSUPPORTED, "%s: phase %d has too many items", who, p);
       }
-      ch->ph[p].share = ch->ph[p].items / ch->grid;
-      ch->ph[p].extra = ch->ph[p].items % ch->grid;
+      share_out(&ch->ph[p], ch->nb, ch->grid);
     }
   } catch (const std::bad_alloc&) {
     delete ch;
@@ -824,7 +867,7 @@ extern "C" int polyq_gemv_chain_create(const polyq_gemv_phase* phases, int n_pha
   ch->init0 = (int)std::min<int64_t>(ch->grid, (out0 + 4 * kConsumers - 1) / (4 * kConsumers));
   int max_recs = 0;
   for (const ChPhase& c : ch->ph) max_recs = std::max(max_recs, c.recs);
-  ch->rec_off = (kWsReady + 4 * (size_t)n_phases + 255) / 256 * 256;
+  ch->rec_off = (kWsReady + 8 * (size_t)n_phases + 255) / 256 * 256;
   ch->ws_bytes = ch->rec_off + (size_t)max_recs * rec_bytes(ch->nb);
   *out = ch;
   return POLYQ_OK;
