@@ -10,12 +10,13 @@
 //    (a per-phase counter in the workspace).
 //  * Warps 0-3 (16 rows each) run the phases in order.  A grid-wide barrier
 //    (an arrival counter) separates phases, because phase p+1 reads what
-//    phase p wrote.  After it (in the first phase, at once), CTA b
-//    builds record b (b+G, ...) of the phase into the workspace: gather, transform (RMSNorm, SiLU * up, rounding to
-//    bf16), activation factor, fp16 rounding, per-chunk sums.  The warps then
-//    set the next phase's outputs to its residual (or zero) and decode and
-//    multiply their items exactly as the per-call kernel does, adding each
-//    tile piece's rows into y with fp32 atomics.
+//    phase p wrote.  After it (in the first phase, at once), CTA b builds
+//    record b (b+G, ...) of the phase into the workspace: gather, transform
+//    (RMSNorm, SiLU * up, rounding to bf16), activation factor, fp16 rounding,
+//    per-chunk sums.  The warps then set the next phase's outputs to its
+//    residual (or zero) and decode and multiply their items exactly as the
+//    per-call kernel does, adding each tile piece's rows into y with fp32
+//    atomics.
 // Items of a phase are (layer, tile, step) in tile-major order.  Each CTA takes
 // a contiguous range of equal length, so it streams the rows of a few tiles
 // from start to end, and then pieces of a pool (see share_out).  (At batch 1 an

@@ -483,6 +483,52 @@ __device__ __forceinline__ void load_words(uint32_t* w, const uint8_t* codes, in
   }
 }
 
+// Scales of the two MMA columns 2t, 2t + 1 of a lane: column col is (batch row
+// col / NGS, chunk col % NGS), so the two are neighbouring chunks of one batch
+// row, and their record entries come in one 8-byte load each.  (One column at a
+// time, each behind a test of its batch row: the Llama2-13B step 53.1 instead of
+// 51.2 us at batch 2, 65.0 instead of 64.7 at batch 4, 45.7 instead of 45.5 at
+// batch 1.  An early return for rows past the batch kept the compiler from
+// interleaving a pair's steps: 81 us at batch 4.)
+template <int NB, int NGS>
+struct ColScales {
+  static_assert(NGS % 2 == 0, "two chunks of a batch row per lane");
+  // Columns past NB * NGS (8-bit steps at batch 1) hold nothing.  Those of batch
+  // rows past the call's batch need no test: a record's rows are zero there, and
+  // flush_rows leaves these lanes' sums out.
+  static constexpr bool kAll = NB * NGS == 8;
+  float2 C1, X, E;
+  uint32_t m[2][2];  // (scale, zero) of rows rA and rB
+  __device__ __forceinline__ void load(const uint32_t* rec, const uint32_t* meta_s, int rA, int rB,
+                                       int g0, int t) {
+    constexpr int NGM = 8 / NB, PW = rec_pair_words(NB);
+    if (!kAll && 2 * t >= NB * NGS) return;
+    const int c = 2 * t % NGS;
+    const float2* recf = reinterpret_cast<const float2*>(rec + PW + 2 * t / NGS * NGM + c);
+    C1 = recf[0];
+    X = recf[NB * NGM / 2];
+    E = recf[NB * NGM];
+#pragma unroll
+    for (int cc = 0; cc < 2; ++cc) {
+      m[0][cc] = meta_s[rA * kMetaBox + g0 + c + cc];
+      m[1][cc] = meta_s[rB * kMetaBox + g0 + c + cc];
+    }
+  }
+  // D: the lane's MMA results, rows rA, rB by columns
+  __device__ __forceinline__ void add(const float (&D)[4], int t, float (&acc)[2]) const {
+    if (!kAll && 2 * t >= NB * NGS) return;
+#pragma unroll
+    for (int cc = 0; cc < 2; ++cc)
+#pragma unroll
+      for (int r = 0; r < 2; ++r) {
+        const float sc = __half2float(__ushort_as_half((uint16_t)(m[r][cc] & 0xFFFFu)));
+        const float ze = __half2float(__ushort_as_half((uint16_t)(m[r][cc] >> 16)));
+        const float x = cc ? X.y : X.x, c1 = cc ? C1.y : C1.x, e = cc ? E.y : E.x;
+        acc[r] += (sc * e) * fmaf(-ze, x, D[2 * r + cc] - c1);
+      }
+  }
+};
+
 // One step of a b<16 block for this warp's 16 rows; adds the chunk results,
 // scaled, into acc[row][batch].
 template <int NB, int BITS>
@@ -493,10 +539,8 @@ __device__ __forceinline__ void step_mma(uint32_t magic, int batch, int uvalid, 
                                          float (&acc)[2]) {
   constexpr int U = step_units(BITS, NB);
   constexpr int NGS = step_chunks(BITS, NB);
-  constexpr int NGM = 8 / NB;
   constexpr int NW = lane_words(BITS, NB);
   constexpr int LW = rec_lane_words(NB);
-  constexpr int PW = rec_pair_words(NB);
   constexpr int GP = group_pairs(BITS), GW = group_words(BITS);
   constexpr int NBX = nbox_of(BITS, NB);
   constexpr int GPB = NW / GW / NBX;      // groups per box
@@ -561,26 +605,9 @@ __device__ __forceinline__ void step_mma(uint32_t magic, int batch, int uvalid, 
     if constexpr (NACC == 4) D[v] += d[2][v] + d[3][v];
   }
 
-  // epilogue: columns 2t, 2t+1 -> (batch, chunk) (col / NGS, col % NGS);
-  // g0 is the step's first group in the meta box
-  const float* recf = reinterpret_cast<const float*>(rec);
-#pragma unroll
-  for (int cc = 0; cc < 2; ++cc) {
-    const int col = 2 * t + cc;
-    const int be = col / NGS, c = col % NGS;
-    if (be < batch) {
-      const float C1 = recf[PW + be * NGM + c];
-      const float X = recf[PW + NB * NGM + be * NGM + c];
-      const float E = recf[PW + 2 * NB * NGM + be * NGM + c];
-#pragma unroll
-      for (int r = 0; r < 2; ++r) {
-        const uint32_t m = meta_s[(r ? rB : rA) * kMetaBox + g0 + c];
-        const float sc = __half2float(__ushort_as_half((uint16_t)(m & 0xFFFFu)));
-        const float ze = __half2float(__ushort_as_half((uint16_t)(m >> 16)));
-        acc[r] += (sc * E) * fmaf(-ze, X, D[2 * r + cc] - C1);  // be is this lane's row
-      }
-    }
-  }
+  ColScales<NB, NGS> cs;  // g0 is the step's first group in the meta box
+  cs.load(rec, meta_s, rA, rB, g0, t);
+  cs.add(D, t, acc);
 }
 
 // Two consecutive one-box steps of a block and tile that share a stage (batch
@@ -594,10 +621,8 @@ __device__ __forceinline__ void step_mma_pair(uint32_t magic, int batch, int g0,
                                               const uint32_t* rec1, const uint32_t* zeros,
                                               int warp, int lane, float (&acc)[2]) {
   constexpr int NGS = step_chunks(BITS, NB);
-  constexpr int NGM = 8 / NB;
   constexpr int NW = lane_words(BITS, NB);
   constexpr int LW = rec_lane_words(NB);
-  constexpr int PW = rec_pair_words(NB);
   constexpr int GP = group_pairs(BITS), GW = group_words(BITS);
   static_assert(nbox_of(BITS, NB) == 1 && GP % 4 == 0 && NW % GW == 0, "pair geometry");
   constexpr int GPB = NW / GW;  // groups per step
@@ -662,24 +687,9 @@ __device__ __forceinline__ void step_mma_pair(uint32_t magic, int batch, int g0,
     float D[4];
 #pragma unroll
     for (int v = 0; v < 4; ++v) D[v] = d[k][0][v] + d[k][1][v];
-    const float* recf = reinterpret_cast<const float*>(k ? rec1 : rec0);
-#pragma unroll
-    for (int cc = 0; cc < 2; ++cc) {
-      const int col = 2 * t + cc;
-      const int be = col / NGS, c = col % NGS;
-      if (be < batch) {
-        const float C1 = recf[PW + be * NGM + c];
-        const float X = recf[PW + NB * NGM + be * NGM + c];
-        const float E = recf[PW + 2 * NB * NGM + be * NGM + c];
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const uint32_t m = meta_s[(r ? rB : rA) * kMetaBox + g0 + k * NGS + c];
-          const float sc = __half2float(__ushort_as_half((uint16_t)(m & 0xFFFFu)));
-          const float ze = __half2float(__ushort_as_half((uint16_t)(m >> 16)));
-          acc[r] += (sc * E) * fmaf(-ze, X, D[2 * r + cc] - C1);  // be is this lane's row
-        }
-      }
-    }
+    ColScales<NB, NGS> cs;
+    cs.load(k ? rec1 : rec0, meta_s, rA, rB, g0 + k * NGS, t);
+    cs.add(D, t, acc);
   }
 }
 
