@@ -105,6 +105,7 @@ struct Cfg {
   static constexpr int TN = TN_, NACC = NACC_, BK = BK_, OPS = OPS_, XS = XS_;
   static constexpr int CODES = CODES_, GROUPS = GROUPS_, EPI = EPI_;
   static constexpr int T = TN * NACC;
+  static constexpr bool kWhole = T == 512;  // see plan_split
   static constexpr int R = T / 2;           // tokens (rows of X) per CTA
   static constexpr int NBUF = NACC == 1 ? 2 : 1;
   static constexpr int HALVES = BK / kSlots;
@@ -149,6 +150,8 @@ struct GmParams {
   int bk;           // 32 or 64
   int r_log2;       // rows of X per CTA and unit: 2^r_log2
   int units_m, units_n, ksplit, units;  // work units: (token tile, N tile, K split)
+  int zero_col0;  // first column of Y that the pre-pass zeroes for a split of K
+  int whole;    // units that one pair computes alone (all, or with streamk the first ones)
   int streamk;  // 1: each pair takes an equal contiguous range of (unit, K tile) pairs:
   int sk_share, sk_extra;  // sk_share of them, the first sk_extra pairs one more
   int has_meta;
@@ -297,36 +300,46 @@ __device__ __forceinline__ int leading(uint32_t ok) { return __ffs(~ok) - 1; }
 
 // The pieces of work a CTA pair takes, in order: an output tile (um, un) and a
 // range [kt_lo, kt_hi) of its K tiles.  Units are strided over the pairs, each
-// with its K split's range; with `streamk`, a pair takes an equal contiguous
-// share (to one) of the units * KT (unit, K tile) pairs in unit-major order,
-// which cuts at most two units per pair short.  Every role of both CTAs walks
-// the same sequence.
+// with its K split's range; with `streamk`, units below `whole` are, and of the
+// (unit, K tile) pairs of the others, in unit-major order, a CTA pair takes an
+// equal contiguous share (to one), which cuts at most two units per pair short.
+// Every role of both CTAs walks the same sequence.
+template <bool WHOLE>  // the kernel takes whole units before a stream-K
 struct Pieces {
-  int g, g_hi;  // stream-K: (unit, K tile) pairs; else: unit
+  int g, g_hi;  // stream-K: (unit, K tile) pairs, g_hi -1 before them; else: unit
   __device__ __forceinline__ void init(const GmParams& P) {
+    g = blockIdx.x >> 1;
+    g_hi = -1;
+    if (!WHOLE && P.streamk) share(P);
+  }
+  __device__ __forceinline__ void share(const GmParams& P) {
     const int b = blockIdx.x >> 1;
-    if (P.streamk) {
-      g = b * P.sk_share + min(b, P.sk_extra);
-      g_hi = g + P.sk_share + (b < P.sk_extra ? 1 : 0);
-    } else {
-      g = b;
-    }
+    g = (WHOLE ? P.whole * P.KT : 0) + b * P.sk_share + min(b, P.sk_extra);
+    g_hi = g + P.sk_share + (b < P.sk_extra ? 1 : 0);
+  }
+  // After next(): the piece is one of several of its tile, to be added.
+  __device__ __forceinline__ bool adds(const GmParams& P) const {
+    return P.ksplit > 1 || (WHOLE ? g_hi >= 0 : P.streamk);
   }
   __device__ __forceinline__ bool next(const GmParams& P, int& um, int& un, int& kt_lo,
                                        int& kt_hi) {
     int uu, ks = 0;
-    if (P.streamk) {
+    if (WHOLE ? g_hi < 0 && g < P.whole : !P.streamk) {
+      if (g >= P.whole) return false;
+      uu = g;
+      g += gridDim.x >> 1;
+      kt_lo = 0;
+      kt_hi = P.KT;
+    } else {
+      if (WHOLE && g_hi < 0) {
+        if (!P.streamk) return false;
+        share(P);
+      }
       if (g >= g_hi) return false;
       uu = g / P.KT;
       kt_lo = g - uu * P.KT;
       kt_hi = min(P.KT, kt_lo + (g_hi - g));
       g += kt_hi - kt_lo;
-    } else {
-      if (g >= P.units) return false;
-      uu = g;
-      g += gridDim.x >> 1;
-      kt_lo = 0;
-      kt_hi = P.KT;
     }
     const int q = uu / P.units_m;
     um = uu - q * P.units_m;
@@ -467,7 +480,22 @@ __device__ __forceinline__ void slot_sources(const GmParams& P, const PrepTables
 }
 
 // Y = 0 by CTA `cta` of `n_cta` (Y is 16-byte aligned).
+template <bool COLS>  // perhaps only the columns from zero_col0 on
 __device__ __forceinline__ void zero_y(const GmParams& P, int cta, int n_cta) {
+  const int col0 = P.zero_col0;
+  if (COLS && col0 > 0) {  // the columns from the first tile on that is added up
+    const int w = P.N - col0;
+    const bool vec = P.N % 4 == 0;
+    const int cw = vec ? w / 4 : w;
+    for (int m = cta; m < P.M; m += n_cta) {
+      float* row = P.y + (size_t)m * P.N + col0;
+      for (int c = threadIdx.x; c < cw; c += blockDim.x) {
+        if (vec) reinterpret_cast<float4*>(row)[c] = make_float4(0.f, 0.f, 0.f, 0.f);
+        else row[c] = 0.f;
+      }
+    }
+    return;
+  }
   const long long total = (long long)P.M * P.N, total4 = total / 4;
   for (long long e = (long long)cta * blockDim.x + threadIdx.x; e < total4;
        e += (long long)n_cta * blockDim.x)
@@ -556,7 +584,7 @@ __global__ void __launch_bounds__(kRowsThreads) gemm_prep_rows(const __grid_cons
   }
   pdl_wait();  // X comes from the previous kernel; Y and the workspace may still be in use
   if (blockIdx.x == 0 && threadIdx.x == 0) *P.status = 0;
-  if (P.ksplit > 1 || P.streamk) zero_y(P, blockIdx.x, gridDim.x);
+  if (P.ksplit > 1 || P.streamk) zero_y<true>(P, blockIdx.x, gridDim.x);
   const int lane = threadIdx.x & 31;
   const int Mp = P.units_m << (P.r_log2 + 1);  // rows past M are zero: their MMA columns must be finite
   const bool vec = (P.K & 7) == 0 && (reinterpret_cast<uintptr_t>(P.x) & 15) == 0;
@@ -700,7 +728,7 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep_wide(const __grid_cons
   const int Kp = P.KT * P.bk, ks = Kp / kSlots;
   pdl_wait();  // X comes from the previous kernel; Y and the workspace may still be in use
   if (blockIdx.x == 0 && threadIdx.x == 0) *P.status = 0;
-  if (P.ksplit > 1 || P.streamk) zero_y(P, blockIdx.x, gridDim.x);
+  if (P.ksplit > 1 || P.streamk) zero_y<true>(P, blockIdx.x, gridDim.x);
   const int Mp = P.units_m << (P.r_log2 + 1);
   for (int m = blockIdx.x; m < Mp; m += gridDim.x) {
     auto value = [&](int k) -> float {  // at clustered slot k
@@ -743,7 +771,7 @@ __global__ void __launch_bounds__(kPrepThreads) gemm_prep_small(const __grid_con
   pdl_trigger();
   if ((int)blockIdx.x >= P.prep_rows) {
     pdl_wait();  // Y may still be in use
-    zero_y(P, (int)blockIdx.x - P.prep_rows, (int)gridDim.x - P.prep_rows);
+    zero_y<false>(P, (int)blockIdx.x - P.prep_rows, (int)gridDim.x - P.prep_rows);
     return;
   }
   __shared__ PrepTables S;
@@ -1067,7 +1095,7 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
     asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(peer), "r"(1) : "memory");
     atomicExch(P.status, code);
   };
-  Pieces pc;
+  Pieces<C::kWhole> pc;
   pc.init(P);
   int um, un, kt_lo, kt_hi;
   BlockCursor B;
@@ -1406,10 +1434,10 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
     const int e0 = (warp - C::kEpiWarp) >> 2;  // chunks e0, e0 + EPI / 4, ...
     constexpr int kChunks = C::T / 32 / (C::EPI / 4);
     const uint32_t acce0 = mapa(smem_u32(&bar_acce[0]), 0);
-    const bool add = P.ksplit > 1 || P.streamk;  // Y was zeroed by the pre-pass
     pdl_wait();  // the row scales come from the pre-pass
     for (int uc = 0; !s_abort && pc.next(P, um, un, kt_lo, kt_hi); ++uc) {
       const int buf = uc % C::NBUF;
+      const bool add = pc.adds(P);  // Y was zeroed by the pre-pass
       // column 32 c of the unit's accumulators: with two, columns [0, TN / 2)
       // of accumulator a are tokens a * TN / 2.. of CTA 0's R, the others of
       // CTA 1's
@@ -1539,26 +1567,39 @@ int resident_pairs(int dev, int* pairs) {
 // A unit's K tile takes `stage` seconds of a pair; a piece costs `piece` more
 // (pipeline fill, draining the accumulator) and splitting adds the zeroing of
 // Y.  Uniform split into k ranges: whole waves of units.  Stream-K: one
-// pair's equal share plus the pieces it touches.  Near ties go to the simpler
-// choice.
+// pair's equal share plus the pieces it touches; with `whole`, also after the
+// full waves of units that pairs compute alone, so that only the last wave is
+// shared.  Near ties go to the simpler choice (a gain of 3% promised to 13824 x
+// 5120, M = 8192 by a shared last wave did not show).  (5120 x 5120, M = 2048 / 4096 /
+// 8192: 87 / 163 / 314 us without the shared last wave, 84 / 150 / 296 with;
+// 13824 x 5120, M = 1536: 153 and 139; 5120 x 13824, M = 4096: 398 and 377.
+// The 256-token kernel is left without: 13824 x 5120, M = 512 59.9 us against
+// 57.5, but 1% slower at M = 256 and 1024 and 8% faster only for 5120 x 5120 at
+// M = 1024.)
 struct Split {
   double t;
   int ksplit, streamk;
+  long long whole;  // stream-K: units before it
 };
 Split plan_split(int64_t M, int64_t N, int T, int KT, int bk, int pairs, double stage,
-                 double piece) {
+                 double piece, bool whole) {
   const long long mn = ((M + T - 1) / T) * ((N + kRowsN - 1) / kRowsN);
   const double zero = (double)M * N * 4.0 / kZeroBytesPerS;
-  Split s = {1e300, 1, 0};
+  Split s = {1e300, 1, 0, 0};
   const int kmax = std::max(1, std::min(64, KT * bk / 512));
   for (int k = 1; k <= kmax; ++k) {
     const long long waves = (mn * k + pairs - 1) / pairs;
     const double t = waves * ((double)KT / k * stage + piece) + (k > 1 ? zero : 0.0);
-    if (t < 0.98 * s.t) s = {t, k, 0};
+    if (t < 0.98 * s.t) s = {t, k, 0, 0};
   }
-  const double share = std::ceil((double)mn * KT / pairs);
-  const double t_sk = share * stage + piece * (std::ceil(share / KT) + 1.0) + zero;
-  if (mn * KT >= pairs && mn * KT < (1ll << 31) && t_sk < 0.98 * s.t) s = {t_sk, 1, 1};
+  for (long long w : {0ll, whole ? mn / pairs : 0ll}) {  // whole waves before the shared units
+    const long long rest = mn - w * pairs;
+    const double share = std::ceil((double)rest * KT / pairs);
+    const double t_sk = w * (KT * stage + piece) + share * stage +
+                        piece * (std::ceil(share / KT) + 1.0) + zero * rest / mn;
+    if (rest * KT >= pairs && mn * KT < (1ll << 31) && t_sk < (w > 0 ? 0.95 : 0.98) * s.t)
+      s = {t_sk, 1, 1, w * pairs};
+  }
   return s;
 }
 
@@ -1695,7 +1736,8 @@ int consider(const polyq_dev_layer* L, int64_t M, int dev, int id, double stage,
   int pairs = 0;
   int rc = resident_pairs<C>(dev, &pairs);
   if (rc) return rc;
-  const Split s = plan_split(M, L->N, C::T, k_tiles(L, C::BK, nullptr), C::BK, pairs, stage, piece);
+  const Split s = plan_split(M, L->N, C::T, k_tiles(L, C::BK, nullptr), C::BK, pairs, stage, piece,
+                             C::kWhole);
   if (best->cfg < 0 || s.t < 0.98 * best->split.t) *best = {id, pairs, s};
   return POLYQ_OK;
 }
@@ -1712,8 +1754,11 @@ int run(const polyq_dev_layer* L, GmParams& P, const Choice& ch, int sms, int de
   P.ksplit = ch.split.ksplit;
   P.streamk = ch.split.streamk;
   P.units = P.units_m * P.units_n * P.ksplit;
+  P.whole = P.units;
   if (P.streamk) {
-    const int total = P.units * P.KT;  // below 2^31, see plan_split
+    P.whole = (int)ch.split.whole;
+    P.zero_col0 = P.whole / P.units_m * kRowsN;
+    const int total = (P.units - P.whole) * P.KT;  // below 2^31, see plan_split
     P.sk_share = total / ch.pairs;
     P.sk_extra = total % ch.pairs;
   }

@@ -173,3 +173,21 @@ def test_gemm_prepass_edges(polyq_lib, M, N, K, seed):
     torch.cuda.synchronize()
     assert polyq_lib.workspace_status(ws[-256:]) == 0
     check_tolerance(Y.cpu().numpy(), O.linear(O.pack_layer(W, a, 3.0, bits=bits), X), X, K)
+
+
+@pytest.mark.parametrize("N,seed", [(1800, 73), (1802, 74)])  # Y zeroed in 16-byte pieces and not
+def test_gemm_shared_last_wave(polyq_lib, N, seed):
+    """A little more than one wave of 512-token units: full units first, stored,
+    then the last ones cut along K and added into zeroed columns of Y, whose
+    first tile holds units of both kinds."""
+    M, K = 5121, 2100
+    W, a = synth.layer_weights(N, K, seed)
+    bits = synth.random_codes_layer_bits(K, seed)
+    Xb, X = synth.activations(a, M, seed)
+    dev = polyq_lib.DeviceLayer(polyq_lib.HostLayer.pack(W, a, 3.0, forced_bits=bits), "cuda")
+    ws = torch.zeros(polyq_lib.gemm_workspace_bytes(dev, M), dtype=torch.uint8, device="cuda")
+    Y = torch.full((M, N), float("nan"), device="cuda")
+    polyq_lib.linear_gemm(dev, _x_dev(Xb), Y=Y, workspace=ws)
+    torch.cuda.synchronize()
+    assert polyq_lib.workspace_status(ws[-256:]) == 0
+    check_tolerance(Y.cpu().numpy(), O.linear(O.pack_layer(W, a, 3.0, bits=bits), X), X, K)
