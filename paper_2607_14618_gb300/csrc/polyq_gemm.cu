@@ -126,7 +126,8 @@ struct Cfg {
   static constexpr size_t kSmem = (size_t)kCodeOff + CODES * kCode + 1024;
   static constexpr uint32_t kIdesc = umma_idesc_f16(kRowsN, TN);
   static_assert(kX % 1024 == 0 && kSmem <= 225 * 1024 + 512 && NACC * NBUF * TN <= (int)kTmemCols, "");
-  static_assert((GROUPS == 3 || GROUPS == 6) && CODES % GROUPS == 0 && OPS % GROUPS == 0 && kCodeProd <= CODES, "");
+  static_assert((GROUPS == 3 || GROUPS == 6) && CODES % GROUPS == 0 && OPS % GROUPS == 0 && kCodeProd <= CODES &&
+                OPS <= 32, "");  // a parity bit per weight slot
 };
 using Cfg32 = Cfg<32, 1, 64, 6, 16, 6, 6, 4>;
 using Cfg64 = Cfg<64, 1, 64, 6, 8, 6, 6, 4>;
@@ -1047,7 +1048,7 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
   __shared__ uint64_t bar_xfree[C::XS];     // its MMAs are done
   __shared__ uint64_t bar_bready[C::OPS];   // leader: both CTAs' weights are in place
   __shared__ uint64_t bar_sfree[C::OPS];    // a weight slot's MMAs are done
-  __shared__ uint64_t bar_w16[C::GROUPS];   // a group's tile of fp16 weights has landed
+  __shared__ uint64_t bar_w16[C::OPS];      // a weight slot's tile of fp16 weights has landed
   __shared__ uint64_t bar_accf[C::NBUF];    // an accumulator is complete
   __shared__ uint64_t bar_acce[C::NBUF];    // leader: both CTAs have drained it
   __shared__ uint64_t bar_done;             // every MMA is done (the leader waits for it)
@@ -1068,12 +1069,12 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
     for (int s = 0; s < C::OPS; ++s) {
       mbar_init(smem_u32(&bar_bready[s]), 2 * C::kDqGroup);  // a group of each CTA
       mbar_init(smem_u32(&bar_sfree[s]), 1);
+      mbar_init(smem_u32(&bar_w16[s]), 1);
     }
     for (int s = 0; s < C::XS; ++s) {
       mbar_init(smem_u32(&bar_xfull[s]), rank == 0 ? 2 : 1);  // the producer; the peer's relay
       mbar_init(smem_u32(&bar_xfree[s]), 1);
     }
-    for (int g = 0; g < C::GROUPS; ++g) mbar_init(smem_u32(&bar_w16[g]), 1);
     for (int b = 0; b < C::NBUF; ++b) {
       mbar_init(smem_u32(&bar_accf[b]), 1);
       mbar_init(smem_u32(&bar_acce[b]), 2 * C::EPI);
@@ -1299,7 +1300,13 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
     // Group g takes the stages k with k % GROUPS == g, thread r of the group
     // weight row r of the CTA.  (Copies may land out of order, and a parity
     // wait cannot tell a phase from the last but one: a code slot always
-    // belongs to one group, as GROUPS divides CODES.)
+    // belongs to one group, as GROUPS divides CODES.  For the same reason no
+    // barrier of the group may get two phases ahead of a warp that still waits
+    // there.  cfull, sfree and w16 of a slot cannot: the slot's next use
+    // needs its MMAs, so an arrival of every warp of the group after its wait.
+    // One w16 barrier for a group's two slots could: with the other slot free,
+    // the warp that asks for the copies passes stage j and completes stage
+    // j + GROUPS on it while another warp has still to look at stage j.)
     const int dq = (warp >> 2) * 3 + (warp & 3) - 1;  // 0..11
     constexpr int RW = C::kDqRows, kRowStep = 32 * C::kDqGroup;
     const int grp = dq / C::kDqGroup;
@@ -1311,7 +1318,8 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
     const uint32_t op_row = smem_u32(smem) + r * 64 + (((r >> 1) & 3) << 4);
     const uint32_t bready0 = mapa(smem_u32(&bar_bready[0]), 0);  // the leader's
     int sc = grp, s = grp;  // code and weight slot of the group's next stage
-    uint32_t cph = 0, sph = 1, w16_ph = 0;
+    uint32_t cph = 0, sph = 1;
+    uint32_t w16_ph = 0;  // bit s: parity of slot s's next fp16 tile
     int skip = grp;  // stages until the group's next one
     while (!s_abort && pc.next(P, um, un, kt_lo, kt_hi)) {
       B.seek(sblk, nblk, kt_lo);
@@ -1390,7 +1398,7 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
             if (!free) w = wait_ab(smem_u32(&bar_sfree[s]), sph, &s_abort);
             if (w != kWaitOk) break;
             if (r == 0) {
-              const uint32_t bar = smem_u32(&bar_w16[grp]);
+              const uint32_t bar = smem_u32(&bar_w16[s]);
               mbar_expect_tx(bar, C::kA);
 #pragma unroll
               for (int h = 0; h < C::HALVES; ++h)
@@ -1398,8 +1406,8 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
                             B.seg_off / 2 + C::BK * tb + kSlots * h,
                             un * kRowsN + (int)rank * kRowsCta, bar);
             }
-            w = wait_ab(smem_u32(&bar_w16[grp]), w16_ph, &s_abort);
-            w16_ph ^= 1u;
+            w = wait_ab(smem_u32(&bar_w16[s]), (w16_ph >> s) & 1u, &s_abort);
+            w16_ph ^= 1u << s;
             break;
         }
         if (w != kWaitOk) {

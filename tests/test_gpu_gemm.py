@@ -191,3 +191,22 @@ def test_gemm_shared_last_wave(polyq_lib, N, seed):
     torch.cuda.synchronize()
     assert polyq_lib.workspace_status(ws[-256:]) == 0
     check_tolerance(Y.cpu().numpy(), O.linear(O.pack_layer(W, a, 3.0, bits=bits), X), X, K)
+
+
+@pytest.mark.parametrize("M,N,K,seed", [
+    (1025, 5000, 320, 75),   # one unit per pair, ten K tiles
+    (3000, 1800, 2100, 76),  # 66 K tiles
+])
+def test_gemm_fp16_tiles_in_two_slots(polyq_lib, M, N, K, seed):
+    """All-16-bit layers with the 512-token kernel, whose groups alternate
+    between two weight slots."""
+    W, a = synth.layer_weights(N, K, seed)
+    Xb, X = synth.activations(a, M, seed)
+    dev = polyq_lib.DeviceLayer(polyq_lib.HostLayer.pack(W, a, 16.0), "cuda")
+    ws = torch.zeros(polyq_lib.gemm_workspace_bytes(dev, M), dtype=torch.uint8, device="cuda")
+    ref = O.linear(O.pack_layer(W, a, 16.0), X)
+    for _ in range(3):
+        Y = polyq_lib.linear_gemm(dev, _x_dev(Xb), workspace=ws)
+        torch.cuda.synchronize()
+        assert polyq_lib.workspace_status(ws[-256:]) == 0
+        check_tolerance(Y.cpu().numpy(), ref, X, K)
