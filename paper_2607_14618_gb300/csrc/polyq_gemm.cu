@@ -270,6 +270,12 @@ __device__ __forceinline__ int wait_sleep_ab(uint32_t bar, uint32_t parity,
   return kWaitTimeout;
 }
 
+// The same without a way out but the limit.
+__device__ __forceinline__ void mbar_wait_sleep(uint32_t bar, uint32_t parity, uint32_t limit) {
+  for (uint32_t it = 0; it < limit && !mbar_try_wait_hint(bar, parity, kSuspendHintNs); ++it) {
+  }
+}
+
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
   uint32_t ok;
   asm volatile(
@@ -1051,7 +1057,7 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
   __shared__ uint64_t bar_w16[C::OPS];      // a weight slot's tile of fp16 weights has landed
   __shared__ uint64_t bar_accf[C::NBUF];    // an accumulator is complete
   __shared__ uint64_t bar_acce[C::NBUF];    // leader: both CTAs have drained it
-  __shared__ uint64_t bar_done;             // every MMA is done (the leader waits for it)
+  __shared__ uint64_t bar_done;             // every MMA is done (both CTAs wait for it)
   __shared__ uint32_t tmem_base_slot;
   __shared__ GmBlock sblk[POLYQ_MAX_BLOCKS];
   __shared__ volatile int s_abort;
@@ -1228,6 +1234,9 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
           }
         }
       }
+      // The leader's commits arrive in this CTA's shared memory too, where no
+      // role waits for those of the last stages: stay for the last of all.
+      mbar_wait_sleep(smem_u32(&bar_done), 0, kWaitLimitSleep);
     }
   } else if (role == kRoleMma) {
     // ---------------- MMA issuer (leader CTA) ----------------
