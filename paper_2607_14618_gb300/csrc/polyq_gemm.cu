@@ -252,6 +252,7 @@ __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity
 // polling does not take issue slots from the dequantisation warps that share
 // their schedulers: at most 2^22 such polls, a few seconds.
 constexpr uint32_t kWaitLimitSleep = 1u << 22;
+constexpr uint32_t kDrainPolls = 1u << 14;  // 0.2 to 16 ms
 constexpr uint32_t kSuspendHintNs = 1000;
 constexpr int kWaitOk = 0, kWaitTimeout = 1, kWaitAborted = 2;
 __device__ __forceinline__ int wait_ab(uint32_t bar, uint32_t parity, const volatile int* abort) {
@@ -1201,9 +1202,14 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
           }
         }
       }
-      if (rank != 0)  // copies still in flight (the leader's MMA thread waits for its own)
+      // Copies still in flight.  The leader's MMA thread has waited for its own
+      // unless a role has given up; then the peer's arrival, which a phase of
+      // the leader needs too, may not come, and the limit is a few hundred times
+      // the copies' own time.
+      if (rank != 0 || s_abort)
         for (int j = max(0, k - C::XS); j < k; ++j)
-          mbar_wait(smem_u32(&bar_xfull[j % C::XS]), (j / C::XS) & 1);
+          mbar_wait_sleep(smem_u32(&bar_xfull[j % C::XS]), (j / C::XS) & 1,
+                          rank != 0 ? kWaitLimitSleep : kDrainPolls);
     }
   } else if (role == kRoleMma && rank != 0) {
     // ---------------- X relay (second CTA) ----------------
@@ -1416,6 +1422,8 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
                             un * kRowsN + (int)rank * kRowsCta, bar);
             }
             w = wait_ab(smem_u32(&bar_w16[s]), (w16_ph >> s) & 1u, &s_abort);
+            // given up: the thread that asked for the copies stays for them
+            if (w == kWaitAborted && r == 0) mbar_wait(smem_u32(&bar_w16[s]), (w16_ph >> s) & 1u);
             w16_ph ^= 1u << s;
             break;
         }
