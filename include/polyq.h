@@ -455,6 +455,8 @@ typedef struct {
  *     output itself: y += W'x in place);
  *   - the outputs of phase p+1 other than in-place ones overlap nothing that
  *     phase p reads or writes (they are initialised while phase p runs).
+ * A residual of phase p+1 may be what phase p writes: such a phase's outputs
+ * are initialised after phase p has finished.
  * *out owns a host plan; upload it to device memory with
  * polyq_gemv_chain_upload before launching. */
 int polyq_gemv_chain_create(const polyq_gemv_phase* phases, int n_phases, int batch,

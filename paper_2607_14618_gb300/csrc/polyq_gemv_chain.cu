@@ -14,8 +14,9 @@
 //    record b (b+G, ...) of the phase into the workspace: gather, transform
 //    (RMSNorm, SiLU * up, rounding to bf16), activation factor, fp16 rounding,
 //    per-chunk sums.  The warps then set the next phase's outputs to its
-//    residual (or zero) and decode and multiply their items exactly as the
-//    per-call kernel does, adding each tile piece's rows into y with fp32
+//    residual (or zero; a residual that this phase writes only after the
+//    barrier, see ChPhase::init) and decode and multiply their items exactly as
+//    the per-call kernel does, adding each tile piece's rows into y with fp32
 //    atomics.
 // Items of a phase are (layer, tile, step) in tile-major order.  Each CTA takes
 // a contiguous range of equal length, so it streams the rows of a few tiles
@@ -72,6 +73,12 @@ struct ChLayer {
 struct ChPhase {
   ChLayer L[POLYQ_MAX_GROUP];
   int n_layers, items, recs, kind;
+  // CTAs that set the phase's outputs once it has begun, counted with its
+  // records: for the first phase, and for one whose residual the phase before
+  // writes.  0: the outputs are set while the phase before runs.
+  int init;
+  int arrivals;  // recs + init
+  int ahead;     // 1: this phase sets the next one's outputs
   float eps;
   int share;   // items that every CTA takes, in order
   int extra;   // no pool: the first CTAs that take one more
@@ -84,11 +91,10 @@ struct ChPhase {
 struct ChParams {
   const ChPhase* ph;
   int n_phases, batch;
-  int init0;  // CTAs that initialise the first phase's outputs
   uint32_t magic;
   int* status;
   unsigned int* bar;    // [0] barrier arrivals, [1] CTAs done, [2] launches completed
-  unsigned int* ready;  // [n_phases] records built, summed over launches
+  unsigned int* ready;  // [n_phases] records built and outputs set by their CTAs, summed over launches
   unsigned int* pool;   // [n_phases] pool pieces asked for, summed over launches
   uint8_t* rec;         // records of the current phase
 };
@@ -102,7 +108,7 @@ struct ChShared {
   const int32_t* gather[POLYQ_MAX_GROUP];
   const float* xscale[POLYQ_MAX_GROUP];
   float* y[POLYQ_MAX_GROUP];
-  int n_layers, kind, recs;
+  int n_layers, kind, recs, init, ahead;
   float eps;
   const float* xa;
   const float* xb;
@@ -158,6 +164,8 @@ __device__ void load_phase(const ChPhase* ph, ChShared* S) {
     S->item0[nl] = ph->items;
     S->rec0[nl] = ph->recs;
     S->recs = ph->recs;
+    S->init = ph->init;
+    S->ahead = ph->ahead;
     S->kind = ph->kind;
     S->eps = ph->eps;
     S->xa = ph->xa;
@@ -259,9 +267,9 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
     const uint8_t* rsrc[kStages]; // record source of each pending stage, by slot
     int rphase[kStages], rbytes[kStages];
     auto wait_ready = [&](int p) -> bool {
-      // the counter grows by recs (and for the first phase init0) per launch
-      // and wraps: compare by signed difference
-      const unsigned target = (epoch + 1u) * (unsigned)(P.ph[p].recs + (p == 0 ? P.init0 : 0));
+      // the counter grows by this much per launch and wraps: compare by signed
+      // difference
+      const unsigned target = (epoch + 1u) * (unsigned)P.ph[p].arrivals;
       uint32_t it = 0;
       while ((int)(target - ld_acquire_gpu(P.ready + p)) > 0) {
         if (++it > kGridWaitLimit || s_abort) return false;
@@ -492,12 +500,14 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
   // ones, which build no record unless there is one for every CTA).  The first
   // stage is complete 8.5 us after the launch instead of 10.5.
   const int init_i = G - 1 - (int)blockIdx.x;
-  if (init_i < P.init0) init_outputs(P.ph, P.batch, init_i, P.init0);
+  const int init0 = P.ph->init;
+  if (init_i < init0) init_outputs(P.ph, P.batch, init_i, init0);
   prepare(0);
   bool alive = true;
   for (int p = 0; p < P.n_phases && alive; ++p) {
     // this CTA's share of the phase's records (the inputs are complete)
-    const bool init = p == 0 && init_i < P.init0;
+    const bool init = init_i < S.init;
+    if (p > 0 && init) init_outputs(P.ph + p, P.batch, init_i, S.init);
     if (blockIdx.x < S.recs || init) {
       int built = 0;
 #pragma unroll 1
@@ -513,7 +523,7 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
       consumer_sync();
       if (threadIdx.x == 0) add_release_gpu(P.ready + p, (unsigned)(built + init));
     }
-    if (p + 1 < P.n_phases) init_outputs(P.ph + p + 1, P.batch, blockIdx.x, G);
+    if (S.ahead) init_outputs(P.ph + p + 1, P.batch, blockIdx.x, G);
     int lo, hi;
     item_range(P.ph + p, &lo, &hi);
     for (bool more = lo < hi; more;) {
@@ -611,7 +621,6 @@ Span span(const void* p, size_t bytes) {
 
 struct polyq_gemv_chain {
   int n_phases = 0, batch = 0, nb = 1, grid = 0;
-  int init0 = 0;
   std::vector<ChPhase> ph;
   size_t plan_bytes = 0;
   size_t rec_off = 0, ws_bytes = 0;  // workspace: records region, total
@@ -668,6 +677,27 @@ void phase_spans(const polyq_gemv_phase& P, int batch, std::vector<Span>* reads,
     if (P.residuals[i] != P.ys[i]) fresh_writes->push_back(span(P.ys[i], ob));
   }
   if (P.in.x_out) writes->push_back(span(P.in.x_out, (size_t)batch * K * 2));
+}
+
+// Whether phase P starts an output from something that the phase before writes.
+bool residual_written(const polyq_gemv_phase& P, const polyq_gemv_phase& before, int batch) {
+  std::vector<Span> rd, wr, fresh;
+  phase_spans(before, batch, &rd, &wr, &fresh);
+  for (int i = 0; i < P.n_layers; ++i) {
+    if (P.residuals[i] == P.ys[i]) continue;
+    const Span res = span(P.residuals[i], (size_t)batch * P.layers[i]->N * 4);
+    for (const Span& w : wr)
+      if (overlap(res, w)) return true;
+  }
+  return false;
+}
+
+// CTAs that set the outputs of a phase which does so itself: four per thread.
+int init_ctas(const polyq_gemv_phase& P, int batch, int grid) {
+  int64_t out = 0;
+  for (int i = 0; i < P.n_layers; ++i)
+    if (P.residuals[i] != P.ys[i]) out += (int64_t)batch * P.layers[i]->N;
+  return (int)std::min<int64_t>(grid, (out + 4 * kConsumers - 1) / (4 * kConsumers));
 }
 
 int fill_phase(const polyq_gemv_phase& P, int nb, ChPhase* C) {
@@ -768,7 +798,6 @@ int launch_chain(const polyq_gemv_chain* ch, void* ws, cudaStream_t st) {
   P.ph = static_cast<const ChPhase*>(ch->plan_dev);
   P.n_phases = ch->n_phases;
   P.batch = ch->batch;
-  P.init0 = ch->init0;
   P.magic = kMagic;
   P.status = static_cast<int*>(ws);
   P.bar = reinterpret_cast<unsigned int*>(static_cast<char*>(ws) + kWsCounters);
@@ -857,16 +886,17 @@ extern "C" int polyq_gemv_chain_create(const polyq_gemv_phase* phases, int n_pha
         return polyq_set_error(POLYQ_EUNSUPPORTED, "%s: phase %d has too many items", who, p);
       }
       share_out(&ch->ph[p], ch->nb, ch->grid);
+      ChPhase& c = ch->ph[p];
+      const bool ahead = p > 0 && !residual_written(phases[p], phases[p - 1], batch);
+      if (ahead) ch->ph[p - 1].ahead = 1;
+      else c.init = init_ctas(phases[p], batch, ch->grid);
+      c.arrivals = c.recs + c.init;
     }
   } catch (const std::bad_alloc&) {
     delete ch;
     return polyq_set_error(POLYQ_ENOMEM, "%s: out of host memory", who);
   }
   ch->plan_bytes = (size_t)n_phases * sizeof(ChPhase);
-  int64_t out0 = 0;  // four outputs per thread
-  for (int i = 0; i < phases[0].n_layers; ++i)
-    if (phases[0].residuals[i] != phases[0].ys[i]) out0 += (int64_t)batch * phases[0].layers[i]->N;
-  ch->init0 = (int)std::min<int64_t>(ch->grid, (out0 + 4 * kConsumers - 1) / (4 * kConsumers));
   int max_recs = 0;
   for (const ChPhase& c : ch->ph) max_recs = std::max(max_recs, c.recs);
   ch->rec_off = (kWsReady + 8 * (size_t)n_phases + 255) / 256 * 256;

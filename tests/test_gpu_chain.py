@@ -256,3 +256,40 @@ def test_chained_phases_at_any_activation_scale(polyq_lib, batch, scale_exp):
     assert polyq_lib.workspace_status(chain.workspace) == 0
     for ph, ref, x in zip(phases, refs, xs):
         check_tolerance(ph["ys"][0].cpu().numpy(), O.linear(ref, x), x, x.shape[1])
+
+
+@pytest.mark.parametrize("batch", [1, 3, 4])
+@pytest.mark.parametrize("in_place", [False, True])
+def test_residual_that_the_phase_before_writes(polyq_lib, batch, in_place):
+    """A residual other than the output itself that the phase before computes
+    (or adds into): the outputs start from its finished value."""
+    N, K = 3000, 1231
+    dev, refs, xs = [], [], []
+    for i in range(3):
+        W, a = synth.layer_weights(N, K, 3400 + i)
+        bits = synth.random_codes_layer_bits(K, 3400 + i)
+        dev.append(polyq_lib.DeviceLayer(polyq_lib.HostLayer.pack(W, a, 3.0, forced_bits=bits),
+                                         "cuda"))
+        xb, x = synth.activations(a, batch, 3400 + i)
+        refs.append(O.linear(O.pack_layer(W, a, 3.0, bits=bits), x))
+        xs.append((_x_dev(xb), x))
+    h, y, z = (torch.empty((batch, N), device="cuda") for _ in range(3))
+    r = torch.randn(batch, N, device="cuda") * float(np.abs(refs[0]).mean())
+    x = lambda i: dict(layers=[dev[i]], kind=polyq_lib.X_BF16, a=xs[i][0])
+    chain = polyq_lib.GemvChain([
+        dict(x(0), ys=[h], residuals=[h] if in_place else [r]),
+        dict(x(1), ys=[y], residuals=[h]),
+        dict(x(2), ys=[z], residuals=[y]),
+    ], batch=batch)
+    r64 = r.cpu().numpy().astype(np.float64)
+    for _ in range(3):
+        h.copy_(r if in_place else torch.full_like(r, float("nan")))
+        y.fill_(float("nan"))
+        z.fill_(float("nan"))
+        chain.run()
+        torch.cuda.synchronize()
+        assert polyq_lib.workspace_status(chain.workspace) == 0
+        want = r64
+        for i, got in enumerate((h, y, z)):
+            want = want + refs[i]
+            check_tolerance(got.cpu().numpy(), want, xs[i][1], K)
