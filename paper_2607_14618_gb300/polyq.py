@@ -382,7 +382,10 @@ def _stream_ptr(stream):
     import torch
     if stream is not None:
         return stream.cuda_stream
-    return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # private: a torch may lack it
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
 def _workspace_of(workspace, need, zeros, dev):

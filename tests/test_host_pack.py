@@ -435,6 +435,23 @@ def test_binding_rejects_wrong_buffers_before_the_library(polyq_lib):
             polyq_lib._cuda_input(x, "x", torch.bfloat16, 16)
 
 
+def test_stream_handle_without_torchs_private_call(polyq_lib, monkeypatch):
+    """The current stream's handle, also from a torch without the raw-handle
+    call, and that of a given stream."""
+    import types
+
+    import torch
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 3)
+    monkeypatch.setattr(torch.cuda, "current_stream",
+                        lambda *a: types.SimpleNamespace(cuda_stream=0x77))
+    monkeypatch.setattr(torch._C, "_cuda_getCurrentRawStream", lambda dev: 0x10 + dev,
+                        raising=False)
+    assert polyq_lib._stream_ptr(None) == 0x13
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream")
+    assert polyq_lib._stream_ptr(None) == 0x77
+    assert polyq_lib._stream_ptr(types.SimpleNamespace(cuda_stream=0x99)) == 0x99
+
+
 def test_gemm_rejects_unaligned_output_on_the_host(polyq_lib):
     W, a = synth.layer_weights(64, 256, 62)
     host = polyq_lib.HostLayer.pack(W, a, 3.0)
