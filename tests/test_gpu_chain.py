@@ -179,6 +179,36 @@ def test_ranges_of_paired_steps(polyq_lib, batch):
             check_tolerance(y.cpu().numpy(), ref, x, K)
 
 
+def test_pool_of_single_steps(polyq_lib):
+    """Phases of more than two items per CTA at batch 1, whose last eighth is a
+    pool of one-item pieces, the second one in place on the first's output."""
+    phases, want = [], []
+    total = None
+    y = torch.full((1, 9000), float("nan"), device="cuda")
+    for i, (N, K, seed) in enumerate(((9000, 2500, 3500), (9000, 3001, 3501))):
+        W, a = synth.layer_weights(N, K, seed)
+        bits = synth.random_codes_layer_bits(K, seed)
+        dev = polyq_lib.DeviceLayer(polyq_lib.HostLayer.pack(W, a, 3.0, forced_bits=bits), "cuda")
+        xb, x = synth.activations(a, 1, seed)
+        phases.append(dict(layers=[dev], kind=polyq_lib.X_BF16, a=_x_dev(xb), ys=[y]))
+        if i:
+            phases[-1]["residuals"] = [y]
+        ref = O.linear(O.pack_layer(W, a, 3.0, bits=bits), x)
+        total = ref if total is None else total + ref
+        want.append((x, K))
+    chain = polyq_lib.GemvChain(phases, batch=1)
+    ctas = 3 * torch.cuda.get_device_properties(0).multi_processor_count
+    for run in range(1, 4):
+        chain.run()
+        torch.cuda.synchronize()
+        assert polyq_lib.workspace_status(chain.workspace) == 0
+        # after the record counters, from byte 256 on: pieces asked for per
+        # phase, one by every CTA more than there are
+        pool = chain.workspace[264:272].view(torch.int32).cpu().numpy()
+        assert all(int(n) > run * ctas and int(n) % run == 0 for n in pool)
+        check_tolerance(y.cpu().numpy(), total, *want[1])
+
+
 def test_phase_with_more_records_than_ctas(polyq_lib):
     # Four layers of 48 rows (one partial tile each) over K = 65536 channels
     # of all five widths at batch 4: 2048 records, so every CTA builds
