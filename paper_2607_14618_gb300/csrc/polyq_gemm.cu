@@ -1553,11 +1553,13 @@ int k_tiles(const polyq_dev_layer* L, int bk, GmBlock* blk) {
 // take it, K slots padded to 64 per block), the row scales [M] fp32, then 256
 // bytes holding the status word; each part starts on a 256-byte boundary.
 // Grows with M, so that a workspace made for M serves fewer rows too.
-size_t gemm_xg_bytes(const polyq_dev_layer* L, int64_t M) {
+size_t gemm_xg_rows(int64_t M) {
   size_t Mp = 32;
   while (Mp < 512 && Mp < (size_t)M) Mp *= 2;
-  if (Mp == 512) Mp = ((size_t)M + 511) / 512 * 512;
-  return Mp * k_tiles(L, 64, nullptr) * 64 * 2;
+  return Mp == 512 ? ((size_t)M + 511) / 512 * 512 : Mp;
+}
+size_t gemm_xg_bytes(const polyq_dev_layer* L, int64_t M) {
+  return gemm_xg_rows(M) * k_tiles(L, 64, nullptr) * 64 * 2;
 }
 size_t gemm_workspace(const polyq_dev_layer* L, int64_t M) {
   return gemm_xg_bytes(L, M) + ((size_t)M * 4 + 255) / 256 * 256 + 256;
@@ -1772,6 +1774,22 @@ int consider(const polyq_dev_layer* L, int64_t M, int dev, int id, double stage,
   return POLYQ_OK;
 }
 
+// The smallest token tile that holds M (a wider one would multiply padding:
+// 13824 x 5120 takes 24 / 28 / 37 us at M = 16 / 96 / 256, and took 53 us at
+// each with 256), or for more than 256 tokens the cheaper of 256 and 512 by
+// the model (stage and piece times measured).  `tokens` > 0: that tile.
+int choose(const polyq_dev_layer* L, int64_t M, int dev, int tokens, Choice* ch) {
+  const int t = tokens ? tokens : M <= 32 ? 32 : M <= 64 ? 64 : M <= 128 ? 128 : 256;
+  if (t == 32) return consider<Cfg32>(L, M, dev, 32, kStage32, kPiece32, ch);
+  if (t == 64) return consider<Cfg64>(L, M, dev, 64, kStage64, kPiece64, ch);
+  if (t == 128) return consider<Cfg128>(L, M, dev, 128, kStage128, kPiece128, ch);
+  int rc = POLYQ_OK;
+  if (t == 256) rc = consider<Cfg256>(L, M, dev, 256, kStage256, kPiece256, ch);
+  if (!rc && (t == 512 || (!tokens && M > 256)))
+    rc = consider<Cfg512>(L, M, dev, 512, kStage512, kPiece512, ch);
+  return rc;
+}
+
 template <class C>
 int run(const polyq_dev_layer* L, GmParams& P, const Choice& ch, int sms, int dev,
         cudaStream_t st) {
@@ -1815,32 +1833,20 @@ extern "C" int polyq_gemm_workspace_bytes(const polyq_dev_layer* L, int64_t M, s
   return POLYQ_OK;
 }
 
-#ifdef POLYQ_DEBUG
-// Debug build only: polyq_linear_gemm with every weight placed in a B tile
-// written to w_out [N][K] (fp16 bits, clustered order).
-extern "C" int polyq_debug_gemm_weights(const polyq_dev_layer* L, const void* X, int64_t M,
-                                        float* Y, void* workspace, size_t ws_bytes,
-                                        uint16_t* w_out, void* stream) {
-  polyq_clear_error();
-  cudaStream_t st = (cudaStream_t)stream;
-  const long long K = L ? L->K : 0;
-  cudaError_t e = cudaMemcpyToSymbolAsync(g_dbg_w, &w_out, sizeof w_out, 0,
-                                          cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess)
-    e = cudaMemcpyToSymbolAsync(g_dbg_wK, &K, sizeof K, 0, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
-  if (e != cudaSuccess) return polyq_set_error(POLYQ_ECUDA, "debug: %s", cudaGetErrorString(e));
-  const int rc = polyq_linear_gemm(L, X, M, Y, workspace, ws_bytes, stream);
-  uint16_t* none = nullptr;
-  cudaMemcpyToSymbolAsync(g_dbg_w, &none, sizeof none, 0, cudaMemcpyHostToDevice, st);
-  cudaStreamSynchronize(st);
-  return rc;
-}
-#endif
+namespace {
 
-extern "C" int polyq_linear_gemm(const polyq_dev_layer* L, const void* X, int64_t M, float* Y,
-                                 void* workspace, size_t ws_bytes, void* stream) {
-  polyq_clear_error();
+int device_index(int* dev) {
+  *dev = 0;
+  cudaGetDevice(dev);
+  if (*dev < 0 || *dev >= kMaxDevices)
+    return polyq_set_error(POLYQ_EUNSUPPORTED, "polyq_linear_gemm: device %d >= %d", *dev,
+                           kMaxDevices);
+  return POLYQ_OK;
+}
+
+// polyq_linear_gemm; tokens > 0 (debug build): with this token tile.
+int gemm_call(const polyq_dev_layer* L, const void* X, int64_t M, float* Y, void* workspace,
+              size_t ws_bytes, int tokens, void* stream) {
   int rc = polyq_check_dev_layer(L, "polyq_linear_gemm");
   if (rc) return rc;
   if (!X || !Y) return polyq_set_error(POLYQ_EINVAL, "polyq_linear_gemm: X or Y is NULL");
@@ -1887,22 +1893,10 @@ extern "C" int polyq_linear_gemm(const polyq_dev_layer* L, const void* X, int64_
   int sms = 0, dev = 0;
   rc = polyq_sm_count(&sms);
   if (rc) return rc;
-  cudaGetDevice(&dev);
-  if (dev < 0 || dev >= kMaxDevices)
-    return polyq_set_error(POLYQ_EUNSUPPORTED, "polyq_linear_gemm: device %d >= %d", dev,
-                           kMaxDevices);
-  // The smallest token tile that holds M (a wider one would multiply padding:
-  // 13824 x 5120 takes 24 / 28 / 37 us at M = 16 / 96 / 256, and took 53 us at
-  // each with 256), or for more than 256 tokens the cheaper of 256 and 512 by
-  // the model (stage and piece times measured).
+  rc = device_index(&dev);
+  if (rc) return rc;
   Choice ch = {-1, 0, {}};
-  if (M <= 32) rc = consider<Cfg32>(L, M, dev, 32, kStage32, kPiece32, &ch);
-  else if (M <= 64) rc = consider<Cfg64>(L, M, dev, 64, kStage64, kPiece64, &ch);
-  else if (M <= 128) rc = consider<Cfg128>(L, M, dev, 128, kStage128, kPiece128, &ch);
-  else {
-    rc = consider<Cfg256>(L, M, dev, 256, kStage256, kPiece256, &ch);
-    if (!rc && M > 256) rc = consider<Cfg512>(L, M, dev, 512, kStage512, kPiece512, &ch);
-  }
+  rc = choose(L, M, dev, tokens, &ch);
   if (rc) return rc;
   switch (ch.cfg) {
     case 32: return run<Cfg32>(L, P, ch, sms, dev, st);
@@ -1912,3 +1906,63 @@ extern "C" int polyq_linear_gemm(const polyq_dev_layer* L, const void* X, int64_
     default: return run<Cfg512>(L, P, ch, sms, dev, st);
   }
 }
+
+}  // namespace
+
+extern "C" int polyq_linear_gemm(const polyq_dev_layer* L, const void* X, int64_t M, float* Y,
+                                 void* workspace, size_t ws_bytes, void* stream) {
+  polyq_clear_error();
+  return gemm_call(L, X, M, Y, workspace, ws_bytes, 0, stream);
+}
+
+#ifdef POLYQ_DEBUG
+// Debug build only: polyq_linear_gemm with a given token tile and, if w_out is
+// not NULL, every weight placed in an A tile written to it ([N][K] fp16 bits,
+// clustered order).
+extern "C" int polyq_debug_linear_gemm(const polyq_dev_layer* L, const void* X, int64_t M,
+                                       float* Y, void* workspace, size_t ws_bytes, int tokens,
+                                       uint16_t* w_out, void* stream) {
+  polyq_clear_error();
+  if (tokens != 0 && tokens != 32 && tokens != 64 && tokens != 128 && tokens != 256 && tokens != 512)
+    return polyq_set_error(POLYQ_EINVAL, "debug: no kernel of %d tokens", tokens);
+  if (tokens && M > 0 && ((size_t)M + tokens - 1) / tokens * tokens > gemm_xg_rows(M))
+    return polyq_set_error(POLYQ_EINVAL, "debug: the workspace of M=%lld holds no tile of %d tokens",
+                           (long long)M, tokens);
+  cudaStream_t st = (cudaStream_t)stream;
+  const long long K = L ? L->K : 0;
+  cudaError_t e = cudaMemcpyToSymbolAsync(g_dbg_w, &w_out, sizeof w_out, 0,
+                                          cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess)
+    e = cudaMemcpyToSymbolAsync(g_dbg_wK, &K, sizeof K, 0, cudaMemcpyHostToDevice, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return polyq_set_error(POLYQ_ECUDA, "debug: %s", cudaGetErrorString(e));
+  const int rc = gemm_call(L, X, M, Y, workspace, ws_bytes, tokens, stream);
+  uint16_t* none = nullptr;
+  cudaMemcpyToSymbolAsync(g_dbg_w, &none, sizeof none, 0, cudaMemcpyHostToDevice, st);
+  cudaStreamSynchronize(st);
+  return rc;
+}
+
+extern "C" int polyq_debug_gemm_weights(const polyq_dev_layer* L, const void* X, int64_t M,
+                                        float* Y, void* workspace, size_t ws_bytes,
+                                        uint16_t* w_out, void* stream) {
+  return polyq_debug_linear_gemm(L, X, M, Y, workspace, ws_bytes, 0, w_out, stream);
+}
+
+// Debug build only: what polyq_linear_gemm would launch.
+extern "C" int polyq_debug_gemm_choice(const polyq_dev_layer* L, int64_t M, polyq_gemm_choice* out) {
+  polyq_clear_error();
+  int rc = polyq_check_dev_layer(L, "polyq_debug_gemm_choice");
+  if (rc) return rc;
+  if (!out || M < 1 || M > (1 << 24))
+    return polyq_set_error(POLYQ_EINVAL, "polyq_debug_gemm_choice: M=%lld", (long long)M);
+  int dev = 0;
+  rc = device_index(&dev);
+  if (rc) return rc;
+  Choice ch = {-1, 0, {}};
+  rc = choose(L, M, dev, 0, &ch);
+  if (rc) return rc;
+  *out = {ch.cfg, ch.pairs, ch.split.ksplit, ch.split.streamk, (int64_t)ch.split.whole};
+  return POLYQ_OK;
+}
+#endif

@@ -5,7 +5,8 @@ tensor cores' operand tile, against the oracle's unpacking of the same packed
 layer (Section 4.2 packing, R1 dequantisation).  The cases cover all five
 widths, ragged blocks (the last, partial group of every block), every 3-bit
 pair window, and the batch-1 (two boxes per step) and batch 2-4 (one box,
-paired steps) geometries."""
+paired steps) geometries, and each of the GEMM's token tiles, whose kernels cut
+K in tiles of 64 and (512 tokens) of 32."""
 import ctypes as C
 
 import numpy as np
@@ -13,22 +14,15 @@ import pytest
 
 from oracle import polyq_oracle as O
 from paper_2607_14618_gb300 import synth
+from tests.gpu_util import check_tolerance
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
 @pytest.fixture(scope="module")
-def dbg(polyq_lib):
-    from paper_2607_14618_gb300 import build
-    lib = C.CDLL(build.build_library(debug=True))
-    P = C.c_void_p
-    lib.polyq_debug_gemv_codes.argtypes = [C.POINTER(polyq_lib.DevLayer), P, C.c_int, P, P,
-                                           C.c_size_t, P, P]
-    lib.polyq_debug_gemm_weights.argtypes = [C.POINTER(polyq_lib.DevLayer), P, C.c_int64, P, P,
-                                             C.c_size_t, P, P]
-    lib.polyq_last_error.restype = C.c_char_p
-    return lib
+def dbg(polyq_debug):
+    return polyq_debug
 
 
 def _x_dev(xb):
@@ -105,3 +99,29 @@ def test_gemm_dequantised_weights_bit_exact(polyq_lib, dbg, M, N, K, B, seed, fo
     want = _oracle_fp16_weights(ref)
     bad = np.argwhere(got != want)
     assert bad.size == 0, f"{len(bad)} weights differ, first (row, pos) {bad[:4].tolist()}"
+
+
+@pytest.mark.parametrize("tokens", [32, 64, 128, 256, 512])
+@pytest.mark.parametrize("N,K,B,seed,forced", [
+    (300, 1100, 3.0, 87, True),    # all five widths, two N tiles, ragged
+    (520, 2100, 6.0, 88, False),   # many 8-bit channels
+    (300, 700, 16.0, 89, False),   # all 16-bit: every stage a copy of fp16 weights
+])
+def test_gemm_weights_bit_exact_by_token_tile(polyq_lib, dbg, tokens, N, K, B, seed, forced):
+    """The same with the kernel of each token tile, whatever M would take."""
+    M = 300
+    dev, ref, a = _layer(polyq_lib, N, K, B, seed, forced)
+    Xb, X = synth.activations(a, M, seed)
+    Xd = _x_dev(Xb)
+    Y = torch.full((M, N), float("nan"), device="cuda")
+    ws = torch.full((polyq_lib.gemm_workspace_bytes(dev, M),), 255, dtype=torch.uint8,
+                    device="cuda")
+    out = torch.full((N, K), -1, dtype=torch.int16, device="cuda")
+    rc = dbg.polyq_debug_linear_gemm(C.byref(dev.desc), Xd.data_ptr(), M, Y.data_ptr(),
+                                     ws.data_ptr(), ws.numel(), tokens, out.data_ptr(), None)
+    assert rc == 0, dbg.polyq_last_error()
+    torch.cuda.synchronize()
+    assert polyq_lib.workspace_status(ws[-256:]) == 0
+    bad = np.argwhere(out.cpu().numpy().view(np.uint16) != _oracle_fp16_weights(ref))
+    assert bad.size == 0, f"{len(bad)} weights differ, first (row, pos) {bad[:4].tolist()}"
+    check_tolerance(Y.cpu().numpy(), O.linear(ref, X), X, K)

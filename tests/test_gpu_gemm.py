@@ -1,4 +1,6 @@
 """GPU parity of the tcgen05 prefill GEMM against the oracle (through the C ABI)."""
+import ctypes as C
+
 import numpy as np
 import pytest
 
@@ -24,7 +26,7 @@ def _x_dev(xb):
     (96, 96, 640, 2.0, 57, False),       # all 2-bit
     (300, 520, 2100, 3.0, 60, True),     # stream-K: ~3 K tiles per CTA, cut across tiles
     (64, 2000, 4000, 3.0, 61, False),    # uniform K split into 8 ranges
-    (2000, 320, 1600, 3.0, 62, True),    # more rows than pre-pass CTAs (rows held in registers)
+    (2000, 320, 1600, 3.0, 62, True),    # more rows than pre-pass CTAs
 ])
 def test_gemm_matches_oracle(polyq_lib, M, N, K, B, seed, forced):
     W, a = synth.layer_weights(N, K, seed)
@@ -110,9 +112,9 @@ def test_gemm_rejects_unaligned_output(polyq_lib):
 
 
 def test_gemm_rows_too_wide_to_stage(polyq_lib):
-    """Rows of X wider than the pre-pass stages in shared memory (K > 49152)
-    are gathered from global memory instead; with activation factors too."""
-    M, N, K, seed = 40, 96, 50003, 63
+    """Rows of X wider than the pre-pass stages in shared memory (above 65520
+    channels whatever their bytes) are gathered from global memory instead."""
+    M, N, K, seed = 40, 96, 65523, 63
     W, a = synth.layer_weights(N, K, seed)
     bits = synth.random_codes_layer_bits(K, seed)
     Xb, X = synth.activations(a, M, seed)
@@ -129,14 +131,17 @@ def test_gemm_rows_too_wide_to_stage(polyq_lib):
     (258, 3001, 64),   # one and a bit tiles of weight rows, ragged K, all five widths
     (129, 70, 65),     # fewer K tiles than pipeline stages
 ])
-def test_gemm_token_tile_edges(polyq_lib, M, N, K, seed):
-    """Each number of tokens at the edge of a kernel's token tile (32 to 512),
-    on a workspace that a larger call left dirty."""
+def test_gemm_token_tile_edges(polyq_lib, polyq_debug, M, N, K, seed):
+    """Each number of tokens at the edge of a kernel's token tile, on a workspace
+    that a larger call left dirty.  These layers take the tiles of 32 to 256
+    tokens (test_gemm_512_token_edges: the other)."""
     W, a = synth.layer_weights(N, K, seed)
     bits = synth.random_codes_layer_bits(K, seed)
     Xb, X = synth.activations(a, M, seed)
     host = polyq_lib.HostLayer.pack(W, a, 3.0, forced_bits=bits)
     dev = polyq_lib.DeviceLayer(host, "cuda")
+    assert polyq_debug.gemm_choice(dev, M).tokens == next(
+        t for t in (32, 64, 128, 256) if M <= t or t == 256)
     need = polyq_lib.gemm_workspace_bytes(dev, M)
     assert need <= polyq_lib.gemm_workspace_bytes(dev, M + 1)  # a workspace serves fewer rows too
     ws = torch.full((need,), 255, dtype=torch.uint8, device="cuda")
@@ -175,16 +180,41 @@ def test_gemm_prepass_edges(polyq_lib, M, N, K, seed):
     check_tolerance(Y.cpu().numpy(), O.linear(O.pack_layer(W, a, 3.0, bits=bits), X), X, K)
 
 
-@pytest.mark.parametrize("N,seed", [(1800, 73), (1802, 74)])  # Y zeroed in 16-byte pieces and not
-def test_gemm_shared_last_wave(polyq_lib, N, seed):
-    """A little more than one wave of 512-token units: full units first, stored,
-    then the last ones cut along K and added into zeroed columns of Y, whose
-    first tile holds units of both kinds."""
-    M, K = 5121, 2100
+@pytest.mark.parametrize("M", [257, 511, 512, 513, 1024, 1025])
+@pytest.mark.parametrize("N,K,seed", [
+    (258, 3001, 64),  # one and a bit tiles of weight rows, ragged K, all five widths
+    (129, 70, 65),    # fewer K tiles than pipeline stages
+])
+def test_gemm_512_token_edges(polyq_lib, polyq_debug, M, N, K, seed):
+    """The 512-token kernel at the edges of its tile, split along K or not."""
     W, a = synth.layer_weights(N, K, seed)
     bits = synth.random_codes_layer_bits(K, seed)
     Xb, X = synth.activations(a, M, seed)
     dev = polyq_lib.DeviceLayer(polyq_lib.HostLayer.pack(W, a, 3.0, forced_bits=bits), "cuda")
+    ws = torch.full((polyq_lib.gemm_workspace_bytes(dev, M),), 255, dtype=torch.uint8,
+                    device="cuda")
+    Y = torch.full((M, N), float("nan"), device="cuda")
+    Xd = _x_dev(Xb)
+    rc = polyq_debug.polyq_debug_linear_gemm(C.byref(dev.desc), Xd.data_ptr(), M, Y.data_ptr(),
+                                             ws.data_ptr(), ws.numel(), 512, None, None)
+    assert rc == 0, polyq_debug.polyq_last_error()
+    torch.cuda.synchronize()
+    assert polyq_lib.workspace_status(ws[-256:]) == 0
+    check_tolerance(Y.cpu().numpy(), O.linear(O.pack_layer(W, a, 3.0, bits=bits), X), X, K)
+
+
+@pytest.mark.parametrize("N,seed", [(2056, 73), (2058, 74)])  # Y zeroed in 16-byte pieces and not
+def test_gemm_shared_last_wave(polyq_lib, polyq_debug, N, seed):
+    """A little more than one wave of 512-token units: full units first, stored,
+    then the last ones cut along K and added into zeroed columns of Y, whose
+    first tile holds units of both kinds."""
+    M, K = 4097, 2100
+    W, a = synth.layer_weights(N, K, seed)
+    bits = synth.random_codes_layer_bits(K, seed)
+    Xb, X = synth.activations(a, M, seed)
+    dev = polyq_lib.DeviceLayer(polyq_lib.HostLayer.pack(W, a, 3.0, forced_bits=bits), "cuda")
+    ch = polyq_debug.gemm_choice(dev, M)
+    assert ch.tokens == 512 and ch.streamk and ch.whole > 0 and ch.whole % -(-M // 512) != 0
     ws = torch.zeros(polyq_lib.gemm_workspace_bytes(dev, M), dtype=torch.uint8, device="cuda")
     Y = torch.full((M, N), float("nan"), device="cuda")
     polyq_lib.linear_gemm(dev, _x_dev(Xb), Y=Y, workspace=ws)
@@ -197,12 +227,13 @@ def test_gemm_shared_last_wave(polyq_lib, N, seed):
     (1025, 5000, 320, 75),   # one unit per pair, ten K tiles
     (3000, 1800, 2100, 76),  # 66 K tiles
 ])
-def test_gemm_fp16_tiles_in_two_slots(polyq_lib, M, N, K, seed):
+def test_gemm_fp16_tiles_in_two_slots(polyq_lib, polyq_debug, M, N, K, seed):
     """All-16-bit layers with the 512-token kernel, whose groups alternate
     between two weight slots."""
     W, a = synth.layer_weights(N, K, seed)
     Xb, X = synth.activations(a, M, seed)
     dev = polyq_lib.DeviceLayer(polyq_lib.HostLayer.pack(W, a, 16.0), "cuda")
+    assert polyq_debug.gemm_choice(dev, M).tokens == 512
     ws = torch.zeros(polyq_lib.gemm_workspace_bytes(dev, M), dtype=torch.uint8, device="cuda")
     ref = O.linear(O.pack_layer(W, a, 16.0), X)
     for _ in range(3):
