@@ -82,7 +82,7 @@ def _oracle_fp16_weights(ref):
 @pytest.mark.parametrize("M,N,K,B,seed,forced", [
     (16, 300, 1100, 3.0, 84, True),    # all five widths, two N tiles, ragged
     (64, 256, 2048, 3.0, 85, False),   # the allocation at B = 3
-    (8, 520, 2100, 6.0, 86, False),    # many 8-bit channels; stream-K
+    (8, 520, 2100, 6.0, 86, False),    # many 8-bit channels; K split into ranges
 ])
 def test_gemm_dequantised_weights_bit_exact(polyq_lib, dbg, M, N, K, B, seed, forced):
     dev, ref, a = _layer(polyq_lib, N, K, B, seed, forced)

@@ -17,15 +17,15 @@ def _x_dev(xb):
 
 
 @pytest.mark.parametrize("M,N,K,B,seed,forced", [
-    (256, 256, 1100, 3.0, 51, True),     # all five widths, one work unit
-    (300, 300, 1100, 3.0, 52, True),     # ragged M and N, two units per axis
+    (256, 256, 1100, 3.0, 51, True),     # all five widths, one output tile
+    (300, 300, 1100, 3.0, 52, True),     # ragged M and N, two tiles per axis
     (1, 100, 700, 3.0, 53, True),        # a single token
     (512, 640, 2048, 3.0, 54, False),    # allocation at B = 3
     (130, 257, 1536, 6.0, 55, False),    # B = 6: many 8-bit channels
     (64, 64, 320, 16.0, 56, False),      # all 16-bit
     (96, 96, 640, 2.0, 57, False),       # all 2-bit
-    (300, 520, 2100, 3.0, 60, True),     # stream-K: ~3 K tiles per CTA, cut across tiles
-    (64, 2000, 4000, 3.0, 61, False),    # uniform K split into 8 ranges
+    (300, 520, 2100, 3.0, 60, True),     # uniform K split into 4 ranges
+    (64, 2000, 4000, 3.0, 61, False),    # uniform K split into 7 ranges
     (2000, 320, 1600, 3.0, 62, True),    # more rows than pre-pass CTAs
 ])
 def test_gemm_matches_oracle(polyq_lib, M, N, K, B, seed, forced):
@@ -198,6 +198,27 @@ def test_gemm_512_token_edges(polyq_lib, polyq_debug, M, N, K, seed):
     rc = polyq_debug.polyq_debug_linear_gemm(C.byref(dev.desc), Xd.data_ptr(), M, Y.data_ptr(),
                                              ws.data_ptr(), ws.numel(), 512, None, None)
     assert rc == 0, polyq_debug.polyq_last_error()
+    torch.cuda.synchronize()
+    assert polyq_lib.workspace_status(ws[-256:]) == 0
+    check_tolerance(Y.cpu().numpy(), O.linear(O.pack_layer(W, a, 3.0, bits=bits), X), X, K)
+
+
+@pytest.mark.parametrize("M,N,K,seed,tokens", [
+    (16, 1000, 1003, 77, 32),     # shares of about one K tile
+    (64, 1500, 1003, 78, 64),     # shares of one or two, cut across output tiles
+    (1100, 2000, 3000, 79, 256),  # shares of about half an output tile
+])
+def test_gemm_stream_k(polyq_lib, polyq_debug, M, N, K, seed, tokens):
+    """Every unit shared along K by equal shares of K tiles."""
+    W, a = synth.layer_weights(N, K, seed)
+    bits = synth.random_codes_layer_bits(K, seed)
+    Xb, X = synth.activations(a, M, seed)
+    dev = polyq_lib.DeviceLayer(polyq_lib.HostLayer.pack(W, a, 3.0, forced_bits=bits), "cuda")
+    ch = polyq_debug.gemm_choice(dev, M)
+    assert ch.tokens == tokens and ch.streamk and ch.whole == 0
+    ws = torch.zeros(polyq_lib.gemm_workspace_bytes(dev, M), dtype=torch.uint8, device="cuda")
+    Y = torch.full((M, N), float("nan"), device="cuda")
+    polyq_lib.linear_gemm(dev, _x_dev(Xb), Y=Y, workspace=ws)
     torch.cuda.synchronize()
     assert polyq_lib.workspace_status(ws[-256:]) == 0
     check_tolerance(Y.cpu().numpy(), O.linear(O.pack_layer(W, a, 3.0, bits=bits), X), X, K)
