@@ -462,13 +462,14 @@ typedef struct {
 int polyq_gemv_chain_create(const polyq_gemv_phase* phases, int n_phases, int batch,
                             polyq_gemv_chain** out);
 
-/* Bytes of device memory the chain's plan needs (tensor maps, block tables
- * and work shares for the current device). */
 /* Bytes of the workspace a launch of the chain needs: a status word, the
- * grid-barrier and launch counters, one record-ready counter per phase and
- * the activation records of the largest phase. */
+ * grid-barrier and launch counters, per phase a record-ready counter and a
+ * counter of the pool pieces taken, and the activation records of the largest
+ * phase. */
 int polyq_gemv_chain_workspace_bytes(const polyq_gemv_chain* chain, size_t* bytes);
 
+/* Bytes of device memory the chain's plan needs (tensor maps, block tables
+ * and work shares for the current device). */
 int polyq_gemv_chain_plan_bytes(const polyq_gemv_chain* chain, size_t* bytes);
 
 /* Copy the plan into plan_dev (device memory of at least

@@ -80,10 +80,12 @@ constexpr double kZeroBytesPerS = 5e12;  // the pre-pass zeroing Y
 constexpr uint32_t kTmemCols = 512;
 // Cost model of the split of K (plan_split), seconds: one stage of a pair and
 // the overhead of a piece, by token tile.
-// (Stages as traced; pieces set so that the model picks the faster of both
-// splits and both tiles on 5120 x 5120, 13824 x 5120 and 5120 x 13824 from M =
-// 16 to 4096, to 2%: 5120 x 5120, M = 512 34.5 us with 4.5 and 5.5, 32.2 with
-// 3.5 and 6.5; 13824 x 5120, M = 256 36.3 and 34.4.)
+// (Stages as traced in short runs, at about 1.9 GHz: with 512 tokens the MMAs'
+// 512 cycles.  Long runs, under the power cap, take 0.33 to 0.36 us for those.
+// Pieces set so that the model picks the faster of both splits and both tiles on
+// 5120 x 5120, 13824 x 5120 and 5120 x 13824 from M = 16 to 4096, to 2%: 5120 x
+// 5120, M = 512 34.5 us with 4.5 and 5.5, 32.2 with 3.5 and 6.5; 13824 x 5120,
+// M = 256 36.3 and 34.4.)
 constexpr double kStage32 = 0.23e-6, kPiece32 = 1.5e-6;
 constexpr double kStage64 = 0.24e-6, kPiece64 = 1.5e-6;
 constexpr double kStage128 = 0.26e-6, kPiece128 = 2e-6;
@@ -142,8 +144,8 @@ using Cfg512 = Cfg<256, 2, 32, 6, 7, 9, 3, 8>;
 enum Role { kRoleCode0 = 0, kRoleCode1, kRoleX, kRoleMma, kRoleDequant, kRoleEpilogue };
 
 struct GmBlock {
-  int bits, n_ch, pos0, seg_off, grp_off, n_grp;
-  int kt0, n_kt;  // K-tile range of the block
+  int bits, n_ch, pos0, seg_off, grp_off;
+  int kt0;  // first K tile of the block
 };
 
 struct GmParams {
@@ -191,7 +193,8 @@ __device__ __forceinline__ void cluster_sync() {
 // Arrive on a barrier of a CTA of the cluster (address from mapa).  With the
 // default scope: what such an arrival announces (weights and X in this CTA's
 // shared memory, drained tensor memory) reaches the other side only through
-// the tensor core, which fence.proxy.async and the tcgen05 fences order.  A
+// the tensor core, which fence.proxy.async and the tcgen05 fences order (by the
+// letter of the memory model the arrival would be at cluster scope too).  A
 // release at cluster scope waits for all of the warp's memory traffic at every
 // stage: gate at M = 2048 took 352 us with it and 281 us without.
 __device__ __forceinline__ void mbar_arrive_cluster(uint32_t bar) {
@@ -1031,9 +1034,10 @@ __device__ __forceinline__ void store_chunk(float* __restrict__ y, uint32_t N, b
 }
 
 // What bounds it, by token tile (13824 x 5120 at B = 3, one call): with 512
-// tokens the tensor core: a stage of 32 K takes 507 cycles of the MMAs' 512,
-// an accumulator drain 9400 cycles per 95000 of a unit (M = 2048: 277 -> 171
-// us; M = 4096: 529 -> 349 us, 1660 TFLOP/s).  With 256 and fewer the latency
+// tokens the tensor core: a stage of 32 K takes the MMAs' 512 cycles (8192
+// multiply-adds a cycle and pair; traced to 1%), an accumulator drain 9400
+// cycles per 95000 of a unit (M = 2048: 277 -> 171 us; M = 4096: 529 -> 349 us,
+// 1660 TFLOP/s).  With 256 and fewer the latency
 // of a stage of 64 K through its rings, 440 to 590 cycles (M = 256: 53.6 -> 37
 // us, M = 96: 54 -> 28 us, M = 16: 53 -> 24 us): the arrival at the leader
 // (1300 cycles of a weight slot's turn of 2640), the commit back (400), and
@@ -1540,10 +1544,8 @@ int k_tiles(const polyq_dev_layer* L, int bk, GmBlock* blk) {
     g.pos0 = b.pos0;
     g.seg_off = b.seg_off;
     g.grp_off = b.grp_off;
-    g.n_grp = b.n_grp;
     g.kt0 = kt;
-    g.n_kt = (b.n_ch + bk - 1) / bk;
-    kt += g.n_kt;
+    kt += (b.n_ch + bk - 1) / bk;
     if (blk) blk[i] = g;
   }
   return kt;

@@ -112,8 +112,9 @@ struct GvParams {
   uint16_t* xout;   // optional bf16 copy of the transformed input
 };
 
-// Per-CTA shared copy of the scalars and block tables (runtime-indexed reads
-// of kernel parameters would become slow generic loads).
+// Per-CTA shared copy of the scalars and block tables that the producer reads
+// for every stage.  (The pre-pass, which needs one record's entries once, indexes
+// the parameters themselves.)
 struct GvShared {
   GvBlock blk[POLYQ_MAX_GROUP][POLYQ_MAX_BLOCKS];
   int n_blocks[POLYQ_MAX_GROUP];

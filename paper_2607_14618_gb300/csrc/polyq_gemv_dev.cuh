@@ -81,9 +81,10 @@ __device__ __forceinline__ void load_pairs(uint32_t* s_pair) {
 }
 
 // Units (inside the step) and scale exponents of the pair that lane `lane` of
-// the warp holding chunk c makes, and the pair's lane t and index jp: the
-// layout's chunk_pair, pair_units and lane_unit with the width as a value, by
-// shifts, so that one short path serves all widths.
+// the warp holding chunk c makes: of the 32 lane pairs that cover the chunk the
+// lane-th, pair jp of the layout's lane t.  The layout's pair_units and
+// lane_unit with the width as a value, by shifts, so that one short path serves
+// all widths.
 __host__ __device__ __forceinline__ void chunk_pair_units(int bits, int nb, int c, int lane,
                                                           const uint32_t* pairs, int* t, int* jp,
                                                           int (&unit)[2], int (&p)[2]) {

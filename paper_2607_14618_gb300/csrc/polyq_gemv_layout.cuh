@@ -170,17 +170,6 @@ __host__ __device__ inline void pair_units(int bits, int j, int* ulo, int* plo, 
   *phi = d.phi;
 }
 
-// The 32 lane pairs that cover chunk c of a step: the q-th of them is pair jp
-// of lane t.
-__host__ __device__ inline void chunk_pair(int bits, int nb, int c, int q, int* t, int* jp) {
-  const int per = lane_per(bits, nb);
-  const int cpb = step_units(bits, nb) / nbox_of(bits, nb) / 64;  // chunks per box
-  const int h = c / cpb, cb = c % cpb;
-  const int lpc = 64 / per;  // lanes per chunk (1 or 2)
-  *t = cb * lpc + q / (per / 2);
-  *jp = h * (per / 2) + q % (per / 2);
-}
-
 // 16-bit steps: step-relative weight index of the lane's i-th weight (i < 32):
 // lane t holds weights [16t, 16t+16) of each 64-weight box.
 __host__ __device__ inline int lane_weight16(int t, int i) {
