@@ -56,6 +56,7 @@
 #include "polyq.h"
 #ifdef POLYQ_DEBUG
 #include "polyq_debug.h"
+#include "polyq_debug_gemm.h"
 #endif
 #include "polyq_dev.cuh"
 #include "polyq_gemv_dev.cuh"

@@ -24,7 +24,7 @@ def polyq_lib():
 
 @pytest.fixture(scope="session")
 def polyq_debug(polyq_lib):
-    """The debug build of the library (include/polyq_debug.h), by ctypes."""
+    """The debug build of the library (include/polyq_debug*.h), by ctypes."""
     import ctypes as C
 
     from paper_2607_14618_gb300 import build

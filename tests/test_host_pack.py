@@ -34,6 +34,17 @@ def test_debug_library_exports_its_declared_symbols(polyq_lib):
         assert not hasattr(lib, n), n
 
 
+def test_debug_library_exports_the_gemm_test_calls(polyq_lib):
+    """The same for include/polyq_debug_gemm.h."""
+    from paper_2607_14618_gb300 import build
+    names = _declared_functions(os.path.join(os.path.dirname(HEADER), "polyq_debug_gemm.h"))
+    assert names == ["polyq_debug_gemm_choice", "polyq_debug_linear_gemm"]
+    dbg = C.CDLL(build.build_library(debug=True))
+    lib = C.CDLL(polyq_lib.LIB_PATH)
+    for n in names:
+        assert hasattr(dbg, n) and not hasattr(lib, n), n
+
+
 def test_library_exports_every_declared_symbol(polyq_lib):
     names = _declared_functions()
     assert len(names) >= 15
