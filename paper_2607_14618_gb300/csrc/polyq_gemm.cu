@@ -40,8 +40,8 @@
 //     pieces are added into a zeroed Y (so the order of those additions
 //     varies); otherwise Y is stored directly.  Every wait is bounded and
 //     reports through the workspace status word.
-// Bound by the tensor pipe at large M (13824 x 5120, M = 2048, B = 3: 173 us for
-// both kernels, 1670 TFLOP/s, the pipe active 83% of the cycles; on single SMs
+// Bound by the tensor pipe at large M (13824 x 5120, M = 2048, B = 3: 174 us for
+// both kernels, 1660 TFLOP/s, the pipe active 83% of the cycles; on single SMs
 // 273 us, 50%) and by the dequantisers' stages and the fixed time of the two
 // launches at small M (5120 x 5120, M = 16: 14.6 us, before 27).
 #include <cuda.h>
