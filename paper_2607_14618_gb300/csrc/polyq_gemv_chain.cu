@@ -210,8 +210,10 @@ __device__ __forceinline__ void item_range(const ChPhase* ph, int* lo, int* hi) 
 __host__ __device__ constexpr int chunk_items(int nb) { return nb == 1 ? 1 : 2; }
 
 // Outputs of a phase start as the residual (or zero): the share of the
-// consumer threads of CTA `cta` of `n_cta`.
-__device__ void init_outputs(const ChPhase* ph, int batch, int cta, int n_cta) {
+// consumer threads of CTA `cta` of `n_cta`.  Out of line: with a third copy of it
+// in the kernel a layer at batch 3 and 4 took 1% longer (107.5 -> 108.6 us on
+// Qwen3-32B's shapes).
+__device__ __noinline__ void init_outputs(const ChPhase* ph, int batch, int cta, int n_cta) {
   const int nl = ph->n_layers;
   const int stride = n_cta * kConsumers;
   for (int l = 0; l < nl; ++l) {
@@ -500,14 +502,12 @@ __global__ void __launch_bounds__(kThreads, kChCtasPerSm) gemv_chain(const __gri
   // ones, which build no record unless there is one for every CTA).  The first
   // stage is complete 8.5 us after the launch instead of 10.5.
   const int init_i = G - 1 - (int)blockIdx.x;
-  const int init0 = P.ph->init;
-  if (init_i < init0) init_outputs(P.ph, P.batch, init_i, init0);
   prepare(0);
   bool alive = true;
   for (int p = 0; p < P.n_phases && alive; ++p) {
     // this CTA's share of the phase's records (the inputs are complete)
     const bool init = init_i < S.init;
-    if (p > 0 && init) init_outputs(P.ph + p, P.batch, init_i, S.init);
+    if (init) init_outputs(P.ph + p, P.batch, init_i, S.init);
     if (blockIdx.x < S.recs || init) {
       int built = 0;
 #pragma unroll 1
