@@ -256,7 +256,7 @@ __device__ __forceinline__ bool mbar_try_wait_hint(uint32_t bar, uint32_t parity
 // polling does not take issue slots from the dequantisation warps that share
 // their schedulers: at most 2^22 such polls, a few seconds.
 constexpr uint32_t kWaitLimitSleep = 1u << 22;
-constexpr uint32_t kDrainPolls = 1u << 14;  // 0.2 to 16 ms
+constexpr long long kAbortStayCycles = 1 << 21;  // a millisecond
 constexpr uint32_t kSuspendHintNs = 1000;
 constexpr int kWaitOk = 0, kWaitTimeout = 1, kWaitAborted = 2;
 __device__ __forceinline__ int wait_ab(uint32_t bar, uint32_t parity, const volatile int* abort) {
@@ -1107,11 +1107,16 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
   pdl_trigger();
 
   const int nblk = P.n_blocks;
+  // A role gives up.  Then nobody waits for the copies of X in the leader and
+  // those of fp16 weights: by staying a thousand times their own time it keeps
+  // both CTAs, which leave together.  (Waits by the roles that asked for them,
+  // or a test at the kernel's end, cost every call 0.1 us.)
   auto fail = [&](int code) {
     s_abort = 1;
     const uint32_t peer = mapa(smem_u32((const void*)&s_abort), rank ^ 1u);
     asm volatile("st.relaxed.cluster.shared::cluster.u32 [%0], %1;" ::"r"(peer), "r"(1) : "memory");
     atomicExch(P.status, code);
+    for (const long long t0 = clock64(); clock64() - t0 < kAbortStayCycles;) __nanosleep(1000);
   };
   Pieces<C::kWhole> pc;
   pc.init(P);
@@ -1207,14 +1212,9 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
           }
         }
       }
-      // Copies still in flight.  The leader's MMA thread has waited for its own
-      // unless a role has given up; then the peer's arrival, which a phase of
-      // the leader needs too, may not come, and the limit is a few hundred times
-      // the copies' own time.
-      if (rank != 0 || s_abort)
+      if (rank != 0)  // copies still in flight (the leader's MMA thread waits for its own)
         for (int j = max(0, k - C::XS); j < k; ++j)
-          mbar_wait_sleep(smem_u32(&bar_xfull[j % C::XS]), (j / C::XS) & 1,
-                          rank != 0 ? kWaitLimitSleep : kDrainPolls);
+          mbar_wait(smem_u32(&bar_xfull[j % C::XS]), (j / C::XS) & 1);
     }
   } else if (role == kRoleMma && rank != 0) {
     // ---------------- X relay (second CTA) ----------------
@@ -1427,8 +1427,6 @@ __global__ void __launch_bounds__(C::kThreads, 1) gemm_main(const __grid_constan
                             un * kRowsN + (int)rank * kRowsCta, bar);
             }
             w = wait_ab(smem_u32(&bar_w16[s]), (w16_ph >> s) & 1u, &s_abort);
-            // given up: the thread that asked for the copies stays for them
-            if (w == kWaitAborted && r == 0) mbar_wait(smem_u32(&bar_w16[s]), (w16_ph >> s) & 1u);
             w16_ph ^= 1u << s;
             break;
         }
